@@ -1,6 +1,6 @@
 """Compile the CUDA library (sm_103a) in-tree: ``_build/libfdtd.so``.
 
-Two translation units, one ``-gencode``; takes about ten seconds.  The
+The translation units compile in parallel, one ``-gencode``.  The
 library links the CUDA runtime statically, so it only needs the driver at
 run time.
 """
@@ -21,6 +21,7 @@ SOURCES = [os.path.join(HERE, "csrc", "fdtd.cu"), os.path.join(HERE, "csrc", "en
 DEPENDS = SOURCES + [
     os.path.join(HERE, "csrc", "line_kernels.cuh"),
     os.path.join(HERE, "csrc", "aux_kernels.cuh"),
+    os.path.join(HERE, "csrc", "coef_kernels.cuh"),
     os.path.join(HERE, "csrc", "adjoint_kernels.cuh"),
     os.path.join(HERE, "csrc", "line4_kernels.cuh"),
     os.path.join(ROOT, "include", "fdtd.h"),
@@ -52,7 +53,7 @@ def build(force: bool = False, verbose: bool = False, bounds: bool = False) -> s
         return path
     os.makedirs(BUILD_DIR, exist_ok=True)
     tmp = path + ".tmp"
-    cmd = [nvcc_path(), ARCH, "-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC",
+    cmd = [nvcc_path(), ARCH, "-O3", "-std=c++17", "-lineinfo", "--threads=0", "-Xcompiler", "-fPIC",
            "-shared", "-o", tmp] + (["-DFDTD_BOUNDS"] if bounds else []) + SOURCES
     if verbose:
         cmd.insert(1, "-Xptxas=-v")

@@ -31,6 +31,7 @@
 #include "../../include/fdtd.h"
 #include "adjoint_kernels.cuh"
 #include "aux_kernels.cuh"
+#include "coef_kernels.cuh"
 #include "line_kernels.cuh"
 #include "line4_kernels.cuh"
 
@@ -123,7 +124,6 @@ struct fdtd_s {
   bool shape_tuned = false;   // per-node y/z launch shapes chosen by timing
   double eps_r = 1.0, mu_r = 1.0;          // uniform media
   double* eps_node[3] = {nullptr, nullptr, nullptr};  // per-node eps_r at E samples (device)
-  std::vector<double> eps_host[3];  // the same on the host, only while coefficients are built
   // lossy media: electric conductivity sigma [S/m]; the loss -sigma/eps E is
   // split evenly between A and B, so each procedure of length h adds
   // b sigma / 4 to the implicit diagonal (a host-side change of the pivots)
@@ -137,10 +137,8 @@ struct fdtd_s {
   void* yseq = nullptr;             // FP64 y/z lines solved one thread per line: the forward
                                     // values, one field-shaped array per E component
   double* sig_node[3] = {nullptr, nullptr, nullptr};  // per-node sigma at E samples (device)
-  std::vector<double> sig_host[3];  // the same on the host, only while coefficients are built
   bool mu_var = false;              // per-node mu (general media kernels)
   double* mu_node[3] = {nullptr, nullptr, nullptr};   // per-face mu_r at H samples (device)
-  std::vector<double> mu_host[3];   // the same on the host, only while coefficients are built
   bool poisoned = false;
   bool pending_init = true;   // FADI/FLOD2: state holds the physical field
   bool output_valid = false;  // scratch holds the physical field of this step
@@ -360,32 +358,8 @@ void free_coef(ProcCoef& pc) {
   pc.valid = false;
 }
 
-// eps_r at every E sample: mean of the in-domain cells sharing the edge.
-// mu_r at the H samples of component c (HX, HY, HZ): the mean of the two
-// cells sharing the face (cells outside the domain skipped).
-void face_mu(const fdtd_t* h, const double* mr, int c, std::vector<double>& out) {
-  const int nx = h->nx, ny = h->ny, nz = h->nz;
-  out.assign((size_t)h->count, 1.0);
-  int sx, sy, sz;
-  comp_extent(c, nx, ny, nz, &sx, &sy, &sz);
-  for (int k = 0; k < sz; ++k)
-    for (int j = 0; j < sy; ++j)
-      for (int i = 0; i < sx; ++i) {
-        double s = 0;
-        int n = 0;
-        for (int a = -1; a <= 0; ++a) {
-          int ci = i, cj = j, ck = k;
-          if (c == HX) ci = i + a;   // Hx (i, j+1/2, k+1/2): cells (i-1..i, j, k)
-          if (c == HY) cj = j + a;   // Hy (i+1/2, j, k+1/2): cells (i, j-1..j, k)
-          if (c == HZ) ck = k + a;   // Hz (i+1/2, j+1/2, k): cells (i, j, k-1..k)
-          if (ci < 0 || cj < 0 || ck < 0 || ci >= nx || cj >= ny || ck >= nz) continue;
-          s += mr[((size_t)ck * ny + cj) * nx + ci];
-          ++n;
-        }
-        out[(size_t)k * h->plane + (size_t)j * h->pitch + i] = n ? s / n : 1.0;
-      }
-}
-
+// eps_r (or sigma) at every E sample on the host, for the conductivity check
+// of fdtd_set_media: mean of the in-domain cells sharing the edge.
 void edge_eps(const fdtd_t* h, const double* er, int c, std::vector<double>& out) {
   const int nx = h->nx, ny = h->ny, nz = h->nz;
   out.assign((size_t)h->count, 0.0);
@@ -647,12 +621,8 @@ int build_proc(fdtd_t* h, int slot, int op, double hh, double loss_sign = 1.0) {
       int rc = upload_any(h, &c.tab, tab);
       if (rc) return rc;
     } else {
-      // Per-node media: rows scaled by 1/b_j (a symmetric matrix),
-      //   q_j w_j / 2 - (|ks| |kd| / 2) (w_{j+1} - 2 w_j + w_{j-1}) = q_j E_j + ks (H_j - H_{j-1}),
-      // q_j = 1/|b_j|, ks = s sign(h) / d_eta.  Every line is factored in FP64
-      // from exactly the q_j, ks, kd the kernel uses (rounded to the field
-      // precision first), so each procedure is an exact Cayley transform of
-      // the medium those rounded values describe.
+      // Per-node media: the lines are factored on the device
+      // (factor_lines_kernel) from the medium at the E and H samples
       const bool f32 = h->prec == FDTD_F32;
       auto rnd = [&](double x) { return f32 ? (double)(float)x : x; };
       c.kd = rnd(c.kd);
@@ -661,87 +631,56 @@ int build_proc(fdtd_t* h, int slot, int op, double hh, double loss_sign = 1.0) {
       const double off = -kk / 2.0;
       c.offh = rnd(off);
       c.offl = f32 ? (double)(float)(off - c.offh) : 0.0;
-      std::vector<double> nq((size_t)h->count, 0.0), nib((size_t)h->count, 0.0), nibl;
-      if (f32) nibl.assign((size_t)h->count, 0.0);
-      // per-node mu: each face f (between nodes f and f+1) has its own
-      // coupling kd_f and off-diagonal -|ks| |kd_f| / 2
-      std::vector<double> nkd, noffh, noffl;
-      if (h->mu_var) {
-        nkd.assign((size_t)h->count, 0.0);
-        noffh.assign((size_t)h->count, 0.0);
-        if (f32) noffl.assign((size_t)h->count, 0.0);
-      }
-      const double* mr = h->mu_var ? h->mu_host[g.hc - 3].data() : nullptr;
-      const double* er = h->eps_host[g.ec].data();
-      const double* sr = (h->lossy && !h->sig_host[g.ec].empty()) ? h->sig_host[g.ec].data() : nullptr;
-      // scaled rows: the loss adds loss_sign * sigma_j / 4 to the diagonal
-      auto loss_at = [&](long long at) {
-        return h->lossy ? loss_sign * (sr ? sr[at] : h->sigma_u) / 4.0 : 0.0;
+      int rc = FDTD_OK;
+      auto zeroed = [&](void** dst) {
+        if (!rc) rc = cuda_fail(h, dev_malloc(dst, (size_t)h->count * h->esize));
+        if (!rc) rc = cuda_fail(h, cudaMemsetAsync(*dst, 0, (size_t)h->count * h->esize, h->stream));
       };
-      const long long nl = g.n_lines();
-      for (long long line = 0; line < nl; ++line) {
-        long long base;
-        if (g.rows) {
-          const int jo = g.o_lo + (int)(line % g.n_o);
-          const int ko = g.o2_lo + (int)(line / g.n_o);
-          base = (long long)ko * g.os2 + (long long)jo * g.os;
-        } else {
-          const int nlx = g.lane_hi - g.lane_lo;
-          const int i = g.lane_lo + (int)(line % nlx);
-          const int o = g.o_lo + (int)(line / nlx);
-          base = (long long)o * g.os + i;
-        }
-        double ibm = 0;
-        if (!h->mu_var) {
-          for (int j = 1; j <= g.N - 1; ++j) {
-            const long long at = base + (long long)j * g.ls;
-            const double b = std::fabs(hh) / (2.0 * kEps0 * er[at]);
-            const double q = rnd(1.0 / b);
-            const double diag = q / 2.0 + kk + loss_at(at);
-            const double beta = diag - off * off * ibm;
-            const double ib = 1.0 / beta;
-            nq[at] = q;
-            nib[at] = rnd(ib);
-            if (f32) nibl[at] = (double)(float)(ib - nib[at]);
-            ibm = ib;
-          }
-          continue;
-        }
-        // kk_f = |ks| |kd_f| of the faces, from the kd_f the kernel uses
-        std::vector<double> kkf((size_t)g.N, 0.0);
-        for (int f = 0; f < g.N; ++f) {
-          const long long at = base + (long long)f * g.ls;
-          const double kdf = rnd(g.sign * (hh / (2.0 * kMu0 * mr[at])) / de);
-          const double kkv = std::fabs(c.ks) * std::fabs(kdf);
-          const double offf = -kkv / 2.0;
-          kkf[(size_t)f] = kkv;
-          nkd[at] = kdf;
-          noffh[at] = rnd(offf);
-          if (f32) noffl[at] = (double)(float)(offf - noffh[at]);
-        }
-        for (int j = 1; j <= g.N - 1; ++j) {
-          const long long at = base + (long long)j * g.ls;
-          const double b = std::fabs(hh) / (2.0 * kEps0 * er[at]);
-          const double q = rnd(1.0 / b);
-          const double diag = q / 2.0 + (kkf[(size_t)j] + kkf[(size_t)j - 1]) / 2.0 + loss_at(at);
-          const double offm = -kkf[(size_t)j - 1] / 2.0;  // face j-1, between nodes j-1 and j
-          const double beta = diag - offm * offm * ibm;
-          const double ib = 1.0 / beta;
-          nq[at] = q;
-          nib[at] = rnd(ib);
-          if (f32) nibl[at] = (double)(float)(ib - nib[at]);
-          ibm = ib;
-        }
-      }
-      int rc = upload_any(h, &c.nq, nq);
-      if (rc) return rc;
-      if ((rc = upload_any(h, &c.nib, nib))) return rc;
-      if (f32 && (rc = upload_any(h, &c.nibl, nibl))) return rc;
+      zeroed(&c.nq);
+      zeroed(&c.nib);
+      if (f32) zeroed(&c.nibl);
       if (h->mu_var) {
-        if ((rc = upload_any(h, &c.nkd, nkd))) return rc;
-        if ((rc = upload_any(h, &c.noffh, noffh))) return rc;
-        if (f32 && (rc = upload_any(h, &c.noffl, noffl))) return rc;
+        zeroed(&c.nkd);
+        zeroed(&c.noffh);
+        if (f32) zeroed(&c.noffl);
       }
+      if (rc) return rc;
+      if (g.N < 1 || g.n_lines() <= 0) continue;
+      fdtd::FactorParams fp;
+      fp.ls = g.ls;
+      fp.os = g.os;
+      fp.os2 = g.os2;
+      fp.lane_lo = g.lane_lo;
+      fp.lane_hi = g.lane_hi;
+      fp.o_lo = g.o_lo;
+      fp.n_o = g.n_o;
+      fp.o2_lo = g.o2_lo;
+      fp.n_o2 = g.n_o2;
+      fp.rows = g.rows ? 1 : 0;
+      fp.N = g.N;
+      fp.er = h->eps_node[g.ec];
+      fp.sr = h->sig_node[g.ec];
+      fp.mr = h->mu_var ? h->mu_node[g.hc - 3] : nullptr;
+      fp.sigma_u = h->sigma_u;
+      fp.loss_sign = h->lossy ? loss_sign : 0.0;
+      fp.h = hh;
+      fp.eps2 = 2.0 * kEps0;
+      fp.mu2 = 2.0 * kMu0;
+      fp.sign = g.sign;
+      fp.de = de;
+      fp.kk = kk;
+      fp.off = off;
+      fp.ks_abs = std::fabs(c.ks);
+      fp.n_elem = h->count;
+      const unsigned blocks = (unsigned)((g.n_lines() + 63) / 64);
+      h->launches++;
+      if (f32)
+        fdtd::factor_lines_kernel<float><<<blocks, 64, 0, h->stream>>>(
+            fp, (float*)c.nq, (float*)c.nib, (float*)c.nibl, (float*)c.nkd, (float*)c.noffh, (float*)c.noffl);
+      else
+        fdtd::factor_lines_kernel<double><<<blocks, 64, 0, h->stream>>>(fp, (double*)c.nq, (double*)c.nib, nullptr,
+                                                                        (double*)c.nkd, (double*)c.noffh, nullptr);
+      if ((rc = cuda_fail(h, cudaGetLastError()))) return rc;
     }
   }
   P.valid = true;
@@ -2398,44 +2337,44 @@ int fdtd_set_media(fdtd_t* h, const double* eps, const double* mu, const double*
   h->per_node = !e_uniform || h->mu_var || sig_var || (h->desc.tune[1] & 2) != 0;
   h->eps_r = h->per_node ? 1.0 : e0;
   h->shape_tuned = false;
-  int rc = FDTD_OK;
-  auto release_host = [&]() {
-    for (int c = 0; c < 3; ++c) {
-      std::vector<double>().swap(h->eps_host[c]);
-      std::vector<double>().swap(h->mu_host[c]);
-      std::vector<double>().swap(h->sig_host[c]);
-    }
-  };
   if (h->per_node) {
+    // the means at the samples, from one device copy of the cell arrays
+    double* d_cell = nullptr;
+    CK(dev_malloc((void**)&d_cell, sizeof(double) * nc));
     std::vector<double> ones;
-    if (!eps) ones.assign(nc, 1.0);
-    for (int c = 0; c < 3; ++c) {
-      edge_eps(h, eps ? eps : ones.data(), c, h->eps_host[c]);
-      CK(dev_malloc((void**)&h->eps_node[c], sizeof(double) * h->eps_host[c].size()));
-      CK(cudaMemcpyAsync(h->eps_node[c], h->eps_host[c].data(), sizeof(double) * h->eps_host[c].size(),
-                         cudaMemcpyHostToDevice, h->stream));
-    }
-    if (h->mu_var) {
-      for (int c = 0; c < 3; ++c) {
-        face_mu(h, mu, HX + c, h->mu_host[c]);
-        CK(dev_malloc((void**)&h->mu_node[c], sizeof(double) * h->mu_host[c].size()));
-        CK(cudaMemcpyAsync(h->mu_node[c], h->mu_host[c].data(), sizeof(double) * h->mu_host[c].size(),
-                           cudaMemcpyHostToDevice, h->stream));
+    int rc = FDTD_OK;
+    auto means = [&](const double* host, double* const* base, int first, double fill, bool faces) {
+      if (!rc) rc = cuda_fail(h, cudaMemcpyAsync(d_cell, host, sizeof(double) * nc, cudaMemcpyHostToDevice, h->stream));
+      for (int c = 0; c < 3 && !rc; ++c) {
+        int sx, sy, sz;
+        comp_extent(first + c, h->nx, h->ny, h->nz, &sx, &sy, &sz);
+        const bool w[3] = {(c == 0) == faces, (c == 1) == faces, (c == 2) == faces};
+        h->launches++;
+        fdtd::cell_mean_kernel<<<152 * 8, 128, 0, h->stream>>>(d_cell, base[c], h->nx, h->ny, h->nz, sx, sy, sz, w[0],
+                                                               w[1], w[2], h->pitch, h->plane, fill);
+        rc = cuda_fail(h, cudaGetLastError());
       }
+    };
+    auto alloc = [&](double** base) {
+      for (int c = 0; c < 3 && !rc; ++c) rc = cuda_fail(h, dev_malloc((void**)&base[c], sizeof(double) * h->count));
+    };
+    if (!eps) ones.assign(nc, 1.0);
+    alloc(h->eps_node);
+    means(eps ? eps : ones.data(), h->eps_node, EX, 0.0, false);
+    if (h->mu_var) {
+      alloc(h->mu_node);
+      means(mu, h->mu_node, HX, 1.0, true);
     }
     if (sig_var) {
       // sigma at an E sample: the mean of the cells sharing its edge, as eps
-      for (int c = 0; c < 3; ++c) {
-        edge_eps(h, sigma, c, h->sig_host[c]);
-        CK(dev_malloc((void**)&h->sig_node[c], sizeof(double) * h->sig_host[c].size()));
-        CK(cudaMemcpyAsync(h->sig_node[c], h->sig_host[c].data(), sizeof(double) * h->sig_host[c].size(),
-                           cudaMemcpyHostToDevice, h->stream));
-      }
+      alloc(h->sig_node);
+      means(sigma, h->sig_node, EX, 0.0, false);
     }
-    CK(cudaStreamSynchronize(h->stream));
+    if (!rc) rc = cuda_fail(h, cudaStreamSynchronize(h->stream));  // the host arrays are the caller's
+    cudaFree(d_cell);
+    if (rc) return rc;
   }
-  rc = build_all_coefs(h);
-  release_host();
+  const int rc = build_all_coefs(h);
   h->output_valid = false;
   h->inv_dirty = true;
   if (rc) return rc;

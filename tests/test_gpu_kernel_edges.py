@@ -1,0 +1,35 @@
+"""GPU kernels at the sizes where their indexing can go wrong (edges of rows,
+segments and tiles, the shortest and longest lines), against the FP64 oracle."""
+import numpy as np
+import pytest
+
+from gpu_helpers import energy_norm_rel, gpu_run, oracle_problem, random_fields
+from oracle import schemes as S
+
+pytestmark = pytest.mark.gpu
+TOL = {"f64": 1e-12, "f32": 1e-4}   # the library's stated bounds for a few steps
+
+
+def random_media(nx, ny, nz, seed):
+    return np.random.default_rng(seed).uniform(1.0, 6.0, (nz, ny, nx))
+
+
+def check(nx, ny, nz, scheme, prec, steps=4, eps=None, tune=(0, 0), cfl=4.0):
+    d = 1e-3
+    dt = cfl * d / (299792458.0 * np.sqrt(3.0 if nz > 1 else 2.0))
+    u0 = random_fields(nx, ny, nz, 11)
+    out, _, _, sim = gpu_run(nx, ny, nz, d, d, d, dt, scheme, prec, u0, steps, eps=eps, tune=tune)
+    sim.close()
+    if prec == "f32":
+        u0 = {c: v.astype(np.float32).astype(np.float64) for c, v in u0.items()}
+    ref, _, _ = S.run_fundamental(oracle_problem(nx, ny, nz, d, d, d, dt, eps=eps), scheme, u0, steps)
+    err = energy_norm_rel(out, ref)
+    assert err <= TOL[prec], err
+    return out
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("dims", [(2, 2, 1), (2, 2, 2), (3, 2, 5), (31, 5, 4), (32, 4, 33), (33, 65, 3), (127, 3, 64)])
+def test_media_formed_on_the_device(dims, prec):
+    """Per-cell eps: means at the samples and line pivots from the device kernels."""
+    check(*dims, "flod", prec, eps=random_media(*dims, 5))
