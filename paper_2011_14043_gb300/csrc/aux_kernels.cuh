@@ -84,9 +84,9 @@ __global__ void add_point_table_kernel(T* y, long long at, const double* table, 
   }
 }
 
-// mode 0: *step = value;  mode 1: *step += 1.
+// mode 0: *step = value;  mode 1: *step += value.
 __global__ void step_counter_kernel(long long* step, long long value, int mode) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *step = mode == 0 ? value : *step + 1;
+  if (threadIdx.x == 0 && blockIdx.x == 0) *step = mode == 0 ? value : *step + value;
 }
 
 // Compact [sz][sy][sx] <-> padded (plane, pitch) layout of one component,

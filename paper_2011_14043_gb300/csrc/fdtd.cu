@@ -33,6 +33,7 @@
 #include "aux_kernels.cuh"
 #include "coef_kernels.cuh"
 #include "line_kernels.cuh"
+#include "fused_kernels.cuh"
 #include "line4_kernels.cuh"
 
 namespace {
@@ -66,6 +67,7 @@ struct PairCoef {
   bool wall_fix = false;  // uniform media: the rank-one wall correction rows are built
   int kg_len = 0;         // the correction is zero from this node on (a multiple of L)
   double qf[2][32] = {{0}}, qb[2][32] = {{0}};
+  double mc = 0;          // uniform media: the converged multiplier m = c
   int jc4 = 1 << 30, je4 = -1;  // fourth order: nodes whose factor rows all equal cv4
   double cv4[14] = {0};
   void* nq = nullptr;     // per-node media (field layout, T): 1/|b_j|
@@ -121,6 +123,8 @@ struct fdtd_s {
   // the second-difference part does not)
   ProcCoef proc[5];
   bool per_node = false;
+  bool adjoint = false;       // a reverse-mode context was created on this handle
+  bool batched = false;       // the handle was put into a batch (which steps it by its own kernels)
   bool shape_tuned = false;   // per-node y/z launch shapes chosen by timing
   double eps_r = 1.0, mu_r = 1.0;          // uniform media
   double* eps_node[3] = {nullptr, nullptr, nullptr};  // per-node eps_r at E samples (device)
@@ -172,9 +176,10 @@ struct fdtd_s {
   // three pairs of each procedure on parallel branches
   cudaStream_t g_run = nullptr, g_br[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t g_in = nullptr, g_out = nullptr, g_fork = nullptr, g_join[3] = {nullptr, nullptr, nullptr};
-  cudaGraphExec_t g_exec = nullptr;
+  cudaGraphExec_t g_exec = nullptr;     // one step
+  cudaGraphExec_t g_run_exec = nullptr; // kStepRun steps (fused procedures)
   std::vector<const void*> g_bound;     // state pointers the graph was captured with
-  long long g_kernels = 0;              // kernels per replay
+  long long g_kernels = 0, g_run_kernels = 0;  // kernels per replay
   double* d_srcval = nullptr;           // f_E(n) = src_scale * I(n), n < src_current.size()
   long long srcval_len = 0;
   long long* d_step = nullptr;          // step index read by graph-replayed source kernels
@@ -572,12 +577,12 @@ int build_proc(fdtd_t* h, int slot, int op, double hh, double loss_sign = 1.0) {
         for (int j = N - 1; j >= 1; --j) gg[j] = yg[j] * ib_inf - mc_inf * gg[j + 1];
         const double delta = beta_inf - diag;
         const double kappa = delta / (1.0 - delta * gg[1]);
-        // terms below 2^-50 of w'_1 change no result: drop them, so that the
+        // terms below 2^-50 (FP64: 2^-60) of w'_1 change no result: drop them, so that the
         // segments past the last nonzero term skip the correction
         int last = 0;
         for (int j = 1; j <= N - 1; ++j) {
           kg[j] = kappa * gg[j];
-          if (std::fabs(kg[j]) < 0x1p-50) kg[j] = 0.0;
+          if (std::fabs(kg[j]) < (h->prec == FDTD_F32 ? 0x1p-50 : 0x1p-60)) kg[j] = 0.0;
           else last = j;
         }
         c.kg_len = last > 0 ? ((last + 1 + L - 1) / L) * L : 0;
@@ -597,7 +602,8 @@ int build_proc(fdtd_t* h, int slot, int op, double hh, double loss_sign = 1.0) {
         const double cvv[3] = {ib_inf, mc_inf, mc_inf};
         for (int k = 0; k < 3; ++k) { c.cv[2 * k] = hi(cvv[k]); c.cv[2 * k + 1] = lo(cvv[k]); }
         double qf = 1.0;
-        for (int t = 0; t < L; ++t) { qf *= -mc_inf; c.qf[0][t] = hi(qf); c.qf[1][t] = lo(qf); }
+        for (int t = 0; t < 32; ++t) { qf *= -mc_inf; c.qf[0][t] = hi(qf); c.qf[1][t] = lo(qf); }
+        c.mc = mc_inf;
         double qb = 1.0;
         for (int t = L - 1; t >= 0; --t) { qb *= -mc_inf; c.qb[0][t] = hi(qb); c.qb[1][t] = lo(qb); }
       }
@@ -714,6 +720,26 @@ int build_all_coefs(fdtd_t* h) {
 // ---------------------------------------------------------------------------
 
 
+// Carry products of runs of segments of L nodes (row_solve_wall) and where
+// they fall below 2^-50 (FP64 fields: 2^-60) of the carry.
+template <typename T>
+void set_scan(fdtd::PairParams<T>& p, const PairCoef& c, int L) {
+  const double least = sizeof(T) == 4 ? 0x1p-50 : 0x1p-60;
+  // the products of longer runs by repeated squaring in the field precision,
+  // as a scan that carries its products along forms them
+  p.sc[0][0] = (T)c.qf[0][L - 1];
+  p.sc[1][0] = (T)c.qf[1][L - 1];
+  for (int k = 1; k < 5; ++k) {
+    p.sc[0][k] = p.sc[0][k - 1] * p.sc[0][k - 1];
+    p.sc[1][k] = T(0);
+  }
+  p.nscan = 32;
+  for (int k = 4; k >= 0; --k)
+    if (std::fabs((double)p.sc[0][k]) < least) p.nscan = 1 << k;
+  p.kx = 1;
+  while (p.kx < 8 && std::pow(std::fabs(c.mc), 32.0 * p.kx) >= least) ++p.kx;
+}
+
 template <typename T>
 fdtd::PairParams<T> make_params(const fdtd_t* h, const PairGeom& g, const PairCoef& c, double sgn,
                                 double alpha, double beta, double kd_mul, void* const* in,
@@ -766,6 +792,7 @@ fdtd::PairParams<T> make_params(const fdtd_t* h, const PairGeom& g, const PairCo
   // the rank-one wall correction (tune[1] bit 7: the table lanes instead)
   p.wall_fix = (c.wall_fix && sizeof(T) == 4 && (h->desc.tune[1] & 128) == 0) ? 1 : 0;
   p.kg_len = c.kg_len;
+  set_scan(p, c, c.L);
   // one scratch array per E component: the three pairs of a procedure run
   // concurrently (graph branches) and each has its own E component
   p.tmp4 = h->tmp4 ? (T*)h->tmp4 + (size_t)g.ec * h->count : nullptr;
@@ -795,9 +822,6 @@ void launch_rows_L(const fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>
   const unsigned blocks = (unsigned)((nl + wpb - 1) / wpb);
   if (per_node)
     fdtd::proc_rows_kernel<T, L, true><<<blocks, wpb * 32, 0, h->stream>>>(p);
-  else if (sizeof(T) == 4 && L >= 2 && p.wall_fix && g.N == 32 * L && (h->desc.tune[1] & 2048) == 0)
-    fdtd::proc_rows_kernel<T, L, false, (sizeof(T) == 4 && L >= 2), (sizeof(T) == 4 && L >= 2)>
-        <<<blocks, wpb * 32, 0, h->stream>>>(p);
   else if (sizeof(T) == 4 && L >= 2 && p.wall_fix)
     fdtd::proc_rows_kernel<T, L, false, (sizeof(T) == 4 && L >= 2)><<<blocks, wpb * 32, 0, h->stream>>>(p);
   else
@@ -1229,22 +1253,8 @@ int ensure_yseq(fdtd_t* h) {
 }
 
 template <typename T>
-int launch_pair(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
-  if (g.empty()) return FDTD_OK;
-  if (h->order == 4 && !h->tmp4) return FDTD_ERR_STATE;
-  if (p.nkd) {
-    h->launches++;
-    return launch_pair_gm<T>(h, g, p);
-  }
+int launch_pair_raw(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
   const bool pn = h->per_node;
-  const int cls = g.axis == AX_Y ? 0 : (g.axis == AX_Z ? 1 : 2);
-  int ev0 = -1, ev1 = -1;
-  if (h->timing) {
-    int rc = take_event(h, &ev0);
-    if (rc) return rc;
-    if ((rc = take_event(h, &ev1))) return rc;
-    CK(cudaEventRecord(h->ev_pool[ev0], h->stream));
-  }
   h->launches++;
   if (h->order == 4) {
     launch_line4_raw<T>(h, g, p, 0);
@@ -1291,14 +1301,184 @@ int launch_pair(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
     launch_strided<T>(h, g, p, pn, cfg.lanes, cfg.L);
   }
   CK(cudaGetLastError());
-  if (h->timing) {
-    CK(cudaEventRecord(h->ev_pool[ev1], h->stream));
-    h->ev_rec.push_back({cls, {ev0, ev1}});
-    // resolve in batches so the pool stays small
-    if (h->ev_rec.size() >= 4096) {
-      int rc = resolve_events(h);
+  return FDTD_OK;
+}
+
+// A launch of class cls with its event pair (per-launch timing).
+template <typename F>
+int timed(fdtd_t* h, int cls, F&& launch) {
+  int ev0 = -1, ev1 = -1, rc;
+  if ((rc = take_event(h, &ev0)) || (rc = take_event(h, &ev1))) return rc;
+  CK(cudaEventRecord(h->ev_pool[ev0], h->stream));
+  if ((rc = launch())) return rc;
+  CK(cudaEventRecord(h->ev_pool[ev1], h->stream));
+  h->ev_rec.push_back({cls, {ev0, ev1}});
+  // resolve in batches so the pool stays small
+  return h->ev_rec.size() >= 4096 ? resolve_events(h) : FDTD_OK;
+}
+
+template <typename T>
+int launch_pair(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
+  if (g.empty()) return FDTD_OK;
+  if (h->order == 4 && !h->tmp4) return FDTD_ERR_STATE;
+  if (p.nkd) {
+    h->launches++;
+    return launch_pair_gm<T>(h, g, p);
+  }
+  const int cls = g.axis == AX_Y ? 0 : (g.axis == AX_Z ? 1 : 2);
+  if (h->timing) return timed(h, cls, [&]() { return launch_pair_raw<T>(h, g, p); });
+  return launch_pair_raw<T>(h, g, p);
+}
+
+// ---------------------------------------------------------------------------
+// One launch per procedure (fused_kernels.cuh)
+// ---------------------------------------------------------------------------
+// FP32 fields, second-order differences, uniform mu, sides of at most 256
+// cells (8 warps of 4 segments of 8 nodes hold a line), arrays of less than
+// 2^32 bytes.  The launch-shape overrides that name another kernel keep it,
+// the reverse pass the kernels whose records and rounding it replays, a
+// batch's handles the kernels that the batch steps them by, and handles with
+// probes the kernels whose rounding their FP64 series have always shown.
+//
+// The line: a procedure that moves at most 256 MB (24 B per cell, 60 B with
+// per-node media), about twice the L2 cache.  FADI steps, fused against a
+// launch per pair on parallel branches, us: 20^3 7.2 / 15.5, 64^3 9.9 / 16.5,
+// 96^3 15.9 / 28.9, 128^3 30.8 / 37.3, 219x101x75 30.3 / 45.7, 192^3
+// 119 / 134, 224^3 206 / 200, 256^3 285 / 273; per-node 64^3 9.9 / 15.3,
+// 128^3 55.7 / 61.7, 160^3 125 / 127, 192^3 243 / 222, 256^3 516 / 473: beyond
+// it, HBM-bound launches want the TMA ring (y, z) and the one-warp-per-line
+// kernel's 40 warps per SM (x).  FP64 fields gain nothing (their pipe binds:
+// 40^3 44.5 against 33.5).
+constexpr double kFusedMaxBytes = 256e6;
+
+bool fused_ok(const fdtd_t* h) {
+  if (h->order != 2 || h->mu_var || h->adjoint || h->batched || h->nprobes > 0 || h->desc.tune[0] != 0 || (h->desc.tune[1] & (1 | 4 | 128)) != 0)
+    return false;
+  if (h->nx > fdtd::kFusedMaxN || h->ny > fdtd::kFusedMaxN || h->nz > fdtd::kFusedMaxN) return false;
+  if ((unsigned long long)h->count * h->esize > 0xffffffffull) return false;
+  return h->prec == FDTD_F32 &&
+         (h->per_node ? 60.0 : 24.0) * (double)h->nx * h->ny * h->nz <= kFusedMaxBytes;
+}
+
+unsigned reciprocal(int d) { return d <= 1 ? 0u : (unsigned)(((1ull << 32) + (unsigned)d - 1) / (unsigned)d); }
+
+template <typename T, bool PN, int LPL>
+cudaError_t launch_fused_k(const fdtd::FusedParams<T>& fp, unsigned blocks, unsigned threads, cudaStream_t st,
+                           bool chained) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fdtd::proc_fused_kernel<T, PN, LPL>, fp);
+}
+
+fdtd::FusedSource no_source() {
+  fdtd::FusedSource s = {};
+  s.ec = -1;
+  return s;
+}
+
+// The pairs of procedure `slot` named by `mask` (bit 0: lines along y, 1: z,
+// 2: x) in one launch.  chained: the launch before it on the stream is
+// another procedure of the same captured step (programmatic edge).
+template <typename T>
+int launch_fused(fdtd_t* h, int slot, double sgn, double alpha, double beta, double kd_mul, void* const* in,
+                 void* const* out, const fdtd::FusedSource& src, bool chained, int mask) {
+  const ProcCoef& P = h->proc[slot];
+  fdtd::FusedParams<T> fp;
+  fp.src = src;
+  int nwarps[3] = {1, 1, 1};
+  bool on[3];
+  for (int q = 0; q < 3; ++q) {
+    const PairGeom& g = h->geom[P.op][q];
+    const int d = g.axis == AX_Y ? 0 : (g.axis == AX_Z ? 1 : 2);
+    fp.p[d] = make_params<T>(h, g, P.pc[q], sgn, alpha, beta, kd_mul, in, out);
+    set_scan(fp.p[d], P.pc[q], fdtd::kFusedL);
+    fp.ec[d] = g.ec;
+    on[d] = !g.empty() && (mask >> d & 1) != 0;
+    if (d == 2) {
+      fp.div[2] = reciprocal(std::max(1, g.n_o));
+    } else {
+      const int lines = 8 * fdtd::Wide<T>::V;
+      fp.tiles_x[d] = std::max(1, (g.lane_hi + lines - 1) / lines);
+      fp.ntiles[d] = on[d] ? (unsigned)fp.tiles_x[d] * (unsigned)g.n_o : 0u;
+      fp.div[d] = reciprocal(fp.tiles_x[d]);
+      nwarps[d] = std::max(1, (g.N + 4 * fdtd::kFusedL - 1) / (4 * fdtd::kFusedL));
+    }
+  }
+  // warps per block: the count (4..8) that leaves the fewest warps idle over
+  // the y and z tiles (a block holds whole tiles)
+  int bw = 8;
+  double least = 1e30;
+  for (int w = 8; w >= 4; --w) {
+    double cost = 0;
+    for (int d = 0; d < 2; ++d) {
+      if (fp.ntiles[d] == 0) continue;
+      if (w < nwarps[d]) cost = 1e30;
+      else cost += (double)fp.ntiles[d] * w / (w / nwarps[d]);
+    }
+    if (cost < least) {
+      least = cost;
+      bw = w;
+    }
+  }
+  for (int d = 0; d < 2; ++d) {
+    fp.wpt[d] = nwarps[d];
+    fp.tpb[d] = std::max(1, bw / nwarps[d]);
+    fp.nb[d] = (int)((fp.ntiles[d] + (unsigned)fp.tpb[d] - 1) / (unsigned)fp.tpb[d]);
+  }
+  const int lpl = h->nx <= 64 ? 8 : (h->nx <= 128 ? 16 : 32);
+  const unsigned rows = on[2] ? (unsigned)fp.p[2].n_o * (unsigned)fp.p[2].n_o2 : 0u;
+  const unsigned rpb = (unsigned)(bw * (32 / lpl));
+  fp.nb[2] = (int)((rows + rpb - 1) / rpb);
+  const unsigned blocks = (unsigned)(fp.nb[0] + fp.nb[1] + fp.nb[2]);
+  if (blocks == 0) return FDTD_OK;
+  const unsigned threads = (unsigned)bw * 32;
+  const bool pn = h->per_node;
+  cudaError_t e;
+  if (lpl == 8)
+    e = pn ? launch_fused_k<T, true, 8>(fp, blocks, threads, h->stream, chained)
+           : launch_fused_k<T, false, 8>(fp, blocks, threads, h->stream, chained);
+  else if (lpl == 16)
+    e = pn ? launch_fused_k<T, true, 16>(fp, blocks, threads, h->stream, chained)
+           : launch_fused_k<T, false, 16>(fp, blocks, threads, h->stream, chained);
+  else
+    e = pn ? launch_fused_k<T, true, 32>(fp, blocks, threads, h->stream, chained)
+           : launch_fused_k<T, false, 32>(fp, blocks, threads, h->stream, chained);
+  h->launches++;
+  return cuda_fail(h, e);
+}
+
+// One procedure by the fused kernel; per-launch timing takes one launch per
+// pair, and x lines on request the TMA-fed kernel.
+template <typename T>
+int run_fused(fdtd_t* h, int slot, double sgn, double alpha, double beta, double kd_mul, void* const* in,
+              void* const* out, const fdtd::FusedSource& src, bool chained) {
+  int mask = 7;
+  const ProcCoef& P = h->proc[slot];
+  for (int q = 0; q < 3; ++q) {
+    const PairGeom& g = h->geom[P.op][q];
+    if (sizeof(T) == 4 && g.rows && rows_tma_eligible(h, g) && !g.empty() && in[g.ec] == h->f[g.ec] &&
+        in[g.hc] == h->f[g.hc]) {
+      mask = 3;
+      int rc = launch_pair<T>(h, g, make_params<T>(h, g, P.pc[q], sgn, alpha, beta, kd_mul, in, out));
       if (rc) return rc;
     }
+  }
+  if (!h->timing) return launch_fused<T>(h, slot, sgn, alpha, beta, kd_mul, in, out, src, chained && mask == 7, mask);
+  for (int q = 0; q < 3; ++q) {
+    const PairGeom& g = h->geom[P.op][q];
+    const int cls = g.axis == AX_Y ? 0 : (g.axis == AX_Z ? 1 : 2);
+    if (g.empty() || (mask >> cls & 1) == 0) continue;
+    int rc = timed(h, cls, [&]() {
+      return launch_fused<T>(h, slot, sgn, alpha, beta, kd_mul, in, out, src, false, 1 << cls);
+    });
+    if (rc) return rc;
   }
   return FDTD_OK;
 }
@@ -1310,6 +1490,8 @@ int run_procedure(fdtd_t* h, int slot, double sgn, double alpha, double beta, do
                   void* const* in, void* const* out) {
   const ProcCoef& P = h->proc[slot];
   NvtxScope range(P.op == 0 ? "procedure A" : "procedure B");
+  if constexpr (sizeof(T) == 4)
+    if (fused_ok(h)) return run_fused<T>(h, slot, sgn, alpha, beta, kd_mul, in, out, no_source(), false);
   for (int q = 0; q < 3; ++q) {
     const PairGeom& g = h->geom[P.op][q];
     fdtd::PairParams<T> p = make_params<T>(h, g, P.pc[q], sgn, alpha, beta, kd_mul, in, out);
@@ -1525,7 +1707,8 @@ int physical_to_scratch(fdtd_t* h, long long n_next = -1);
 void graph_release(fdtd_t* h) {
   if (h->g_run) cudaStreamSynchronize(h->g_run);
   if (h->g_exec) cudaGraphExecDestroy(h->g_exec);
-  h->g_exec = nullptr;
+  if (h->g_run_exec) cudaGraphExecDestroy(h->g_run_exec);
+  h->g_exec = h->g_run_exec = nullptr;
   h->g_bound.clear();
 }
 
@@ -1534,70 +1717,111 @@ bool graph_usable(const fdtd_t* h) {
          (h->src_comp < 0 || h->d_srcval != nullptr);
 }
 
-// nsteps steps as replays of a captured one-step graph: each procedure forks
-// its three pair launches (disjoint arrays) onto parallel branches and joins
-// them before the next procedure; a point source is added by kernels that
-// read each step's value from a device table indexed by a device step
-// counter.  Same kernels, same arguments, same results as one_step.
+// Steps of a run captured in one graph where a step is a few short launches:
+// a replay costs the device about 2 us between graphs, and the host 2-3 us.
+constexpr int kStepRun = 16;
+
 int ensure_branches(fdtd_t* h);
 
-int step_graph(fdtd_t* h, int64_t nsteps) {
-  if (int rc = ensure_branches(h)) return rc;
+// Capture `count` steps as a graph.  Fused procedures: one launch each, the
+// source added inside it, chained by programmatic edges.  Otherwise each
+// procedure forks its three pair launches (disjoint arrays) onto parallel
+// branches and joins them before the next procedure, and a point source is
+// added by kernels of its own.  The source reads each step's value from a
+// device table indexed by a device step counter.  Same arithmetic, same
+// results as one_step.
+int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernels) {
   const bool src = h->src_comp >= 0;
-  std::vector<const void*> ptrs(h->f, h->f + 6);
-  if (!h->g_exec || ptrs != h->g_bound) {
-    graph_release(h);
-    if (h->prec == FDTD_F32) CK((ensure_tma_attr<float, 16, 2, 2>()));
-    if (h->prec == FDTD_F32) CK(ensure_rows_tma_attr());
-    static const int seq_fss[3] = {0, 1, 0};
-    static const int seq_two[2] = {0, 1};
-    const int* seq = h->scheme == FDTD_FSS ? seq_fss : seq_two;
-    const int nproc = h->scheme == FDTD_FSS ? 3 : 2;
-    // the source terms of one_step: coefficient of f added before and after
-    // each procedure (0 = none), and the step offset of the value after it
-    const double dt = h->dt;
-    double pre[3] = {0, 0, 0}, post[3] = {0, 0, 0};
-    double pre2[3] = {0, 0, 0}, post2[3] = {0, 0, 0};   // second terms, step offset 1
-    int post_off[3] = {0, 0, 0};
-    if (h->scheme == FDTD_FADI) {
-      post[0] = 0.5 * dt;
-      post[1] = 0.5 * dt;
-      post_off[1] = 1;
-    } else if (h->scheme == FDTD_FSS) {
-      pre[0] = post[0] = 0.125 * dt;
-      pre[1] = post[1] = 0.25 * dt;
-      pre[2] = post[2] = 0.125 * dt;
-    } else if (h->scheme == FDTD_FLOD2) {
-      // B: (dt/4) of the mean of f(t_n + dt/2) and f(t_n + 3dt/2), as two
-      // terms (dt/8) f of offsets 0 and 1 (procedure_two_terms)
-      pre[0] = post[0] = 0.25 * dt;
-      pre[1] = post[1] = 0.125 * dt;
-      pre2[1] = post2[1] = 0.125 * dt;
-    } else {
-      pre[0] = post[0] = 0.25 * dt;
-      pre[1] = post[1] = 0.25 * dt;
-    }
-    if (src && !h->d_step) CK(dev_malloc((void**)&h->d_step, sizeof(long long)));
-    const long long src_at = src ? elem_index(h, h->src_i, h->src_j, h->src_k) : 0;
-    auto add_src = [&](double coef, int off) -> cudaError_t {
-      if (!src || coef == 0.0) return cudaSuccess;
-      if (h->prec == FDTD_F64)
-        fdtd::add_point_table_kernel<double><<<1, 32, 0, h->g_run>>>((double*)h->f[h->src_comp], src_at,
-                                                                     h->d_srcval, h->srcval_len, h->d_step, off, coef);
-      else
-        fdtd::add_point_table_kernel<float><<<1, 32, 0, h->g_run>>>((float*)h->f[h->src_comp], src_at, h->d_srcval,
-                                                                    h->srcval_len, h->d_step, off, coef);
-      h->launches++;
-      return cudaGetLastError();
-    };
-    cudaStream_t home = h->stream;
-    const long long before = h->launches;
-    NvtxScope range("step graph capture");
-    CK(cudaStreamBeginCapture(h->g_run, cudaStreamCaptureModeThreadLocal));
-    int rc = FDTD_OK;
+  const bool fused = fused_ok(h);
+  if (h->prec == FDTD_F32) CK((ensure_tma_attr<float, 16, 2, 2>()));
+  if (h->prec == FDTD_F32) CK(ensure_rows_tma_attr());
+  static const int seq_fss[3] = {0, 1, 0};
+  static const int seq_two[2] = {0, 1};
+  const int* seq = h->scheme == FDTD_FSS ? seq_fss : seq_two;
+  const int nproc = h->scheme == FDTD_FSS ? 3 : 2;
+  // the source terms of one_step: coefficient of f added before and after
+  // each procedure (0 = none), and the step offset of the value after it
+  const double dt = h->dt;
+  double pre[3] = {0, 0, 0}, post[3] = {0, 0, 0};
+  double pre2[3] = {0, 0, 0}, post2[3] = {0, 0, 0};   // second terms, step offset 1
+  int post_off[3] = {0, 0, 0};
+  if (h->scheme == FDTD_FADI) {
+    post[0] = 0.5 * dt;
+    post[1] = 0.5 * dt;
+    post_off[1] = 1;
+  } else if (h->scheme == FDTD_FSS) {
+    pre[0] = post[0] = 0.125 * dt;
+    pre[1] = post[1] = 0.25 * dt;
+    pre[2] = post[2] = 0.125 * dt;
+  } else if (h->scheme == FDTD_FLOD2) {
+    // B: (dt/4) of the mean of f(t_n + dt/2) and f(t_n + 3dt/2), as two
+    // terms (dt/8) f of offsets 0 and 1 (procedure_two_terms)
+    pre[0] = post[0] = 0.25 * dt;
+    pre[1] = post[1] = 0.125 * dt;
+    pre2[1] = post2[1] = 0.125 * dt;
+  } else {
+    pre[0] = post[0] = 0.25 * dt;
+    pre[1] = post[1] = 0.25 * dt;
+  }
+  if (src && !h->d_step) CK(dev_malloc((void**)&h->d_step, sizeof(long long)));
+  const long long src_at = src ? elem_index(h, h->src_i, h->src_j, h->src_k) : 0;
+  // the sample lies on a line of its component's pair in either procedure,
+  // unless that pair has no unknowns (lines of one cell)
+  bool src_inside = fused && src;
+  for (int op = 0; op < 2 && src; ++op)
+    for (int q = 0; q < 3; ++q)
+      if (h->geom[op][q].ec == h->src_comp && h->geom[op][q].empty()) src_inside = false;
+  auto add_src = [&](double coef, int off) -> cudaError_t {
+    if (!src || coef == 0.0) return cudaSuccess;
+    if (h->prec == FDTD_F64)
+      fdtd::add_point_table_kernel<double><<<1, 32, 0, h->g_run>>>((double*)h->f[h->src_comp], src_at,
+                                                                   h->d_srcval, h->srcval_len, h->d_step, off, coef);
+    else
+      fdtd::add_point_table_kernel<float><<<1, 32, 0, h->g_run>>>((float*)h->f[h->src_comp], src_at, h->d_srcval,
+                                                                  h->srcval_len, h->d_step, off, coef);
+    h->launches++;
+    return cudaGetLastError();
+  };
+  cudaStream_t home = h->stream;
+  const long long before = h->launches;
+  NvtxScope range("step graph capture");
+  CK(cudaStreamBeginCapture(h->g_run, cudaStreamCaptureModeThreadLocal));
+  int rc = FDTD_OK;
+  bool chained = false;  // the last launch on g_run is a fused procedure
+  for (int st = 0; st < count && rc == FDTD_OK; ++st) {
     for (int k = 0; k < nproc && rc == FDTD_OK; ++k) {
-      if (add_src(pre[k], 0) != cudaSuccess) rc = FDTD_ERR_CUDA;
-      if (rc == FDTD_OK && add_src(pre2[k], 1) != cudaSuccess) rc = FDTD_ERR_CUDA;
+      if (fused) {
+        fdtd::FusedSource fs = no_source();
+        if (src_inside) {
+          fs.ec = h->src_comp;
+          fs.i = h->src_i;
+          fs.j = h->src_j;
+          fs.k = h->src_k;
+          fs.table = h->d_srcval;
+          fs.step = h->d_step;
+          fs.len = h->srcval_len;
+          fs.sub = st;
+          fs.pre[0] = pre[k];
+          fs.pre[1] = pre2[k];
+          fs.post[0] = post[k];
+          fs.post[1] = post2[k];
+          fs.pre_off[1] = fs.post_off[1] = 1;
+          fs.post_off[0] = post_off[k];
+        } else if (src && (add_src(pre[k], st) != cudaSuccess || add_src(pre2[k], st + 1) != cudaSuccess)) {
+          rc = FDTD_ERR_CUDA;
+        }
+        if (src && !src_inside) chained = false;
+        h->stream = h->g_run;
+        if (rc == FDTD_OK) rc = run_fused<float>(h, seq[k], 1.0, 1.0, -1.0, 1.0, h->f, h->f, fs, chained);
+        h->stream = home;
+        chained = true;
+        if (rc == FDTD_OK && src && !src_inside &&
+            (add_src(post[k], st + post_off[k]) != cudaSuccess || add_src(post2[k], st + 1) != cudaSuccess))
+          rc = FDTD_ERR_CUDA;
+        continue;
+      }
+      if (add_src(pre[k], st) != cudaSuccess) rc = FDTD_ERR_CUDA;
+      if (rc == FDTD_OK && add_src(pre2[k], st + 1) != cudaSuccess) rc = FDTD_ERR_CUDA;
       if (rc == FDTD_OK && cudaEventRecord(h->g_fork, h->g_run) != cudaSuccess) rc = FDTD_ERR_CUDA;
       const ProcCoef& P = h->proc[seq[k]];
       for (int q = 0; q < 3 && rc == FDTD_OK; ++q) {
@@ -1616,29 +1840,45 @@ int step_graph(fdtd_t* h, int64_t nsteps) {
                               cudaStreamWaitEvent(h->g_run, h->g_join[q], 0) != cudaSuccess))
           rc = FDTD_ERR_CUDA;
       }
-      if (rc == FDTD_OK && add_src(post[k], post_off[k]) != cudaSuccess) rc = FDTD_ERR_CUDA;
-      if (rc == FDTD_OK && add_src(post2[k], 1) != cudaSuccess) rc = FDTD_ERR_CUDA;
+      if (rc == FDTD_OK && add_src(post[k], st + post_off[k]) != cudaSuccess) rc = FDTD_ERR_CUDA;
+      if (rc == FDTD_OK && add_src(post2[k], st + 1) != cudaSuccess) rc = FDTD_ERR_CUDA;
     }
-    if (rc == FDTD_OK && src) {
-      fdtd::step_counter_kernel<<<1, 32, 0, h->g_run>>>(h->d_step, 0, 1);
-      h->launches++;
-      if (cudaGetLastError() != cudaSuccess) rc = FDTD_ERR_CUDA;
-    }
-    h->stream = home;
-    cudaGraph_t graph = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(h->g_run, &graph);
-    h->g_kernels = h->launches - before;
-    h->launches = before;
-    if (rc != FDTD_OK || e != cudaSuccess) {
-      if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
-      return rc != FDTD_OK ? rc : cuda_fail(h, e);
-    }
-    const cudaError_t ie = cudaGraphInstantiate(&h->g_exec, graph, 0);
-    cudaGraphDestroy(graph);
-    CK(ie);
-    h->g_bound = ptrs;
   }
+  if (rc == FDTD_OK && src) {
+    fdtd::step_counter_kernel<<<1, 32, 0, h->g_run>>>(h->d_step, count, 1);
+    h->launches++;
+    if (cudaGetLastError() != cudaSuccess) rc = FDTD_ERR_CUDA;
+  }
+  h->stream = home;
+  cudaGraph_t graph = nullptr;
+  const cudaError_t e = cudaStreamEndCapture(h->g_run, &graph);
+  *kernels = h->launches - before;
+  h->launches = before;
+  if (rc != FDTD_OK || e != cudaSuccess) {
+    if (graph) cudaGraphDestroy(graph);
+    cudaGetLastError();
+    return rc != FDTD_OK ? rc : cuda_fail(h, e);
+  }
+  const cudaError_t ie = cudaGraphInstantiate(exec, graph, 0);
+  cudaGraphDestroy(graph);
+  CK(ie);
+  return FDTD_OK;
+}
+
+// nsteps steps as graph replays: runs of kStepRun steps (fused procedures),
+// then single steps.  Recaptured when the state arrays moved.
+int step_graph(fdtd_t* h, int64_t nsteps) {
+  if (int rc = ensure_branches(h)) return rc;
+  const bool src = h->src_comp >= 0;
+  std::vector<const void*> ptrs(h->f, h->f + 6);
+  if (ptrs != h->g_bound) graph_release(h);
+  const int64_t runs = fused_ok(h) ? nsteps / kStepRun : 0;
+  const int64_t singles = nsteps - runs * kStepRun;
+  if (runs > 0 && !h->g_run_exec)
+    if (int rc = capture_steps(h, kStepRun, &h->g_run_exec, &h->g_run_kernels)) return rc;
+  if (singles > 0 && !h->g_exec)
+    if (int rc = capture_steps(h, 1, &h->g_exec, &h->g_kernels)) return rc;
+  h->g_bound = ptrs;
   CK(cudaEventRecord(h->g_in, h->stream));
   CK(cudaStreamWaitEvent(h->g_run, h->g_in, 0));
   if (src) {
@@ -1647,11 +1887,12 @@ int step_graph(fdtd_t* h, int64_t nsteps) {
   }
   {
     NvtxScope range("step graph replays");
-    for (int64_t k = 0; k < nsteps; ++k) CK(cudaGraphLaunch(h->g_exec, h->g_run));
+    for (int64_t k = 0; k < runs; ++k) CK(cudaGraphLaunch(h->g_run_exec, h->g_run));
+    for (int64_t k = 0; k < singles; ++k) CK(cudaGraphLaunch(h->g_exec, h->g_run));
   }
   CK(cudaEventRecord(h->g_out, h->g_run));
   CK(cudaStreamWaitEvent(h->stream, h->g_out, 0));
-  h->launches += nsteps * h->g_kernels;
+  h->launches += runs * h->g_run_kernels + singles * h->g_kernels;
   h->steps += nsteps;
   return FDTD_OK;
 }
@@ -2484,10 +2725,10 @@ int fdtd_step(fdtd_t* h, int64_t nsteps) {
   rc = scheme_init(h);
   if (rc) return rc;
   if ((rc = take_invariant_ref(h))) return rc;
-  if (h->per_node && !h->shape_tuned && h->desc.tune[0] == 0) {
+  if (h->per_node && !h->shape_tuned && h->desc.tune[0] == 0 && !fused_ok(h)) {
     if ((rc = single_tune(h))) return rc;
   }
-  h->shape_tuned = true;
+  if (!fused_ok(h)) h->shape_tuned = true;
   if ((rc = ensure_probe_capacity(h, h->steps + nsteps))) return rc;
   if (graph_usable(h)) {
     if ((rc = step_graph(h, nsteps))) return rc;
@@ -3538,6 +3779,10 @@ int fdtd_batch_create(fdtd_t* const* handles, int count, void* stream, fdtd_batc
   fdtd_batch_t* b = new (std::nothrow) fdtd_batch_s();
   if (!b) return FDTD_ERR_OOM;
   b->h.assign(handles, handles + count);
+  for (fdtd_t* h : b->h) {
+    if (!h->batched) graph_release(h);
+    h->batched = true;
+  }
   b->prec = handles[0]->prec;
   b->scheme = handles[0]->scheme;
   b->stream = (cudaStream_t)stream;
@@ -4103,6 +4348,7 @@ int fdtd_adj_create(fdtd_t* h, const int32_t block[6], int64_t nsteps, int32_t c
   fdtd_adj_t* a = new (std::nothrow) fdtd_adj_s();
   if (!a) return FDTD_ERR_OOM;
   a->h = h;
+  h->adjoint = true;
   a->nsteps = nsteps;
   a->every = checkpoint_every;
   a->nseg = (int)((nsteps + checkpoint_every - 1) / checkpoint_every);

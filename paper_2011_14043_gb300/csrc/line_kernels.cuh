@@ -116,6 +116,11 @@ struct PairParams {
                          // TB_KGH/TB_KGL) instead of table lanes near the walls
   int kg_len;            // the wall correction is zero from this node on (a multiple of
                          // the segment length)
+  // uniform media, x lines: carry products (-m)^(L d) of d = 1, 2, 4, 8, 16 segments
+  // (hi, lo); nscan: the first d whose product is below 2^-50 (the scan stops there);
+  // kx: the same in runs of 32 nodes (the y/z tiles' carries over warps)
+  T sc[2][5];
+  int nscan, kx;
   T* tmp4;               // fourth-order differences: field-shaped scratch of the line solve
   T c2_4;                // fourth-order difference weight -1/24 in the field precision
   int jc4, je4;          // fourth-order differences: the factor rows of nodes jc4..je4 all
@@ -1220,12 +1225,12 @@ __device__ __forceinline__ T warp_chain_backward(T b, HiLo<T> pm) {
 // One x line (a warp): solve and store.  E, H (and per-node qn, ibn, ibl)
 // hold the line's segment of this lane, zero past the line end.
 template <typename T, int L, bool PER_NODE>
-__device__ __forceinline__ void row_solve_store(const PairParams<T>& p, long long line, T (&E)[L], T (&H)[L],
+__device__ __forceinline__ void row_solve_store(const PairParams<T>& p, unsigned line, T (&E)[L], T (&H)[L],
                                                 const T (&qn)[L], const T (&ibn)[L], const T (&ibl)[L]) {
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int jo = p.o_lo + (int)(line % p.n_o);
-  const int ko = p.o2_lo + (int)(line / p.n_o);
+  const int jo = p.o_lo + (int)(line % (unsigned)p.n_o);
+  const int ko = p.o2_lo + (int)(line / (unsigned)p.n_o);
   const long long base = (long long)ko * p.os2 + (long long)jo * p.os;
   const bool ok = row_ok<T, L>(p, base);
   const int j0 = lane * L;
@@ -1304,6 +1309,20 @@ __device__ __forceinline__ void row_solve_store(const PairParams<T>& p, long lon
   }
 }
 
+// (r0, r1) = (a0, a1) (b0, b1) + (c0, c1): one packed FP32 FMA (the same
+// rounding as two scalar ones), two FP64 FMAs
+template <typename T>
+__device__ __forceinline__ void fma_pair(T& r0, T& r1, T a0, T a1, T b0, T b1, T c0, T c1) {
+  if constexpr (sizeof(T) == 4) {
+    const float2 r = __ffma2_rn(make_float2(a0, a1), make_float2(b0, b1), make_float2(c0, c1));
+    r0 = r.x;
+    r1 = r.y;
+  } else {
+    r0 = fma(a0, b0, c0);
+    r1 = fma(a1, b1, c1);
+  }
+}
+
 // One x line of a homogeneous medium without divergent lanes.  The line
 // matrix T (nodes 1..N-1) has LU factors that vary only near node 1 and
 // converge to constants; the constant factors L' U' are the exact LU of
@@ -1314,86 +1333,128 @@ __device__ __forceinline__ void row_solve_store(const PairParams<T>& p, long lon
 // kappa = delta / (1 - delta g_1): one broadcast of w'_1 and one hi + lo FMA
 // per node with kappa g_j from the table (it decays geometrically from the
 // wall; zero at node 0 and from node N on).  Node 0 and nodes >= N carry no
-// unknown: their right-hand side is zero, their factors 1/beta and c zero,
-// and node 0 is set to zero after the solve.  The result equals the
+// unknown: their y is zero before the backward sweep, which makes their w
+// zero, and node 0 is set to zero after it.  The result equals the
 // table-factor solve up to rounding (not bit for bit).
-template <typename T, int L, bool FULL_LINE = false>
-__device__ __forceinline__ void row_solve_store_wall(const PairParams<T>& p, long long line, T (&E)[L],
-                                                     T (&H)[L]) {
+//
+// LPL lanes of a warp hold one line (lane sl its nodes [sl L, sl L + L)).  A
+// segment's carry product is the constant (-m)^L, so the scans shuffle the
+// carries alone and stop after the first distance whose product is below
+// 2^-50.  What bounds these lines is instruction issue: the elementwise
+// parts run as packed FMAs on neighbouring nodes.
+// On return E, H hold the new values.
+template <typename T, int L, int LPL>
+__device__ __forceinline__ void row_solve_wall(const PairParams<T>& p, int sl, T (&E)[L], T (&H)[L]) {
   const unsigned FULL = 0xffffffffu;
+  const int j0 = sl * L;
+  const int N = p.N;
+  const HiLo<T> nm = {-p.cv[2], -p.cv[3]};
+  T y[L];
+  T hp = __shfl_up_sync(FULL, H[L - 1], 1, LPL);
+  if (sl == 0) hp = T(0);
+  // forward sweep with the constant multiplier
+#pragma unroll
+  for (int t = 0; t < L; t += 2) {
+    const int u = t + 1 < L ? t + 1 : t;
+    T r0, r1;
+    fma_pair<T>(r0, r1, p.kb, p.kb, H[t] - hp, H[u] - H[t], E[t], E[u]);
+    hp = H[u];
+    if (t == 0) r0 = sl == 0 ? T(0) : r0;  // node 0: the wall
+    y[t] = t == 0 ? r0 : fma2(nm, y[t == 0 ? 0 : t - 1], r0);
+    if (t + 1 < L) y[u] = fma2(nm, y[t], r1);
+  }
+  T a = y[L - 1];
+#pragma unroll
+  for (int d = 1, k = 0; d < LPL; d <<= 1, ++k) {
+    if (d >= p.nscan) break;
+    const T up = __shfl_up_sync(FULL, a, d, LPL);
+    const T an = d == 1 ? fma2(HiLo<T>{p.sc[0][0], p.sc[1][0]}, up, a) : fma(p.sc[0][k], up, a);
+    a = sl >= d ? an : a;
+  }
+  T yin = __shfl_up_sync(FULL, a, 1, LPL);
+  if (sl == 0) yin = T(0);
+#pragma unroll
+  for (int t = 0; t < L; t += 2) {
+    const int u = t + 1 < L ? t + 1 : t;
+    T v0 = y[t], v1 = y[u];
+    if constexpr (use_hilo<T>()) fma_pair<T>(v0, v1, p.qf[1][t], p.qf[1][u], yin, yin, v0, v1);
+    fma_pair<T>(v0, v1, p.qf[0][t], p.qf[0][u], yin, yin, v0, v1);
+    y[t] = v0;
+    if (t + 1 < L) y[u] = v1;
+  }
+  if (N != LPL * L) {  // the same for every lane
+#pragma unroll
+    for (int t = 0; t < L; ++t) y[t] = j0 + t < N ? y[t] : T(0);
+  }
+  T wn = T(0);
+#pragma unroll
+  for (int t = L - 1; t >= 0; --t) {
+    T u;
+    if constexpr (use_hilo<T>()) u = fma(nm.hi, wn, fma(nm.lo, wn, y[t] * p.cv[1]));
+    else u = nm.hi * wn;
+    y[t] = fma(y[t], p.cv[0], u);
+    wn = y[t];
+  }
+  T b = y[0];
+#pragma unroll
+  for (int d = 1, k = 0; d < LPL; d <<= 1, ++k) {
+    if (d >= p.nscan) break;
+    const T dn = __shfl_down_sync(FULL, b, d, LPL);
+    const T bn = d == 1 ? fma2(HiLo<T>{p.sc[0][0], p.sc[1][0]}, dn, b) : fma(p.sc[0][k], dn, b);
+    b = sl + d < LPL ? bn : b;
+  }
+  T win = __shfl_down_sync(FULL, b, 1, LPL);
+  if (sl == LPL - 1) win = T(0);
+#pragma unroll
+  for (int t = 0; t < L; t += 2) {
+    const int u = t + 1 < L ? t + 1 : t;
+    T v0 = y[t], v1 = y[u];
+    if constexpr (use_hilo<T>()) fma_pair<T>(v0, v1, p.qf[1][L - 1 - t], p.qf[1][L - 1 - u], win, win, v0, v1);
+    fma_pair<T>(v0, v1, p.qf[0][L - 1 - t], p.qf[0][L - 1 - u], win, win, v0, v1);
+    y[t] = v0;
+    if (t + 1 < L) y[u] = v1;
+  }
+  if (sl == 0) y[0] = T(0);  // node 0: the wall
+  // rank-one correction w = w' + kappa g w'_1 (w'_1: node 1, from its lane)
+  const T w1 = (L >= 2) ? __shfl_sync(FULL, y[1 % L], 0, LPL) : __shfl_sync(FULL, y[0], 1, LPL);
+  if (j0 < p.kg_len) {
+    const T* kg = p.tab + TB_KGH * p.tlen + j0;
+    const T* kl = p.tab + TB_KGL * p.tlen + j0;
+#pragma unroll
+    for (int t = 0; t < L; ++t) y[t] = fma2(HiLo<T>{__ldg(kg + t), __ldg(kl + t)}, w1, y[t]);
+  }
+  // H update needs w at the next lane's first node (after the correction)
+  T wnl = __shfl_down_sync(FULL, y[0], 1, LPL);
+  if (sl == LPL - 1) wnl = T(0);
+#pragma unroll
+  for (int t = 0; t < L; t += 2) {
+    const int u = t + 1 < L ? t + 1 : t;
+    const T n0 = (t + 1 < L) ? y[u] : wnl, n1 = (t + 2 < L) ? y[t + 2 < L ? t + 2 : t] : wnl;
+    T h0, h1, e0, e1;
+    fma_pair<T>(h0, h1, p.kd, p.kd, n0 - y[t], n1 - y[u], H[t], H[u]);
+    fma_pair<T>(e0, e1, p.beta, p.beta, E[t], E[u], p.alpha * y[t], p.alpha * y[u]);
+    H[t] = h0;
+    E[t] = e0;
+    if (t + 1 < L) {
+      H[u] = h1;
+      E[u] = e1;
+    }
+  }
+}
+
+// One warp per line: row_solve_wall and the stores.
+template <typename T, int L>
+__device__ __forceinline__ void row_solve_store_wall(const PairParams<T>& p, unsigned line, T (&E)[L], T (&H)[L]) {
   const int lane = threadIdx.x & 31;
-  const int jo = p.o_lo + (int)(line % p.n_o);
-  const int ko = p.o2_lo + (int)(line / p.n_o);
+  const int jo = p.o_lo + (int)(line % (unsigned)p.n_o);
+  const int ko = p.o2_lo + (int)(line / (unsigned)p.n_o);
   const long long base = (long long)ko * p.os2 + (long long)jo * p.os;
   const bool ok = row_ok<T, L>(p, base);
   const int j0 = lane * L;
   const int N = p.N;
-  // the wall correction of this lane's nodes (vector loads; cache-resident)
-  T kgh[L], kgl[L];
-  load_seg<T, L>(p.tab + TB_KGH * p.tlen + j0, kgh);
-  load_seg<T, L>(p.tab + TB_KGL * p.tlen + j0, kgl);
-  T y[L];
-  T hm1 = __shfl_up_sync(FULL, H[L - 1], 1);
-  if (lane == 0) hm1 = T(0);
-  const HiLo<T> m = {p.cv[2], p.cv[3]};
-  const HiLo<T> ib = {p.cv[0], p.cv[1]};
-  const HiLo<T> c = {p.cv[4], p.cv[5]};
-  // forward sweep with the constant multiplier
-  T hprev = hm1;
-#pragma unroll
-  for (int t = 0; t < L; ++t) {
-    const int j = j0 + t;
-    T r = fma(p.kb, H[t] - hprev, E[t]);
-    hprev = H[t];
-    if constexpr (FULL_LINE) {
-      if (t == 0) r = (lane == 0) ? T(0) : r;  // node 0: the wall
-    } else {
-      r = (j == 0 || j >= N) ? T(0) : r;
-    }
-    y[t] = (t == 0) ? r : fma2(HiLo<T>{-m.hi, -m.lo}, y[t - 1], r);
-  }
-  const T yin = warp_chain_forward<T>(y[L - 1], HiLo<T>{p.qf[0][L - 1], p.qf[1][L - 1]});
-#pragma unroll
-  for (int t = 0; t < L; ++t) y[t] = fma2(HiLo<T>{p.qf[0][t], p.qf[1][t]}, yin, y[t]);
-  // backward sweep; nodes >= N hold w = 0 and do not couple (masks by
-  // selects: one code path keeps the kernel at 48 registers, where two
-  // paths needed 64 and ran slower)
-  const bool full = FULL_LINE || j0 + L <= N;
-  T wn = T(0);
-#pragma unroll
-  for (int t = L - 1; t >= 0; --t) {
-    const bool in = FULL_LINE || j0 + t < N;
-    const T ch = in ? c.hi : T(0), cl = in ? c.lo : T(0);
-    const T ih = in ? ib.hi : T(0), il = in ? ib.lo : T(0);
-    T u;
-    if constexpr (use_hilo<T>()) u = fma(-ch, wn, fma(-cl, wn, y[t] * il));
-    else u = -ch * wn;
-    y[t] = fma(y[t], ih, u);
-    wn = y[t];
-  }
-  const HiLo<T> pb0 = full ? HiLo<T>{p.qb[0][0], p.qb[1][0]} : HiLo<T>{T(0), T(0)};
-  const T win = warp_chain_backward<T>(y[0], pb0);
-#pragma unroll
-  for (int t = 0; t < L; ++t) {
-    const HiLo<T> pbt = full ? HiLo<T>{p.qb[0][t], p.qb[1][t]} : HiLo<T>{T(0), T(0)};
-    y[t] = fma2(pbt, win, y[t]);
-  }
-  if (lane == 0) y[0] = T(0);  // node 0: the wall
-  // rank-one correction w = w' + kappa g w'_1 (w'_1: node 1, from its lane)
-  const T w1 = (L >= 2) ? __shfl_sync(FULL, y[1 % L], 0) : __shfl_sync(FULL, y[0], 1);
-#pragma unroll
-  for (int t = 0; t < L; ++t) y[t] = fma2(HiLo<T>{kgh[t], kgl[t]}, w1, y[t]);
-  // H update needs w at the next lane's first node (after the correction)
-  T wnl = __shfl_down_sync(FULL, y[0], 1);
-  if (lane == 31) wnl = T(0);
-#pragma unroll
-  for (int t = 0; t < L; ++t) {
-    const T wnext = (t + 1 < L) ? y[t + 1] : wnl;
-    H[t] = fma(p.kd, wnext - y[t], H[t]);
-  }
-  e_update<T, L>(p, y, E);
+  row_solve_wall<T, L, 32>(p, lane, E, H);
   if (!ok) return;
-  if (FULL_LINE || j0 + L <= N) {
+  if (j0 + L <= N) {
     store_seg<T, L>(p.e_out + base + j0, E);
     store_seg<T, L>(p.h_out + base + j0, H);
   } else if (j0 < N) {
@@ -1410,7 +1471,7 @@ __device__ __forceinline__ void row_solve_store_wall(const PairParams<T>& p, lon
 // Homogeneous media: the rank-one wall correction path when the host built
 // it (p.wall_fix), else the table lanes.
 template <typename T, int L>
-__device__ __forceinline__ void row_solve_store_uniform(const PairParams<T>& p, long long line, T (&E)[L], T (&H)[L],
+__device__ __forceinline__ void row_solve_store_uniform(const PairParams<T>& p, unsigned line, T (&E)[L], T (&H)[L],
                                                         const T (&qn)[L], const T (&ibn)[L], const T (&ibl)[L]) {
   if (p.wall_fix) row_solve_store_wall<T, L>(p, line, E, H);
   else row_solve_store<T, L, false>(p, line, E, H, qn, ibn, ibl);
@@ -1418,12 +1479,12 @@ __device__ __forceinline__ void row_solve_store_uniform(const PairParams<T>& p, 
 
 // Load this lane's segment of x line `line` (zeros past the line end).
 // Segments never run past the padded row (the row pitch is >= 32*L).
-template <typename T, int L, bool PER_NODE, bool FULL_LINE = false>
-__device__ __forceinline__ void row_load(const PairParams<T>& p, long long line, T (&E)[L], T (&H)[L],
+template <typename T, int L, bool PER_NODE>
+__device__ __forceinline__ void row_load(const PairParams<T>& p, unsigned line, T (&E)[L], T (&H)[L],
                                          T (&qn)[L], T (&ibn)[L], T (&ibl)[L]) {
   const int lane = threadIdx.x & 31;
-  const int jo = p.o_lo + (int)(line % p.n_o);
-  const int ko = p.o2_lo + (int)(line / p.n_o);
+  const int jo = p.o_lo + (int)(line % (unsigned)p.n_o);
+  const int ko = p.o2_lo + (int)(line / (unsigned)p.n_o);
   const long long base = (long long)ko * p.os2 + (long long)jo * p.os;
   const int j0 = lane * L;
 #pragma unroll
@@ -1434,7 +1495,7 @@ __device__ __forceinline__ void row_load(const PairParams<T>& p, long long line,
     ibn[t] = T(0);
     ibl[t] = T(0);
   }
-  if ((FULL_LINE || j0 < p.N) && row_ok<T, L>(p, base)) {  // lanes wholly past the line end touch no memory
+  if (j0 < p.N && row_ok<T, L>(p, base)) {  // lanes wholly past the line end touch no memory
     load_seg<T, L>(p.e_in + base + j0, E);
     load_seg<T, L>(p.h_in + base + j0, H);
     if constexpr (PER_NODE) {
@@ -1443,33 +1504,29 @@ __device__ __forceinline__ void row_load(const PairParams<T>& p, long long line,
       if constexpr (use_hilo<T>()) load_seg<T, L>(p.nibl + base + j0, ibl);
     }
   }
-  if constexpr (!FULL_LINE) {
 #pragma unroll
-    for (int t = 0; t < L; ++t) {
-      if (j0 + t >= p.N) {
-        E[t] = T(0);
-        H[t] = T(0);
-        qn[t] = T(0);
-        ibn[t] = T(0);
-        ibl[t] = T(0);
-      }
+  for (int t = 0; t < L; ++t) {
+    if (j0 + t >= p.N) {
+      E[t] = T(0);
+      H[t] = T(0);
+      qn[t] = T(0);
+      ibn[t] = T(0);
+      ibl[t] = T(0);
     }
   }
 }
 
 // One warp per x line.  WALL: homogeneous media with the rank-one wall
 // correction (p.wall_fix), a separate instantiation so that each path gets
-// its own register allocation.  FULL_LINE (with WALL): lines of exactly 32 L
-// cells, where every lane's nodes lie inside the line, so the end-of-line
-// masks go (the same arithmetic on every node that the masked path keeps).
-template <typename T, int L, bool PER_NODE, bool WALL = false, bool FULL_LINE = false>
+// its own register allocation.
+template <typename T, int L, bool PER_NODE, bool WALL = false>
 __global__ void proc_rows_kernel(const PairParams<T> p) {
-  const long long line = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (line >= (long long)p.n_o * p.n_o2) return;  // whole warp leaves together
+  const unsigned line = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (line >= (unsigned)p.n_o * (unsigned)p.n_o2) return;  // whole warp leaves together
   T E[L], H[L], qn[L], ibn[L], ibl[L];
-  row_load<T, L, PER_NODE, FULL_LINE>(p, line, E, H, qn, ibn, ibl);
+  row_load<T, L, PER_NODE>(p, line, E, H, qn, ibn, ibl);
   if constexpr (PER_NODE) row_solve_store<T, L, true>(p, line, E, H, qn, ibn, ibl);
-  else if constexpr (WALL) row_solve_store_wall<T, L, FULL_LINE>(p, line, E, H);
+  else if constexpr (WALL) row_solve_store_wall<T, L>(p, line, E, H);
   else row_solve_store<T, L, false>(p, line, E, H, qn, ibn, ibl);
 }
 
@@ -1595,7 +1652,7 @@ __global__ void __launch_bounds__((R + 1) * 32, MINB)
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[stage]);  // this warp is done with the stage
     if (jl < p.n_o) {
-      const long long line = (long long)kl * p.n_o + jl;
+      const unsigned line = (unsigned)kl * (unsigned)p.n_o + (unsigned)jl;
       if constexpr (WALL) row_solve_store_wall<T, L>(p, line, E, H);
       else row_solve_store<T, L, false>(p, line, E, H, qn, ibn, ibl);
     }
@@ -1740,7 +1797,7 @@ __global__ void proc_rows_batch_kernel(const PairParams<T>* __restrict__ params,
     else hi = mid;
   }
   const PairParams<T>& p = params[lo];
-  const long long line = gline - line_start[lo];
+  const unsigned line = (unsigned)(gline - line_start[lo]);
   T E[L], H[L], qn[L], ibn[L], ibl[L];
   if (p.nq != nullptr) {
     row_load<T, L, true>(p, line, E, H, qn, ibn, ibl);
@@ -1785,6 +1842,35 @@ __device__ __forceinline__ T group_chain_backward(T b, HiLo<T> pm, int sl) {
   }
   const T win = __shfl_down_sync(FULL, b, 1, LPL);
   return sl == LPL - 1 ? T(0) : win;
+}
+
+// One x line of a per-node medium on LPL lanes (lane sl its nodes
+// [sl L, sl L + L)): the solve of phase_forward / phase_backward with the
+// group scans.  On return E, H hold the new values.
+template <typename T, int L, int LPL>
+__device__ __forceinline__ void row_solve_pn(const PairParams<T>& p, int sl, T (&E)[L], T (&H)[L], const T (&qn)[L],
+                                             const T (&ibn)[L], const T (&ibl)[L]) {
+  const unsigned FULL = 0xffffffffu;
+  T y[L];
+  T hm1 = __shfl_up_sync(FULL, H[L - 1], 1, LPL);
+  HiLo<T> ib_prev = {__shfl_up_sync(FULL, ibn[L - 1], 1, LPL), T(0)};
+  if constexpr (use_hilo<T>()) ib_prev.lo = __shfl_up_sync(FULL, ibl[L - 1], 1, LPL);
+  if (sl == 0) {
+    hm1 = T(0);
+    ib_prev = {T(0), T(0)};
+  }
+  const int j0 = sl * L;
+  const HiLo<T> pf = phase_forward<T, L, 2>(p, j0, E, H, hm1, qn, ibn, ibl, ib_prev, y);
+  const T yin = group_chain_forward<T, LPL>(y[L - 1], pf, sl);
+  const HiLo<T> pb = phase_backward<T, L, 2>(p, j0, yin, ibn, ibl, ib_prev, y);
+  const T win = group_chain_backward<T, LPL>(y[0], pb, sl);
+  phase_fix<T, L, 2>(p, j0, win, ibn, ibl, y);
+#pragma unroll
+  for (int t = 0; t < L; ++t) {
+    const T wnext = (t + 1 < L) ? y[t + 1] : win;
+    H[t] = fma(p.kd, wnext - y[t], H[t]);
+  }
+  e_update<T, L>(p, y, E);
 }
 
 // x lines of uniform media, LPL lanes per line (32 / LPL lines per warp) and
@@ -1897,7 +1983,7 @@ __device__ __forceinline__ void rows_batch_pn_warp(const PairParams<T>* __restri
   const bool valid = in_batch && FDTD_IN_RANGE(base, base + N, p.n_elem);
   const bool full = j0 + L <= N;
 
-  T E[L], H[L], qn[L], ibn[L], ibl[L], y[L];
+  T E[L], H[L], qn[L], ibn[L], ibl[L];
 #pragma unroll
   for (int t = 0; t < L; ++t) {
     E[t] = T(0);
@@ -1927,25 +2013,7 @@ __device__ __forceinline__ void rows_batch_pn_warp(const PairParams<T>* __restri
       }
     }
   }
-  const unsigned FULL = 0xffffffffu;
-  T hm1 = __shfl_up_sync(FULL, H[L - 1], 1, LPL);
-  HiLo<T> ib_prev = {__shfl_up_sync(FULL, ibn[L - 1], 1, LPL), T(0)};
-  if constexpr (use_hilo<T>()) ib_prev.lo = __shfl_up_sync(FULL, ibl[L - 1], 1, LPL);
-  if (sl == 0) {
-    hm1 = T(0);
-    ib_prev = {T(0), T(0)};
-  }
-  const HiLo<T> pf = phase_forward<T, L, 2>(p, j0, E, H, hm1, qn, ibn, ibl, ib_prev, y);
-  const T yin = group_chain_forward<T, LPL>(y[L - 1], pf, sl);
-  const HiLo<T> pb = phase_backward<T, L, 2>(p, j0, yin, ibn, ibl, ib_prev, y);
-  const T win = group_chain_backward<T, LPL>(y[0], pb, sl);
-  phase_fix<T, L, 2>(p, j0, win, ibn, ibl, y);
-#pragma unroll
-  for (int t = 0; t < L; ++t) {
-    const T wnext = (t + 1 < L) ? y[t + 1] : win;
-    H[t] = fma(p.kd, wnext - y[t], H[t]);
-  }
-  e_update<T, L>(p, y, E);
+  row_solve_pn<T, L, LPL>(p, sl, E, H, qn, ibn, ibl);
   if (!valid) return;
   if (full) {
     store_seg<T, L>(p.e_out + base + j0, E);

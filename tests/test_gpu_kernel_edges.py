@@ -33,3 +33,30 @@ def check(nx, ny, nz, scheme, prec, steps=4, eps=None, tune=(0, 0), cfl=4.0):
 def test_media_formed_on_the_device(dims, prec):
     """Per-cell eps: means at the samples and line pivots from the device kernels."""
     check(*dims, "flod", prec, eps=random_media(*dims, 5))
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("media", ["uniform", "blocks"])
+@pytest.mark.parametrize("dims", [(2, 2, 2), (15, 9, 8), (16, 32, 7), (17, 33, 31), (64, 31, 32), (65, 64, 5),
+                                  (128, 5, 65), (129, 97, 3), (256, 3, 129), (5, 161, 96), (6, 256, 9), (3, 4, 255),
+                                  (33, 40, 1)])
+def test_procedure_in_one_launch(dims, media, prec):
+    """Lines along y, z and x of one procedure in one launch: line lengths on
+    both sides of a segment (8), a warp (32) and a tile (256), odd numbers of
+    columns, a source on the first and last unknown, runs of 16 steps and
+    single ones."""
+    from paper_2011_14043_gb300 import Simulation
+    nx, ny, nz = dims
+    d, steps = 1e-3, 19
+    eps = random_media(nx, ny, nz, 3) if media == "blocks" else None
+    u0 = random_fields(nx, ny, nz, 7)
+    dt = 5.0 * d / (299792458.0 * np.sqrt(3.0 if nz > 1 else 2.0))
+    cur = np.random.default_rng(1).standard_normal(steps) * 1e-3
+    for scheme, at in (("fadi", (1, 1, 0)), ("fss", (nx - 1, ny - 1, nz - 1)), ("flod2", (nx // 2, ny // 2, nz // 2))):
+        src = ("ez",) + at + (cur,)
+        out, _, _, sim = gpu_run(nx, ny, nz, d, d, d, dt, scheme, prec, u0, steps, eps=eps, source=src)
+        sim.close()
+        w0 = {c: v.astype(np.float32).astype(np.float64) if prec == "f32" else v for c, v in u0.items()}
+        ref, _, _ = S.run_fundamental(oracle_problem(nx, ny, nz, d, d, d, dt, eps=eps, source=src), scheme, w0, steps)
+        err = energy_norm_rel(out, ref)
+        assert err <= TOL[prec], (scheme, err)
