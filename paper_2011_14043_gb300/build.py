@@ -23,6 +23,7 @@ DEPENDS = SOURCES + [
     os.path.join(HERE, "csrc", "aux_kernels.cuh"),
     os.path.join(HERE, "csrc", "coef_kernels.cuh"),
     os.path.join(HERE, "csrc", "fused_kernels.cuh"),
+    os.path.join(HERE, "csrc", "plane_kernels.cuh"),
     os.path.join(HERE, "csrc", "adjoint_kernels.cuh"),
     os.path.join(HERE, "csrc", "line4_kernels.cuh"),
     os.path.join(ROOT, "include", "fdtd.h"),

@@ -34,6 +34,7 @@
 #include "coef_kernels.cuh"
 #include "line_kernels.cuh"
 #include "fused_kernels.cuh"
+#include "plane_kernels.cuh"
 #include "line4_kernels.cuh"
 
 namespace {
@@ -1723,6 +1724,38 @@ constexpr int kStepRun = 16;
 
 int ensure_branches(fdtd_t* h);
 
+// The source terms of one_step: coefficient of f added before and after each
+// procedure (0 = none), and the step offset of the value after it.
+struct SourceTerms {
+  double pre[3] = {0, 0, 0}, post[3] = {0, 0, 0};
+  double pre2[3] = {0, 0, 0}, post2[3] = {0, 0, 0};   // second terms, step offset 1
+  int post_off[3] = {0, 0, 0};
+};
+
+SourceTerms source_terms(const fdtd_t* h) {
+  SourceTerms s;
+  const double dt = h->dt;
+  if (h->scheme == FDTD_FADI) {
+    s.post[0] = 0.5 * dt;
+    s.post[1] = 0.5 * dt;
+    s.post_off[1] = 1;
+  } else if (h->scheme == FDTD_FSS) {
+    s.pre[0] = s.post[0] = 0.125 * dt;
+    s.pre[1] = s.post[1] = 0.25 * dt;
+    s.pre[2] = s.post[2] = 0.125 * dt;
+  } else if (h->scheme == FDTD_FLOD2) {
+    // B: (dt/4) of the mean of f(t_n + dt/2) and f(t_n + 3dt/2), as two
+    // terms (dt/8) f of offsets 0 and 1 (procedure_two_terms)
+    s.pre[0] = s.post[0] = 0.25 * dt;
+    s.pre[1] = s.post[1] = 0.125 * dt;
+    s.pre2[1] = s.post2[1] = 0.125 * dt;
+  } else {
+    s.pre[0] = s.post[0] = 0.25 * dt;
+    s.pre[1] = s.post[1] = 0.25 * dt;
+  }
+  return s;
+}
+
 // Capture `count` steps as a graph.  Fused procedures: one launch each, the
 // source added inside it, chained by programmatic edges.  Otherwise each
 // procedure forks its three pair launches (disjoint arrays) onto parallel
@@ -1739,30 +1772,9 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
   static const int seq_two[2] = {0, 1};
   const int* seq = h->scheme == FDTD_FSS ? seq_fss : seq_two;
   const int nproc = h->scheme == FDTD_FSS ? 3 : 2;
-  // the source terms of one_step: coefficient of f added before and after
-  // each procedure (0 = none), and the step offset of the value after it
-  const double dt = h->dt;
-  double pre[3] = {0, 0, 0}, post[3] = {0, 0, 0};
-  double pre2[3] = {0, 0, 0}, post2[3] = {0, 0, 0};   // second terms, step offset 1
-  int post_off[3] = {0, 0, 0};
-  if (h->scheme == FDTD_FADI) {
-    post[0] = 0.5 * dt;
-    post[1] = 0.5 * dt;
-    post_off[1] = 1;
-  } else if (h->scheme == FDTD_FSS) {
-    pre[0] = post[0] = 0.125 * dt;
-    pre[1] = post[1] = 0.25 * dt;
-    pre[2] = post[2] = 0.125 * dt;
-  } else if (h->scheme == FDTD_FLOD2) {
-    // B: (dt/4) of the mean of f(t_n + dt/2) and f(t_n + 3dt/2), as two
-    // terms (dt/8) f of offsets 0 and 1 (procedure_two_terms)
-    pre[0] = post[0] = 0.25 * dt;
-    pre[1] = post[1] = 0.125 * dt;
-    pre2[1] = post2[1] = 0.125 * dt;
-  } else {
-    pre[0] = post[0] = 0.25 * dt;
-    pre[1] = post[1] = 0.25 * dt;
-  }
+  const SourceTerms tm = source_terms(h);
+  const auto &pre = tm.pre, &post = tm.post, &pre2 = tm.pre2, &post2 = tm.post2;
+  const auto& post_off = tm.post_off;
   if (src && !h->d_step) CK(dev_malloc((void**)&h->d_step, sizeof(long long)));
   const long long src_at = src ? elem_index(h, h->src_i, h->src_j, h->src_k) : 0;
   // the sample lies on a line of its component's pair in either procedure,
@@ -1930,6 +1942,111 @@ int fork_pairs(fdtd_t* h, F&& launch) {
   }
   h->stream = home;
   return rc;
+}
+
+// ---------------------------------------------------------------------------
+// Small 2-D grids: every step in one launch (plane_kernels.cuh)
+// ---------------------------------------------------------------------------
+// Homogeneous media, sides that a warp holds as one line: 128 cells in FP64
+// (L <= 4; beyond, 16 SMs' FP64 pipes lose to the whole chip's) and 256 in
+// FP32 (L <= 8).  FP32 handles with probes keep the kernels whose rounding
+// their FP64 series have always shown; FLOD2 probes need the output
+// processing of the whole state every step.
+bool plane_ok(const fdtd_t* h) {
+  if (h->nz != 1 || h->order != 2 || h->per_node || h->mu_var || h->batched || h->adjoint || h->timing) return false;
+  if (h->desc.tune[0] != 0 || (h->desc.tune[1] & (1 | 4 | 8 | 16 | 128 | 1024)) != 0) return false;
+  const int most = h->prec == FDTD_F64 ? 128 : 256;
+  if (h->nx > most || h->ny > most) return false;
+  if (h->src_comp >= 0 && (h->src_comp != EZ || !h->d_srcval)) return false;
+  return h->nprobes == 0 || (h->prec == FDTD_F64 && h->scheme != FDTD_FLOD2);
+}
+
+template <typename T>
+const void* plane_fn(int L) {
+  if (L == 2) return (const void*)fdtd::plane_steps_kernel<T, 2>;
+  if (L == 4) return (const void*)fdtd::plane_steps_kernel<T, 4>;
+  if constexpr (sizeof(T) == 4) return (const void*)fdtd::plane_steps_kernel<T, 8>;
+  return nullptr;
+}
+
+template <typename T>
+int plane_steps(fdtd_t* h, int64_t nsteps) {
+  const int N = std::max(h->nx, h->ny);
+  const int L = N <= 64 ? 2 : (N <= 128 ? 4 : 8);
+  fdtd::PlaneParams<T> p = {};
+  for (int op = 0; op < 2; ++op)
+    for (int q = 0; q < 3; ++q) {
+      const PairGeom& g = h->geom[op][q];
+      if (g.ec != EZ) continue;
+      p.p[op] = make_params<T>(h, g, h->proc[op].pc[q], 1.0, 1.0, -1.0, 1.0, h->f, h->f);
+      set_scan(p.p[op], h->proc[op].pc[q], L);
+    }
+  p.ez = (T*)h->f[EZ];
+  p.hx = (T*)h->f[HX];
+  p.hy = (T*)h->f[HY];
+  p.nx = h->nx;
+  p.ny = h->ny;
+  p.pitch = h->pitch;
+  p.R = (h->ny + fdtd::kPlaneBlocks - 1) / fdtd::kPlaneBlocks;
+  p.ld = (h->nx + 1 + 3) / 4 * 4;
+  static const int seq_fss[3] = {0, 1, 0};
+  p.nproc = h->scheme == FDTD_FSS ? 3 : 2;
+  for (int k = 0; k < 3; ++k) p.seq[k] = seq_fss[k];
+  p.si = p.sj = -1;
+  if (h->src_comp >= 0) {
+    const SourceTerms tm = source_terms(h);
+    p.si = h->src_i;
+    p.sj = h->src_j;
+    p.table = h->d_srcval;
+    p.len = h->srcval_len;
+    for (int k = 0; k < 3; ++k) {
+      p.pre[k][0] = tm.pre[k];
+      p.pre[k][1] = tm.pre2[k];
+      p.post[k][0] = tm.post[k];
+      p.post[k][1] = tm.post2[k];
+      p.pre_off[k][1] = p.post_off[k][1] = 1;
+      p.post_off[k][0] = tm.post_off[k];
+    }
+  }
+  p.nprobes = h->nprobes;
+  p.average = h->scheme == FDTD_FADI ? 1 : 0;
+  for (int q = 0; q < h->nprobes; ++q) {
+    const int c = h->probe_comp[q];
+    const long long at = h->probe_at[q];
+    const int k = (int)(at / h->plane), j = (int)(at % h->plane / h->pitch), i = (int)(at % h->pitch);
+    p.pk[q] = (k > 0 || j >= h->ny || (c != EZ && c != HX && c != HY)) ? 3 : (c == EZ ? 0 : (c == HX ? 1 : 2));
+    p.pi[q] = i;
+    p.pj[q] = j;
+    p.pptr[q] = (const T*)h->f[c] + at;
+    p.pat_src[q] = c == h->src_comp && i == h->src_i && j == h->src_j && k == h->src_k;
+  }
+  p.out = h->d_probe;
+  p.cap = h->probe_cap;
+  const void* fn = plane_fn<T>(L);
+  const size_t smem = 3 * (size_t)p.R * p.ld * sizeof(T);
+  CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  CK(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(fdtd::kPlaneBlocks);
+  cfg.blockDim = dim3((unsigned)std::min(16, std::max(4, p.R)) * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = h->stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = fdtd::kPlaneBlocks;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  while (nsteps > 0) {  // launches of a few milliseconds
+    p.n0 = h->steps;
+    p.nsteps = std::min<int64_t>(nsteps, 2048);
+    void* args[] = {&p};
+    CK(cudaLaunchKernelExC(&cfg, fn, args));
+    h->launches++;
+    h->steps += p.nsteps;
+    nsteps -= p.nsteps;
+  }
+  return FDTD_OK;
 }
 
 int one_step(fdtd_t* h) {
@@ -2730,7 +2847,9 @@ int fdtd_step(fdtd_t* h, int64_t nsteps) {
   }
   if (!fused_ok(h)) h->shape_tuned = true;
   if ((rc = ensure_probe_capacity(h, h->steps + nsteps))) return rc;
-  if (graph_usable(h)) {
+  if (plane_ok(h)) {
+    if ((rc = h->prec == FDTD_F64 ? plane_steps<double>(h, nsteps) : plane_steps<float>(h, nsteps))) return rc;
+  } else if (graph_usable(h)) {
     if ((rc = step_graph(h, nsteps))) return rc;
   } else {
     for (int64_t q = 0; q < nsteps; ++q)

@@ -60,3 +60,31 @@ def test_procedure_in_one_launch(dims, media, prec):
         ref, _, _ = S.run_fundamental(oracle_problem(nx, ny, nz, d, d, d, dt, eps=eps, source=src), scheme, w0, steps)
         err = energy_norm_rel(out, ref)
         assert err <= TOL[prec], (scheme, err)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("dims", [(2, 2, 1), (3, 5, 1), (16, 17, 1), (64, 64, 1), (65, 33, 1), (63, 128, 1), (128, 127, 1),
+                                  (256, 20, 1)])
+def test_plane_steps_in_one_launch(dims, prec):
+    """2-D grids whose steps run in one launch: lines on both sides of a
+    lane's 2, 4 and 8 nodes, strips of one to several rows, a source and (FP64)
+    probes of every component at it, beside it and on the walls."""
+    nx, ny, nz = dims
+    d, steps = 1e-3, 7
+    u0 = random_fields(nx, ny, nz, 5)
+    dt = 5.0 * d / (299792458.0 * np.sqrt(2.0))
+    cur = np.random.default_rng(2).standard_normal(steps) * 1e-3
+    i, j = nx // 2, ny - 1
+    probes = [] if prec == "f32" else [("ez", i, j, 0), ("ez", 1, 1, 0), ("hx", nx, 0, 0), ("hy", 0, ny, 0),
+                                       ("hz", 0, 0, 1), ("hy", nx - 1, 1, 0), ("hx", 1, ny - 1, 0)]
+    w0 = {c: v.astype(np.float32).astype(np.float64) if prec == "f32" else v for c, v in u0.items()}
+    for scheme in ("fadi", "flod", "fss", "flod2"):
+        src = ("ez", i, j, 0, cur)
+        pr = probes if scheme != "flod2" else []
+        out, series, _, sim = gpu_run(nx, ny, nz, d, d, d, dt, scheme, prec, u0, steps, source=src, probes=pr)
+        sim.close()
+        P = oracle_problem(nx, ny, nz, d, d, d, dt, source=src)
+        ref, _, want = S.run_fundamental(P, scheme, w0, steps, probes=pr)
+        assert energy_norm_rel(out, ref) <= TOL[prec], scheme
+        for a, b in zip(series, want):
+            assert np.max(np.abs(a - b)) <= TOL[prec] * max(np.max(np.abs(b)), 1e-300), scheme
