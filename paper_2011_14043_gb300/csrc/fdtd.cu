@@ -109,6 +109,8 @@ struct fdtd_s {
   StridedCfg strided_cfg[2];  // y lines, z lines
   int num_sms = 0;
   int* d_err = nullptr;       // set by kernels whose bounded waits gave up
+  bool waits = false;         // a kernel with bounded waits is launched by this handle
+  bool err_due = false;       // ... and has run since the flag was last read
   bool use_tma = true;
   // TMA descriptors of the y/z line tiles, per component and box kind
   // TMA descriptors per component and box kind (0: y-line tiles, 1: z-line
@@ -1014,6 +1016,7 @@ int launch_strided_tma(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& 
                  : fdtd::proc_strided_tma_kernel<T, LANES, L, MINB, NST>;
   CK((ensure_tma_attr<T, LANES, MINB, NST>()));
   const int grid = std::min(q.n_tiles, MINB * h->num_sms);
+  h->waits = h->err_due = true;
   kern<<<grid, P * LANES, smem, h->stream>>>(*tE, *tH, p, q);
   return FDTD_OK;
 }
@@ -1079,6 +1082,7 @@ int launch_rows_tma(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<float>&
   q.tpp = (g.n_o + kRowsR - 1) / kRowsR;
   q.n_tiles = q.tpp * g.n_o2;
   CK(ensure_rows_tma_attr());
+  h->waits = h->err_due = true;
   switch ((h->desc.tune[1] >> 5) & 3) {
     case 1: launch_rows_tma_v<2, 4>(h, tE, tH, p, q); break;
     case 2: launch_rows_tma_v<4, 3>(h, tE, tH, p, q); break;
@@ -1288,8 +1292,10 @@ int launch_pair_raw(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) 
       case 32: launch_rows_L<T, 32>(h, g, p, pn); break;
       default: return FDTD_ERR_UNSUPPORTED;
     }
-  } else if (sizeof(T) == 4 && tma_eligible(h, g) && p.e_in == p.e_out && p.e_in == (const T*)h->f[g.ec] &&
-             p.h_in == (const T*)h->f[g.hc]) {
+  } else if (sizeof(T) == 4 && tma_eligible(h, g) && (p.e_in == p.e_out || (h->desc.tune[1] & 4) == 0) &&
+             p.e_in == (const T*)h->f[g.ec] && p.h_in == (const T*)h->f[g.hc]) {
+    // (the register-store kernel also writes out of place: the tensor maps
+    // only describe what it loads)
     // 16-line tiles, two blocks per SM, two-stage ring (measured at 256^3:
     // a three-stage ring 9 % slower, three blocks per SM 12 % slower, 32-line
     // tiles with one block per SM equal)
@@ -2102,23 +2108,38 @@ int one_step(fdtd_t* h) {
 }
 
 // Scratch receives the B procedure's (or explicit operator's) output line by
-// line; the samples no line of it covers keep the state's values: the three
-// H components are copied whole (their samples on the walls, normal H, are
-// in no line), and both arrays of a pair without unknowns (lines of one
-// cell).  E outside the lines is the walls and the row padding, zero in the
+// line; the samples no line of it covers keep the state's values: the H
+// samples on the walls (normal H) are copied, and both arrays of a pair
+// without unknowns (lines of one cell).  E outside the lines is the walls and the row padding, zero in the
 // state and in scratch alike (no kernel writes a nonzero value there).
 int copy_uncovered_to_scratch(fdtd_t* h, int slot) {
   int rc = ensure_scratch(h);
   if (rc) return rc;
   const ProcCoef& P = h->proc[slot];
   bool copied[6] = {false, false, false, false, false, false};
-  for (int c = 3; c < 6; ++c) copied[c] = true;
-  for (int q = 0; q < 3; ++q)
-    if (h->geom[P.op][q].empty()) copied[h->geom[P.op][q].ec] = true;
+  for (int q = 0; q < 3; ++q) {
+    const PairGeom& g = h->geom[P.op][q];
+    if (g.empty()) copied[g.ec] = copied[g.hc] = true;
+  }
   for (int c = 0; c < 6; ++c)
     if (copied[c])
       CK(cudaMemcpyAsync(h->scratch[c], h->f[c], (size_t)h->count * h->esize, cudaMemcpyDeviceToDevice,
                          h->stream));
+  auto walls = [&](auto zero) {
+    using T = decltype(zero);
+    fdtd::WallCopy<T> w;
+    for (int c = 0; c < 3; ++c) {
+      w.src[c] = (const T*)h->f[HX + c];
+      w.dst[c] = (T*)h->scratch[HX + c];
+    }
+    const long long most = 2LL * std::max({h->ny * (long long)h->nz, h->nx * (long long)h->nz, h->nx * (long long)h->ny});
+    fdtd::copy_h_walls_kernel<T><<<dim3((unsigned)std::min<long long>((most + 255) / 256, 152 * 8), 3), 256, 0,
+                                   h->stream>>>(w, h->nx, h->ny, h->nz, h->pitch, h->plane);
+  };
+  h->launches++;
+  if (h->prec == FDTD_F64) walls(0.0);
+  else walls(0.0f);
+  CK(cudaGetLastError());
   return FDTD_OK;
 }
 
@@ -2176,6 +2197,7 @@ int check_device_flag(fdtd_t* h) {
   CK(cudaMemcpyFromSymbol(&b, fdtd::g_bounds_err, sizeof(int)));
   if (b) return FDTD_ERR_BOUNDS;
 #endif
+  h->err_due = v != 0;
   return v ? FDTD_ERR_TIMEOUT : FDTD_OK;
 }
 
@@ -2258,6 +2280,28 @@ int stage_pack(fdtd_t* h, int sx, int sy, int sz, const void* src_padded) {
   return FDTD_OK;
 }
 
+// Between a padded component and the caller's compact device array by
+// repack_rows_kernel; 1 when the caller's pointer is not aligned to its
+// elements (the pitched copy takes any address).
+int repack(fdtd_t* h, bool pack, int sx, int sy, int sz, const void* src, void* dst) {
+  if (((uintptr_t)src | (uintptr_t)dst) % h->esize != 0) return 1;
+  const long long rows = (long long)sy * sz;
+  const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>((rows + 7) / 8, 152LL * 16));
+  auto go = [&](auto zero) {
+    using T = decltype(zero);
+    if (pack)
+      fdtd::repack_rows_kernel<T, true><<<blocks, 256, 0, h->stream>>>((const T*)src, (T*)dst, sx, sy, sz, h->pitch,
+                                                                       h->plane);
+    else
+      fdtd::repack_rows_kernel<T, false><<<blocks, 256, 0, h->stream>>>((const T*)src, (T*)dst, sx, sy, sz, h->pitch,
+                                                                        h->plane);
+  };
+  if (h->prec == FDTD_F64) go(0.0);
+  else go(0.0f);
+  CK(cudaGetLastError());
+  return FDTD_OK;
+}
+
 int copy_component(fdtd_t* h, int comp, const void* src_padded, void* dst, int on_device) {
   int sx, sy, sz;
   comp_extent(comp, h->nx, h->ny, h->nz, &sx, &sy, &sz);
@@ -2271,14 +2315,14 @@ int copy_component(fdtd_t* h, int comp, const void* src_padded, void* dst, int o
     CK(cudaStreamSynchronize(h->stream));
     return FDTD_OK;
   }
+  if (int rc = repack(h, true, sx, sy, sz, src_padded, dst); rc != 1) return rc;
   cudaMemcpy3DParms m = {};
   m.srcPtr = make_cudaPitchedPtr((void*)src_padded, (size_t)h->pitch * h->esize, (size_t)h->pitch,
                                  (size_t)(h->ny + 1));
   m.dstPtr = make_cudaPitchedPtr(dst, (size_t)sx * h->esize, (size_t)sx, (size_t)sy);
   m.extent = make_cudaExtent((size_t)sx * h->esize, (size_t)sy, (size_t)sz);
-  m.kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+  m.kind = cudaMemcpyDeviceToDevice;
   CK(cudaMemcpy3DAsync(&m, h->stream));
-  if (!on_device) CK(cudaStreamSynchronize(h->stream));
   return FDTD_OK;
 }
 
@@ -2299,14 +2343,14 @@ int copy_in_component(fdtd_t* h, int comp, const void* src, void* dst_padded, in
     CK(cudaStreamSynchronize(h->stream));
     return FDTD_OK;
   }
+  if (int rc = repack(h, false, sx, sy, sz, src, dst_padded); rc != 1) return rc;
   cudaMemcpy3DParms m = {};
   m.srcPtr = make_cudaPitchedPtr((void*)src, (size_t)sx * h->esize, (size_t)sx, (size_t)sy);
   m.dstPtr = make_cudaPitchedPtr(dst_padded, (size_t)h->pitch * h->esize, (size_t)h->pitch,
                                  (size_t)(h->ny + 1));
   m.extent = make_cudaExtent((size_t)sx * h->esize, (size_t)sy, (size_t)sz);
-  m.kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+  m.kind = cudaMemcpyDeviceToDevice;
   CK(cudaMemcpy3DAsync(&m, h->stream));
-  if (!on_device) CK(cudaStreamSynchronize(h->stream));
   return FDTD_OK;
 }
 
@@ -2759,7 +2803,12 @@ int fdtd_set_field(fdtd_t* h, int comp, const void* data, int on_device) {
 int fdtd_get_field(fdtd_t* h, int comp, void* out, int on_device) {
   if (!h || !out || check_comp(comp)) return FDTD_ERR_INVALID_ARG;
   if (h->poisoned) return FDTD_ERR_STATE;
-  if (int rc0 = check_device_flag(h)) return rc0;
+  // a read into device memory waits for the flag only when a kernel that can
+  // set it has run since it was last read
+#ifndef FDTD_BOUNDS
+  if (!on_device || h->err_due)
+#endif
+    if (int rc0 = check_device_flag(h)) return rc0;
   if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS || h->pending_init)
     return copy_component(h, comp, h->f[comp], out, on_device);
   int rc = physical_to_scratch(h);
@@ -2847,6 +2896,7 @@ int fdtd_step(fdtd_t* h, int64_t nsteps) {
   }
   if (!fused_ok(h)) h->shape_tuned = true;
   if ((rc = ensure_probe_capacity(h, h->steps + nsteps))) return rc;
+  if (h->waits) h->err_due = true;
   if (plane_ok(h)) {
     if ((rc = h->prec == FDTD_F64 ? plane_steps<double>(h, nsteps) : plane_steps<float>(h, nsteps))) return rc;
   } else if (graph_usable(h)) {

@@ -88,3 +88,36 @@ def test_plane_steps_in_one_launch(dims, prec):
         assert energy_norm_rel(out, ref) <= TOL[prec], scheme
         for a, b in zip(series, want):
             assert np.max(np.abs(a - b)) <= TOL[prec] * max(np.max(np.abs(b)), 1e-300), scheme
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("dims", [(2, 3, 1), (31, 4, 3), (32, 5, 2), (255, 3, 4), (256, 2, 3), (257, 3, 2), (520, 2, 2)])
+def test_device_copies_of_every_component(dims, prec):
+    """Fields set from and read into device memory: rows on both sides of a
+    warp (32) and of a lane's 8 elements in flight (256), from tensors that
+    start one element into their storage; before a step and after FADI's
+    output processing (wall samples of H included)."""
+    import torch
+    from paper_2011_14043_gb300 import Simulation
+    u0 = random_fields(*dims, 3)
+    dt = torch.float64 if prec == "f64" else torch.float32
+    npt = np.float64 if prec == "f64" else np.float32
+    for scheme in ("flod", "fadi"):
+        host = Simulation(*dims, 1e-3, scheme=scheme, precision=prec, cfl=3.0)
+        dev = Simulation(*dims, 1e-3, scheme=scheme, precision=prec, cfl=3.0)
+        for c, v in u0.items():
+            host.set_field(c, v)
+            store = torch.empty(v.size + 1, dtype=dt, device="cuda")
+            t = store[1:].view(*v.shape)
+            t.copy_(torch.from_numpy(v))
+            dev.set_field(c, t)
+            assert np.array_equal(dev.get_field(c, device=True).cpu().numpy(), v.astype(npt)), c
+        host.step(2)
+        dev.step(2)
+        for c in u0:
+            a = host.get_field(c)
+            assert np.array_equal(dev.get_field(c, device=True).cpu().numpy(), a), (scheme, c)
+        for c, w in (("hx", (slice(None), slice(None), 0)), ("hy", (slice(None), -1)), ("hz", (0,))):
+            assert np.array_equal(host.get_field(c)[w], u0[c].astype(npt)[w]), c
+        host.close()
+        dev.close()
