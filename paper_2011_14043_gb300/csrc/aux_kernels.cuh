@@ -202,6 +202,11 @@ struct ProbeParams {
   long long at[kMaxProbes];
   double sub[kMaxProbes];  // mode 1: subtracted from value (a source added after the solve)
   int n;
+  // captured steps (step != nullptr): col counts from *step, and sub is the
+  // coefficient of table[*step + table_off]
+  const long long* step;
+  const double* table;
+  long long table_len, table_off;
 };
 
 // mode 0: stash[p] = value;  mode 1: out[p][col] = (stash[p] + value - sub[p])/2;
@@ -212,10 +217,18 @@ __global__ void probe_kernel(const ProbeParams<T> pp, double* stash, double* out
   const int q = threadIdx.x;
   if (q >= pp.n) return;
   const double v = (double)pp.arr[q][pp.at[q]];
+  double sub = pp.sub[q];
+  if (pp.step) {
+    // a captured step: the column and the added source's value from the
+    // device step counter
+    const long long n = *pp.step + pp.table_off;
+    if (sub != 0.0) sub = __dmul_rn(sub, (n >= 0 && n < pp.table_len) ? pp.table[n] : 0.0);
+    col += *pp.step;
+  }
   if (mode == 0) {
     stash[q] = v;
   } else if (mode == 1) {
-    out[(long long)q * ld + col] = 0.5 * (stash[q] + v - pp.sub[q]);
+    out[(long long)q * ld + col] = 0.5 * (stash[q] + v - sub);
   } else {
     out[(long long)q * ld + col] = v;
   }

@@ -1656,10 +1656,12 @@ int scheme_init(fdtd_t* h) {
   return FDTD_OK;
 }
 
+// sub_step >= 0: inside a captured step, that many steps past the device
+// counter; post is then the coefficient of the source value at offset 1.
 template <typename T>
-int record_probes(fdtd_t* h, int mode, double post, void* const* arrays) {
+int record_probes(fdtd_t* h, int mode, double post, void* const* arrays, int sub_step = -1) {
   if (h->nprobes == 0) return FDTD_OK;
-  fdtd::ProbeParams<T> pp;
+  fdtd::ProbeParams<T> pp = {};
   pp.n = h->nprobes;
   const long long src_at = h->src_comp >= 0 ? elem_index(h, h->src_i, h->src_j, h->src_k) : -1;
   for (int q = 0; q < h->nprobes; ++q) {
@@ -1668,7 +1670,14 @@ int record_probes(fdtd_t* h, int mode, double post, void* const* arrays) {
     pp.sub[q] = (h->probe_comp[q] == h->src_comp && h->probe_at[q] == src_at) ? post : 0.0;
   }
   h->launches++;
-  fdtd::probe_kernel<T><<<1, 32, 0, h->stream>>>(pp, h->d_stash, h->d_probe, h->probe_cap, h->steps, mode);
+  if (sub_step >= 0) {
+    pp.step = h->d_step;
+    pp.table = h->d_srcval;
+    pp.table_len = h->d_srcval ? h->srcval_len : 0;
+    pp.table_off = sub_step + 1;
+  }
+  fdtd::probe_kernel<T><<<1, 32, 0, h->stream>>>(pp, h->d_stash, h->d_probe, h->probe_cap,
+                                                 sub_step >= 0 ? sub_step : h->steps, mode);
   CK(cudaGetLastError());
   return FDTD_OK;
 }
@@ -1681,10 +1690,13 @@ int probes(fdtd_t* h, int mode, double post = 0.0, void* const* arrays = nullptr
                              : record_probes<float>(h, mode, post, arrays);
 }
 
+void graph_release(fdtd_t* h);
+
 int ensure_probe_capacity(fdtd_t* h, long long need) {
   if (h->nprobes == 0 || need <= h->probe_cap) return FDTD_OK;
   long long cap = std::max<long long>(need, 2 * h->probe_cap);
   cap = std::max<long long>(cap, 1024);
+  graph_release(h);  // captured steps write the old buffer
   double* np = nullptr;
   CK(dev_malloc((void**)&np, sizeof(double) * fdtd::kMaxProbes * cap));
   CK(cudaMemsetAsync(np, 0, sizeof(double) * fdtd::kMaxProbes * cap, h->stream));
@@ -1719,8 +1731,9 @@ void graph_release(fdtd_t* h) {
   h->g_bound.clear();
 }
 
+// (FLOD2 probes run the output processing of every step, one by one)
 bool graph_usable(const fdtd_t* h) {
-  return !h->timing && h->nprobes == 0 && (h->desc.tune[1] & 8) == 0 &&
+  return !h->timing && (h->nprobes == 0 || h->scheme != FDTD_FLOD2) && (h->desc.tune[1] & 8) == 0 &&
          (h->src_comp < 0 || h->d_srcval != nullptr);
 }
 
@@ -1781,7 +1794,8 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
   const SourceTerms tm = source_terms(h);
   const auto &pre = tm.pre, &post = tm.post, &pre2 = tm.pre2, &post2 = tm.post2;
   const auto& post_off = tm.post_off;
-  if (src && !h->d_step) CK(dev_malloc((void**)&h->d_step, sizeof(long long)));
+  const bool counted = src || h->nprobes > 0;  // the step reads the device step counter
+  if (counted && !h->d_step) CK(dev_malloc((void**)&h->d_step, sizeof(long long)));
   const long long src_at = src ? elem_index(h, h->src_i, h->src_j, h->src_k) : 0;
   // the sample lies on a line of its component's pair in either procedure,
   // unless that pair has no unknowns (lines of one cell)
@@ -1860,9 +1874,18 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
       }
       if (rc == FDTD_OK && add_src(post[k], st + post_off[k]) != cudaSuccess) rc = FDTD_ERR_CUDA;
       if (rc == FDTD_OK && add_src(post2[k], st + 1) != cudaSuccess) rc = FDTD_ERR_CUDA;
+      // probes as one_step records them
+      if (rc == FDTD_OK && h->nprobes > 0 && (h->scheme == FDTD_FADI || k == nproc - 1)) {
+        const int mode = h->scheme == FDTD_FADI ? k : 2;
+        const double sub = mode == 1 ? post[1] : 0.0;
+        h->stream = h->g_run;
+        rc = h->prec == FDTD_F64 ? record_probes<double>(h, mode, sub, h->f, st)
+                                 : record_probes<float>(h, mode, sub, h->f, st);
+        h->stream = home;
+      }
     }
   }
-  if (rc == FDTD_OK && src) {
+  if (rc == FDTD_OK && counted) {
     fdtd::step_counter_kernel<<<1, 32, 0, h->g_run>>>(h->d_step, count, 1);
     h->launches++;
     if (cudaGetLastError() != cudaSuccess) rc = FDTD_ERR_CUDA;
@@ -1887,7 +1910,7 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
 // then single steps.  Recaptured when the state arrays moved.
 int step_graph(fdtd_t* h, int64_t nsteps) {
   if (int rc = ensure_branches(h)) return rc;
-  const bool src = h->src_comp >= 0;
+  const bool src = h->src_comp >= 0;  // (a step without a source or probes reads no counter)
   std::vector<const void*> ptrs(h->f, h->f + 6);
   if (ptrs != h->g_bound) graph_release(h);
   const int64_t runs = fused_ok(h) ? nsteps / kStepRun : 0;
@@ -1899,7 +1922,7 @@ int step_graph(fdtd_t* h, int64_t nsteps) {
   h->g_bound = ptrs;
   CK(cudaEventRecord(h->g_in, h->stream));
   CK(cudaStreamWaitEvent(h->g_run, h->g_in, 0));
-  if (src) {
+  if (src || h->nprobes > 0) {
     fdtd::step_counter_kernel<<<1, 32, 0, h->g_run>>>(h->d_step, h->steps, 0);
     CK(cudaGetLastError());
   }
@@ -2872,6 +2895,7 @@ int fdtd_add_probe(fdtd_t* h, int comp, int i, int j, int k, int* id) {
   int sx, sy, sz;
   comp_extent(comp, h->nx, h->ny, h->nz, &sx, &sy, &sz);
   if (i < 0 || j < 0 || k < 0 || i >= sx || j >= sy || k >= sz) return FDTD_ERR_INVALID_ARG;
+  graph_release(h);  // captured steps know the probes
   const int q = h->nprobes;
   h->probe_comp[q] = comp;
   h->probe_at[q] = elem_index(h, i, j, k);
