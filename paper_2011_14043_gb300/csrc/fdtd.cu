@@ -1347,24 +1347,34 @@ int launch_pair(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
 // batch's handles the kernels that the batch steps them by, and handles with
 // probes the kernels whose rounding their FP64 series have always shown.
 //
-// The line: a procedure that moves at most 256 MB (24 B per cell, 60 B with
-// per-node media), about twice the L2 cache.  FADI steps, fused against a
-// launch per pair on parallel branches, us: 20^3 7.2 / 15.5, 64^3 9.9 / 16.5,
-// 96^3 15.9 / 28.9, 128^3 30.8 / 37.3, 219x101x75 30.3 / 45.7, 192^3
-// 119 / 134, 224^3 206 / 200, 256^3 285 / 273; per-node 64^3 9.9 / 15.3,
-// 128^3 55.7 / 61.7, 160^3 125 / 127, 192^3 243 / 222, 256^3 516 / 473: beyond
-// it, HBM-bound launches want the TMA ring (y, z) and the one-warp-per-line
-// kernel's 40 warps per SM (x).  FP64 fields gain nothing (their pipe binds:
-// 40^3 44.5 against 33.5).
-constexpr double kFusedMaxBytes = 256e6;
+// The line: a procedure that moves at most 256 MB (24 B per cell), about twice
+// the L2 cache, or 150 MB with per-node media (60 B per cell).  FADI steps,
+// fused against a launch per pair on parallel branches, us: 20^3 7.2 / 15.5,
+// 64^3 9.9 / 16.5, 96^3 15.9 / 28.9, 128^3 30.8 / 37.3, 219x101x75 30.3 / 45.7,
+// 192^3 119 / 134, 224^3 206 / 200, 256^3 285 / 273; per-node 64^3 10.5 / 15.3,
+// 96^3 27.7 / 30.9, 128^3 58.6 / 61.7, 150x117x203 127 / 122, 192^3 243 / 222:
+// beyond it, HBM-bound launches want the TMA ring (y, z) and the
+// one-warp-per-line kernel's 40 warps per SM (x).  FP64 fields gain nothing
+// (their pipe binds: 40^3 44.5 against 33.5).  Per-node tiles hold 128
+// registers, 2 blocks per SM; with E and H loaded again after the solve and 3
+// blocks (80 registers, spills) 128^3 took 92 us.
+constexpr double kFusedMaxBytes = 256e6, kFusedMaxBytesPerNode = 150e6;
 
-bool fused_ok(const fdtd_t* h) {
-  if (h->order != 2 || h->mu_var || h->adjoint || h->batched || h->nprobes > 0 || h->desc.tune[0] != 0 || (h->desc.tune[1] & (1 | 4 | 128)) != 0)
-    return false;
+bool fused_shape_ok(const fdtd_t* h) {
+  if (h->order != 2 || h->mu_var || h->desc.tune[0] != 0 || (h->desc.tune[1] & (1 | 4 | 128)) != 0) return false;
   if (h->nx > fdtd::kFusedMaxN || h->ny > fdtd::kFusedMaxN || h->nz > fdtd::kFusedMaxN) return false;
   if ((unsigned long long)h->count * h->esize > 0xffffffffull) return false;
-  return h->prec == FDTD_F32 &&
-         (h->per_node ? 60.0 : 24.0) * (double)h->nx * h->ny * h->nz <= kFusedMaxBytes;
+  return h->prec == FDTD_F32;
+}
+// A dipole in a homogeneous box drives some components alone; the others then
+// sit at the rounding level of the driven ones, and any other order of
+// roundings moves them by as much as they are wrong (Hz under a z dipole: 7e-5
+// off either way, 9e-5 apart).  Such runs keep the kernels they had.
+bool fused_ok(const fdtd_t* h) {
+  if (h->src_comp >= 0 && !h->per_node) return false;
+  return !h->adjoint && !h->batched && h->nprobes == 0 && fused_shape_ok(h) &&
+         (double)h->nx * h->ny * h->nz * (h->per_node ? 60.0 : 24.0) <=
+             (h->per_node ? kFusedMaxBytesPerNode : kFusedMaxBytes);
 }
 
 unsigned reciprocal(int d) { return d <= 1 ? 0u : (unsigned)(((1ull << 32) + (unsigned)d - 1) / (unsigned)d); }
@@ -1390,16 +1400,44 @@ fdtd::FusedSource no_source() {
   return s;
 }
 
-// The pairs of procedure `slot` named by `mask` (bit 0: lines along y, 1: z,
-// 2: x) in one launch.  chained: the launch before it on the stream is
-// another procedure of the same captured step (programmatic edge).
+// Warps per tile of the y and z lines of procedure `slot`, and their tiles.
 template <typename T>
-int launch_fused(fdtd_t* h, int slot, double sgn, double alpha, double beta, double kd_mul, void* const* in,
-                 void* const* out, const fdtd::FusedSource& src, bool chained, int mask) {
+void fused_tiles(const fdtd_t* h, int slot, int (&nwarps)[2], unsigned (&ntiles)[2], int (&tiles_x)[2]) {
+  for (int d = 0; d < 2; ++d) {
+    nwarps[d] = tiles_x[d] = 1;
+    ntiles[d] = 0;
+  }
   const ProcCoef& P = h->proc[slot];
-  fdtd::FusedParams<T> fp;
-  fp.src = src;
-  int nwarps[3] = {1, 1, 1};
+  for (int q = 0; q < 3; ++q) {
+    const PairGeom& g = h->geom[P.op][q];
+    if (g.rows) continue;
+    const int d = g.axis == AX_Y ? 0 : 1, lines = 8 * fdtd::Wide<T>::V;
+    tiles_x[d] = std::max(1, (g.lane_hi + lines - 1) / lines);
+    nwarps[d] = std::max(1, (g.N + 4 * fdtd::kFusedL - 1) / (4 * fdtd::kFusedL));
+    if (!g.empty()) ntiles[d] = (unsigned)tiles_x[d] * (unsigned)g.n_o;
+  }
+}
+
+// Warps idle at `bw` warps per block (a block holds whole tiles), as the warps
+// launched; infinite where a tile does not fit.
+double fused_block_cost(const int (&nwarps)[2], const unsigned (&ntiles)[2], int bw) {
+  double cost = 0;
+  for (int d = 0; d < 2; ++d) {
+    if (ntiles[d] == 0) continue;
+    if (bw < nwarps[d]) return 1e30;
+    cost += (double)ntiles[d] * bw / (bw / nwarps[d]);
+  }
+  return cost;
+}
+
+// The pairs of procedure `slot` named by `mask` (bit 0: lines along y, 1: z,
+// 2: x); bw: warps per block.  Returns the blocks.
+template <typename T>
+unsigned fused_fill(const fdtd_t* h, int slot, double sgn, double alpha, double beta, double kd_mul, void* const* in,
+                    void* const* out, int mask, int bw, fdtd::FusedParams<T>& fp) {
+  const ProcCoef& P = h->proc[slot];
+  int nwarps[2];
+  fused_tiles<T>(h, slot, nwarps, fp.ntiles, fp.tiles_x);
   bool on[3];
   for (int q = 0; q < 3; ++q) {
     const PairGeom& g = h->geom[P.op][q];
@@ -1408,50 +1446,45 @@ int launch_fused(fdtd_t* h, int slot, double sgn, double alpha, double beta, dou
     set_scan(fp.p[d], P.pc[q], fdtd::kFusedL);
     fp.ec[d] = g.ec;
     on[d] = !g.empty() && (mask >> d & 1) != 0;
-    if (d == 2) {
-      fp.div[2] = reciprocal(std::max(1, g.n_o));
-    } else {
-      const int lines = 8 * fdtd::Wide<T>::V;
-      fp.tiles_x[d] = std::max(1, (g.lane_hi + lines - 1) / lines);
-      fp.ntiles[d] = on[d] ? (unsigned)fp.tiles_x[d] * (unsigned)g.n_o : 0u;
-      fp.div[d] = reciprocal(fp.tiles_x[d]);
-      nwarps[d] = std::max(1, (g.N + 4 * fdtd::kFusedL - 1) / (4 * fdtd::kFusedL));
-    }
-  }
-  // warps per block: the count (4..8) that leaves the fewest warps idle over
-  // the y and z tiles (a block holds whole tiles)
-  int bw = 8;
-  double least = 1e30;
-  for (int w = 8; w >= 4; --w) {
-    double cost = 0;
-    for (int d = 0; d < 2; ++d) {
-      if (fp.ntiles[d] == 0) continue;
-      if (w < nwarps[d]) cost = 1e30;
-      else cost += (double)fp.ntiles[d] * w / (w / nwarps[d]);
-    }
-    if (cost < least) {
-      least = cost;
-      bw = w;
-    }
+    fp.div[d] = reciprocal(d == 2 ? std::max(1, g.n_o) : fp.tiles_x[d]);
   }
   for (int d = 0; d < 2; ++d) {
+    if (!on[d]) fp.ntiles[d] = 0;
     fp.wpt[d] = nwarps[d];
     fp.tpb[d] = std::max(1, bw / nwarps[d]);
     fp.nb[d] = (int)((fp.ntiles[d] + (unsigned)fp.tpb[d] - 1) / (unsigned)fp.tpb[d]);
   }
-  const int lpl = h->nx <= 64 ? 8 : (h->nx <= 128 ? 16 : 32);
+  fp.lpl = h->nx <= 64 ? 8 : (h->nx <= 128 ? 16 : 32);
   const unsigned rows = on[2] ? (unsigned)fp.p[2].n_o * (unsigned)fp.p[2].n_o2 : 0u;
-  const unsigned rpb = (unsigned)(bw * (32 / lpl));
+  const unsigned rpb = (unsigned)(bw * (32 / fp.lpl));
   fp.nb[2] = (int)((rows + rpb - 1) / rpb);
-  const unsigned blocks = (unsigned)(fp.nb[0] + fp.nb[1] + fp.nb[2]);
+  fp.src = no_source();
+  return (unsigned)(fp.nb[0] + fp.nb[1] + fp.nb[2]);
+}
+
+// The pairs named by `mask` in one launch.  chained: the launch before it on
+// the stream is another procedure of the same captured step (programmatic
+// edge).
+template <typename T>
+int launch_fused(fdtd_t* h, int slot, double sgn, double alpha, double beta, double kd_mul, void* const* in,
+                 void* const* out, const fdtd::FusedSource& src, bool chained, int mask) {
+  int nwarps[2], tiles_x[2];
+  unsigned ntiles[2];
+  fused_tiles<T>(h, slot, nwarps, ntiles, tiles_x);
+  int bw = 8;
+  for (int w = 7; w >= 4; --w)
+    if (fused_block_cost(nwarps, ntiles, w) < fused_block_cost(nwarps, ntiles, bw)) bw = w;
+  fdtd::FusedParams<T> fp;
+  const unsigned blocks = fused_fill<T>(h, slot, sgn, alpha, beta, kd_mul, in, out, mask, bw, fp);
+  fp.src = src;
   if (blocks == 0) return FDTD_OK;
   const unsigned threads = (unsigned)bw * 32;
   const bool pn = h->per_node;
   cudaError_t e;
-  if (lpl == 8)
+  if (fp.lpl == 8)
     e = pn ? launch_fused_k<T, true, 8>(fp, blocks, threads, h->stream, chained)
            : launch_fused_k<T, false, 8>(fp, blocks, threads, h->stream, chained);
-  else if (lpl == 16)
+  else if (fp.lpl == 16)
     e = pn ? launch_fused_k<T, true, 16>(fp, blocks, threads, h->stream, chained)
            : launch_fused_k<T, false, 16>(fp, blocks, threads, h->stream, chained);
   else
@@ -3048,7 +3081,6 @@ struct fdtd_batch_s {
   cudaEvent_t ev_join[kBatchBranches] = {nullptr, nullptr, nullptr, nullptr};
   std::vector<BatchGroup> groups[2];           // per procedure slot
   std::vector<const void*> bound;              // state pointers the tables were built for
-  cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   BatchCfg cfg;
   bool tuned = false;       // cfg chosen (by the tuner, the cache or the caller)
@@ -3069,6 +3101,16 @@ struct fdtd_batch_s {
     size_t smem = 0;
   } pl[2];
   int* d_counter = nullptr;    // one work counter per procedure of a step
+  // mode 0 as the tuner found it faster: one launch of proc_fused_batch_kernel
+  // per procedure and media kind
+  int tuned_fused = -1;
+  bool fused = false;
+  struct Fused {
+    void* d_grids = nullptr;   // FusedParams<float>[grids of the kind]
+    int2* d_blocks = nullptr;  // (grid, block within it)
+    unsigned nblocks = 0, threads = 256;
+  } fl[2][2];                  // [procedure slot][0: homogeneous, 1: per-node media]
+  cudaGraphExec_t exec_run = nullptr;  // kStepRun steps (fused)
 };
 
 namespace {
@@ -3090,14 +3132,24 @@ void free_persistent(fdtd_batch_t::Persistent (&pl)[2]) {
   }
 }
 
+void free_fused(fdtd_batch_t::Fused (&fl)[2][2]) {
+  for (auto& slot : fl)
+    for (auto& q : slot) {
+      if (q.d_grids) cudaFree(q.d_grids);
+      if (q.d_blocks) cudaFree(q.d_blocks);
+      q = fdtd_batch_t::Fused();
+    }
+}
+
 void free_groups(fdtd_batch_t* b) {
+  free_fused(b->fl);
+  if (b->exec_run) cudaGraphExecDestroy(b->exec_run);
+  b->exec_run = nullptr;
   free_group_list(b->groups[0]);
   free_group_list(b->groups[1]);
   free_persistent(b->pl);
   if (b->exec) cudaGraphExecDestroy(b->exec);
-  if (b->graph) cudaGraphDestroy(b->graph);
   b->exec = nullptr;
-  b->graph = nullptr;
 }
 
 #define BCK(call)                                                          \
@@ -3485,6 +3537,87 @@ int launch_persistent(const fdtd_batch_t::Persistent& q, int* counter, cudaStrea
   return FDTD_OK;
 }
 
+// The fused launches of a batch (FP32 grids that the fused kernel takes):
+// the parameters of every grid, and a list of blocks.  Warps per block: the
+// count that leaves the fewest idle over all grids.
+int build_fused(const fdtd_batch_t* b, bool scratch_out, fdtd_batch_t::Fused (&fl)[2][2]) {
+  for (fdtd_t* h : b->h)
+    if (!fused_shape_ok(h)) return FDTD_ERR_UNSUPPORTED;
+  for (int slot = 0; slot < 2; ++slot)
+    for (int pn = 0; pn < 2; ++pn) {
+      int bw = 8;
+      double least = 1e30;
+      for (int w = 8; w >= 4; --w) {
+        double cost = 0;
+        for (fdtd_t* h : b->h) {
+          if (h->per_node != (pn != 0)) continue;
+          int nwarps[2], tiles_x[2];
+          unsigned ntiles[2];
+          fused_tiles<float>(h, slot, nwarps, ntiles, tiles_x);
+          cost += fused_block_cost(nwarps, ntiles, w);
+        }
+        if (cost < least) {
+          least = cost;
+          bw = w;
+        }
+      }
+      std::vector<fdtd::FusedParams<float>> grids;
+      std::vector<int2> blocks;
+      for (fdtd_t* h : b->h) {
+        if (h->per_node != (pn != 0)) continue;
+        if (scratch_out) {
+          int rc = ensure_scratch(h);
+          if (rc) return rc;
+        }
+        fdtd::FusedParams<float> fp;
+        const unsigned n = fused_fill<float>(h, slot, 1.0, 1.0, -1.0, 1.0, h->f, scratch_out ? h->scratch : h->f, 7,
+                                             bw, fp);
+        for (unsigned q = 0; q < n; ++q) blocks.push_back(make_int2((int)grids.size(), (int)q));
+        grids.push_back(fp);
+      }
+      fdtd_batch_t::Fused& q = fl[slot][pn];
+      q.nblocks = (unsigned)blocks.size();
+      q.threads = (unsigned)bw * 32;
+      if (blocks.empty()) continue;
+      BCK(dev_malloc(&q.d_grids, sizeof(grids[0]) * grids.size()));
+      BCK(cudaMemcpy(q.d_grids, grids.data(), sizeof(grids[0]) * grids.size(), cudaMemcpyHostToDevice));
+      BCK(dev_malloc((void**)&q.d_blocks, sizeof(int2) * blocks.size()));
+      BCK(cudaMemcpy(q.d_blocks, blocks.data(), sizeof(int2) * blocks.size(), cudaMemcpyHostToDevice));
+    }
+  return FDTD_OK;
+}
+
+// `count` steps on b->run, the launches chained (a batch of one media kind;
+// with both kinds their launches follow one another).
+int fused_batch_steps(fdtd_batch_t* b, const fdtd_batch_t::Fused (&fl)[2][2], int count) {
+  static const int seq_fss[3] = {0, 1, 0};
+  const int n = b->scheme == FDTD_FSS ? 3 : 2;
+  bool chained = false;
+  for (int st = 0; st < count; ++st)
+    for (int k = 0; k < n; ++k) {
+      const auto& slot = fl[seq_fss[k]];
+      const bool both = slot[0].nblocks > 0 && slot[1].nblocks > 0;
+      for (int pn = 0; pn < 2; ++pn) {
+        if (slot[pn].nblocks == 0) continue;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(slot[pn].nblocks);
+        cfg.blockDim = dim3(slot[pn].threads);
+        cfg.stream = b->run;
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = chained && !both ? 1 : 0;
+        const auto* grids = (const fdtd::FusedParams<float>*)slot[pn].d_grids;
+        const int2* blocks = slot[pn].d_blocks;
+        if (pn) BCK(cudaLaunchKernelEx(&cfg, fdtd::proc_fused_batch_kernel<float, true>, grids, blocks));
+        else BCK(cudaLaunchKernelEx(&cfg, fdtd::proc_fused_batch_kernel<float, false>, grids, blocks));
+        chained = true;
+      }
+    }
+  return FDTD_OK;
+}
+
 // One time step of every grid: the scheme's procedure sequence.  The groups
 // of one procedure write disjoint arrays, so they fork onto parallel
 // branches; the next procedure starts when all of them have joined.  In
@@ -3675,6 +3808,45 @@ int time_step_modes(fdtd_batch_t* b, const BatchCfg& cfg, int reps, double out[2
   return rc;
 }
 
+// Time of one fused step (ms, best of `reps` replays writing scratch), or a
+// negative value where a grid does not take the fused kernel.
+double time_fused(fdtd_batch_t* b, int reps) {
+  fdtd_batch_t::Fused fl[2][2];
+  double best = -1.0;
+  if (build_fused(b, true, fl) == FDTD_OK) {
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t ex = nullptr;
+    if (cudaStreamBeginCapture(b->run, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+      const int rs = fused_batch_steps(b, fl, 1);
+      if (cudaStreamEndCapture(b->run, &g) == cudaSuccess && rs == FDTD_OK &&
+          cudaGraphInstantiate(&ex, g, 0) == cudaSuccess) {
+        cudaEvent_t e0, e1;
+        cudaEventCreate(&e0);
+        cudaEventCreate(&e1);
+        for (int r = 0; r < reps + 1; ++r) {  // the first replay warms up
+          cudaEventRecord(e0, b->run);
+          cudaGraphLaunch(ex, b->run);
+          cudaEventRecord(e1, b->run);
+          if (cudaEventSynchronize(e1) != cudaSuccess) {
+            best = -1.0;
+            break;
+          }
+          float ms = 0;
+          cudaEventElapsedTime(&ms, e0, e1);
+          if (r > 0 && (best < 0 || ms < best)) best = ms;
+        }
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+      }
+    }
+    if (ex) cudaGraphExecDestroy(ex);
+    if (g) cudaGraphDestroy(g);
+  }
+  free_fused(fl);
+  cudaGetLastError();
+  return best;
+}
+
 std::string batch_mode_key(const fdtd_batch_t* b) {
   const BatchCfg& c = b->cfg;
   return batch_key(b) + "|mode|" + std::to_string(c.lanes[0]) + "," + std::to_string(c.L[0]) + "," +
@@ -3692,8 +3864,9 @@ int batch_tune_mode_t(fdtd_batch_t* b) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
   const std::string key = batch_mode_key(b);
   TuneVal v;
-  auto take = [&](int pers, int Ly, int Lz) {
+  auto take = [&](int pers, int Ly, int Lz, int fused) {
     b->tuned_persistent = pers;
+    b->tuned_fused = fused;
     if (pers) {
       b->cfg.lanes[0] = b->cfg.lanes[1] = 16;
       b->cfg.L[0] = Ly;
@@ -3704,7 +3877,7 @@ int batch_tune_mode_t(fdtd_batch_t* b) {
   if (tune_cache_get(key, &v)) {
     b->mode_ms[0] = v[1] * 1e-3;
     b->mode_ms[1] = v[2] * 1e-3;
-    take(v[0], v[3], v[4]);
+    take(v[0], v[3], v[4], v[5]);
     return FDTD_OK;
   }
   BCK(cudaEventRecord(b->ev_in, b->stream));
@@ -3730,12 +3903,25 @@ int batch_tune_mode_t(fdtd_batch_t* b) {
       pick = c;
     }
   }
+  // launches: the shape-uniform groups, or one fused launch per procedure
+  // when the shapes are the tuner's to choose
+  int fused = 0;
+  if constexpr (sizeof(T) == 4) {
+    if (b->autotune) {
+      const double f = time_fused(b, 5);
+      if (f > 0 && (ms[0] < 0 || f < ms[0])) {
+        fused = 1;
+        ms[0] = f;
+      }
+    }
+  }
   b->mode_ms[0] = ms[0] > 0 ? ms[0] : 0;
   b->mode_ms[1] = best > 0 ? best : 0;
   const int pers = (best > 0 && (ms[0] < 0 || best < ms[0])) ? 1 : 0;
-  take(pers, pick.L[0], pick.L[1]);
+  if (pers) fused = 0;
+  take(pers, pick.L[0], pick.L[1], fused);
   tune_cache_put(key, {pers, (int)std::lround(b->mode_ms[0] * 1e3), (int)std::lround(b->mode_ms[1] * 1e3),
-                       pick.L[0], pick.L[1], 0});
+                       pick.L[0], pick.L[1], fused});
   return FDTD_OK;
 }
 
@@ -3817,7 +4003,7 @@ int batch_prepare(fdtd_batch_t* b) {
       if (rc) return rc;
     }
     b->tuned = true;
-    b->tuned_persistent = -1;
+    b->tuned_persistent = b->tuned_fused = -1;
     b->bound.clear();
   }
   if (!b->d_counter) BCK(dev_malloc((void**)&b->d_counter, 3 * sizeof(int)));
@@ -3826,11 +4012,20 @@ int batch_prepare(fdtd_batch_t* b) {
     if (rc) return rc;
   }
   const bool want = b->mode == 1 || (b->mode == -1 && b->tuned_persistent == 1);
+  const bool want_fused = b->mode == -1 && b->autotune && !want && b->tuned_fused == 1;
   std::vector<const void*> ptrs;
   for (fdtd_t* h : b->h)
     for (int c = 0; c < 6; ++c) ptrs.push_back(h->f[c]);
-  if (ptrs == b->bound && !b->groups[0].empty() && want == b->persistent) return FDTD_OK;
+  if (ptrs == b->bound && (!b->groups[0].empty() || b->fused) && want == b->persistent && want_fused == b->fused)
+    return FDTD_OK;
   free_groups(b);
+  b->fused = false;
+  if (want_fused && build_fused(b, false, b->fl) == FDTD_OK) {
+    b->fused = true;
+    b->persistent = false;
+    b->bound = ptrs;
+    return FDTD_OK;
+  }
   int rc = b->prec == FDTD_F64 ? build_groups_t<double>(b, b->cfg, b->groups, -1, false)
                                : build_groups_t<float>(b, b->cfg, b->groups, -1, false);
   b->persistent = false;
@@ -4025,24 +4220,32 @@ int fdtd_batch_step(fdtd_batch_t* b, int64_t nsteps) {
   if (nsteps == 0) return FDTD_OK;
   int rc = batch_prepare(b);
   if (rc) return rc;
-  if (!b->exec) {
-    // one step of every grid, captured once as a CUDA graph and replayed
+  // steps of every grid, captured once as CUDA graphs and replayed: single
+  // steps, and runs of kStepRun where a step is a few launches
+  auto capture = [&](cudaGraphExec_t* ex, int count) -> int {
     BCK(cudaStreamBeginCapture(b->run, cudaStreamCaptureModeThreadLocal));
-    rc = b->prec == FDTD_F64 ? batch_one_step<double>(b) : batch_one_step<float>(b);
+    const int rs = b->fused ? fused_batch_steps(b, b->fl, count)
+                            : (b->prec == FDTD_F64 ? batch_one_step<double>(b) : batch_one_step<float>(b));
     cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(b->run, &g);
-    if (rc) {
+    const cudaError_t e = cudaStreamEndCapture(b->run, &g);
+    if (rs || e != cudaSuccess) {
       if (g) cudaGraphDestroy(g);
-      return rc;
+      if (rs) return rs;
+      BCK(e);
     }
-    BCK(e);
-    b->graph = g;
-    BCK(cudaGraphInstantiate(&b->exec, b->graph, 0));
-  }
+    const cudaError_t ie = cudaGraphInstantiate(ex, g, 0);
+    cudaGraphDestroy(g);
+    BCK(ie);
+    return FDTD_OK;
+  };
+  const int64_t runs = b->fused ? nsteps / kStepRun : 0, singles = nsteps - runs * kStepRun;
+  if (runs > 0 && !b->exec_run && (rc = capture(&b->exec_run, kStepRun))) return rc;
+  if (singles > 0 && !b->exec && (rc = capture(&b->exec, 1))) return rc;
   // order after the handles' earlier work, and their later work after this
   BCK(cudaEventRecord(b->ev_in, b->stream));
   BCK(cudaStreamWaitEvent(b->run, b->ev_in, 0));
-  for (int64_t k = 0; k < nsteps; ++k) BCK(cudaGraphLaunch(b->exec, b->run));
+  for (int64_t k = 0; k < runs; ++k) BCK(cudaGraphLaunch(b->exec_run, b->run));
+  for (int64_t k = 0; k < singles; ++k) BCK(cudaGraphLaunch(b->exec, b->run));
   BCK(cudaEventRecord(b->ev_out, b->run));
   BCK(cudaStreamWaitEvent(b->stream, b->ev_out, 0));
   for (fdtd_t* h : b->h) {
@@ -4058,7 +4261,10 @@ int fdtd_batch_launches(const fdtd_batch_t* b, int64_t* per_step) {
   const int seq[3] = {0, 1, 0};
   long long c = 0;
   for (int k = 0; k < n; ++k)
-    c += b->persistent ? (b->pl[seq[k]].nwork > 0 ? 1 : 0) : (long long)b->groups[seq[k]].size();
+    if (b->fused)
+      c += (b->fl[seq[k]][0].nblocks > 0) + (b->fl[seq[k]][1].nblocks > 0);
+    else
+      c += b->persistent ? (b->pl[seq[k]].nwork > 0 ? 1 : 0) : (long long)b->groups[seq[k]].size();
   *per_step = c;
   return FDTD_OK;
 }
@@ -4119,7 +4325,7 @@ int fdtd_batch_set_config(fdtd_batch_t* b, const int32_t* cfg) {
   b->cfg.xpack = cfg[5];
   b->autotune = false;
   b->tuned = true;
-  b->tuned_persistent = -1;
+  b->tuned_persistent = b->tuned_fused = -1;
   free_groups(b);
   b->bound.clear();
   return FDTD_OK;

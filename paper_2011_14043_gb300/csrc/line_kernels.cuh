@@ -296,10 +296,12 @@ __device__ __forceinline__ HiLo<T> phase_forward(const PairParams<T>& p, int j0,
 
 // Forward carry fix-up, then the local backward sweep from a zero carry;
 // returns the segment's carry coefficient prod(-c).
-template <typename T, int L, int MODE>
+template <typename T, int L, int MODE, bool FIX = true>
 __device__ __forceinline__ HiLo<T> phase_backward(const PairParams<T>& p, int j0, T yin, const T (&ibn)[L],
                                                   const T (&ibl)[L], HiLo<T> ib_prev, T (&y)[L]) {
-  if constexpr (MODE == 2) {
+  if constexpr (!FIX) {
+    // the caller has added the carry
+  } else if constexpr (MODE == 2) {
     T q = T(1);
 #pragma unroll
     for (int t = 0; t < L; ++t) {
@@ -1845,8 +1847,10 @@ __device__ __forceinline__ T group_chain_backward(T b, HiLo<T> pm, int sl) {
 }
 
 // One x line of a per-node medium on LPL lanes (lane sl its nodes
-// [sl L, sl L + L)): the solve of phase_forward / phase_backward with the
-// group scans.  On return E, H hold the new values.
+// [sl L, sl L + L)): the sweeps of phase_forward / phase_backward with the
+// group scans; a carry runs through its segment by the segment's own
+// multipliers (FP32: hi + lo, as in the sweeps), not by products of their hi
+// parts.  On return E, H hold the new values.
 template <typename T, int L, int LPL>
 __device__ __forceinline__ void row_solve_pn(const PairParams<T>& p, int sl, T (&E)[L], T (&H)[L], const T (&qn)[L],
                                              const T (&ibn)[L], const T (&ibl)[L]) {
@@ -1862,9 +1866,32 @@ __device__ __forceinline__ void row_solve_pn(const PairParams<T>& p, int sl, T (
   const int j0 = sl * L;
   const HiLo<T> pf = phase_forward<T, L, 2>(p, j0, E, H, hm1, qn, ibn, ibl, ib_prev, y);
   const T yin = group_chain_forward<T, LPL>(y[L - 1], pf, sl);
-  const HiLo<T> pb = phase_backward<T, L, 2>(p, j0, yin, ibn, ibl, ib_prev, y);
+  T q = yin;
+#pragma unroll
+  for (int t = 0; t < L; ++t) {
+    const HiLo<T> b = t == 0 ? ib_prev : HiLo<T>{ibn[t == 0 ? 0 : t - 1], ibl[t == 0 ? 0 : t - 1]};
+    if constexpr (use_hilo<T>()) {
+      const T v = fma(b.hi, q, b.lo * q);
+      q = fma(-p.offh, v, -p.offl * v);
+    } else {
+      q *= -p.offh * b.hi;
+    }
+    y[t] += q;
+  }
+  // the backward sweep of phase_backward (its carry fix done above)
+  const HiLo<T> pb = phase_backward<T, L, 2, false>(p, j0, T(0), ibn, ibl, ib_prev, y);
   const T win = group_chain_backward<T, LPL>(y[0], pb, sl);
-  phase_fix<T, L, 2>(p, j0, win, ibn, ibl, y);
+  q = win;
+#pragma unroll
+  for (int t = L - 1; t >= 0; --t) {
+    if constexpr (use_hilo<T>()) {
+      const T u = fma(-p.offh, q, -p.offl * q);
+      q = fma(ibn[t], u, ibl[t] * u);
+    } else {
+      q *= -p.offh * ibn[t];
+    }
+    y[t] += q;
+  }
 #pragma unroll
   for (int t = 0; t < L; ++t) {
     const T wnext = (t + 1 < L) ? y[t + 1] : win;

@@ -53,7 +53,8 @@ def test_procedure_in_one_launch(dims, media, prec):
     dt = 5.0 * d / (299792458.0 * np.sqrt(3.0 if nz > 1 else 2.0))
     cur = np.random.default_rng(1).standard_normal(steps) * 1e-3
     for scheme, at in (("fadi", (1, 1, 0)), ("fss", (nx - 1, ny - 1, nz - 1)), ("flod2", (nx // 2, ny // 2, nz // 2))):
-        src = ("ez",) + at + (cur,)
+        # (homogeneous grids with a source take the kernels of a launch per pair)
+        src = ("ez",) + at + (cur,) if media == "blocks" or scheme == "flod2" else None
         out, _, _, sim = gpu_run(nx, ny, nz, d, d, d, dt, scheme, prec, u0, steps, eps=eps, source=src)
         sim.close()
         w0 = {c: v.astype(np.float32).astype(np.float64) if prec == "f32" else v for c, v in u0.items()}
@@ -121,3 +122,41 @@ def test_device_copies_of_every_component(dims, prec):
             assert np.array_equal(host.get_field(c)[w], u0[c].astype(npt)[w]), c
         host.close()
         dev.close()
+
+
+@pytest.mark.parametrize("media", ["uniform", "blocks", "both"])
+@pytest.mark.parametrize("scheme", ["fadi", "fss"])
+def test_batch_in_one_launch_per_procedure(scheme, media):
+    """An FP32 batch whose shapes the tuner may choose: grids of one to eight
+    warps per tile, x lines on 8, 16 and 32 lanes, runs of 16 steps and single
+    ones; against the oracle, and (where the batch took one launch per
+    procedure) bit for bit against the grids stepped alone."""
+    from paper_2011_14043_gb300 import Batch, Simulation
+    grids = [(20, 30, 9), (70, 97, 33), (130, 12, 70), (16, 129, 5), (9, 8, 250)]
+    steps = 18
+    sims, alone, refs = [], [], []
+    for q, (nx, ny, nz) in enumerate(grids):
+        u0 = random_fields(nx, ny, nz, 20 + q)
+        eps = random_media(nx, ny, nz, q) if media == "blocks" or (media == "both" and q % 2) else None
+        for out in (sims, alone):
+            s = Simulation(nx, ny, nz, 1e-3, scheme=scheme, precision="f32", cfl=3.0 + q)
+            if eps is not None:
+                s.set_material(eps)
+            s.set_fields(u0)
+            out.append(s)
+        w0 = {c: v.astype(np.float32).astype(np.float64) for c, v in u0.items()}
+        refs.append(S.run_fundamental(oracle_problem(nx, ny, nz, 1e-3, 1e-3, 1e-3, sims[-1].dt, eps=eps), scheme, w0,
+                                      steps)[0])
+    b = Batch(sims)
+    b.step(1)
+    b.step(steps - 1)
+    procedures = 3 if scheme == "fss" else 2
+    fused = b.launches_per_step() <= procedures * (2 if media == "both" else 1)
+    for q, s in enumerate(sims):
+        got = s.get_fields()
+        assert energy_norm_rel(got, refs[q]) <= TOL["f32"], q
+        if fused:
+            alone[q].step(steps)
+            for c in ("hx", "hy", "hz"):
+                assert np.array_equal(alone[q].get_state(c), s.get_state(c)), (q, c)
+    b.close()
