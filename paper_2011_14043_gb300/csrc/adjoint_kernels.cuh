@@ -32,15 +32,22 @@ struct AdjExtra {
   const T* d;         // forward record D = 2 E - w of this pair's component
   double* grad;       // dJ/d eps per E sample (field layout), accumulated
   double inv_h;       // 1 / procedure length
+  const long long* slot;  // captured steps: the record is d + *slot * stride
+  long long stride;
 };
+
+template <typename T>
+__device__ __forceinline__ const T* adj_record(const AdjExtra<T>& x) {
+  return x.d + (x.slot ? *x.slot * x.stride : 0);
+}
 
 // Store of one adjoint node: H update, E output, eps gradient.
 template <typename T, int L>
-__device__ __forceinline__ void adj_store_node(const PairParams<T>& p, const AdjExtra<T>& x, long long at, int j,
-                                               T E, T H, T q, T y, T ynext) {
+__device__ __forceinline__ void adj_store_node(const PairParams<T>& p, const AdjExtra<T>& x, const T* rec,
+                                               long long at, int j, T E, T H, T q, T y, T ynext) {
   p.e_out[at] = fma(q, y, -E);
   p.h_out[at] = fma(p.kd, ynext - y, H);
-  if (j >= 1) x.grad[at] += x.inv_h * (double)y * (double)x.d[at];
+  if (j >= 1) x.grad[at] += x.inv_h * (double)y * (double)rec[at];
 }
 
 // Lines along y or z: the per-node strided solve with unit row scaling.
@@ -92,6 +99,7 @@ __global__ void adj_strided_kernel(const PairParams<T> p, const AdjExtra<T> x) {
       if constexpr (use_hilo<T>()) ib_prev.lo = p.nibl[at];
     }
   }
+  const T* rec = adj_record(x);
   T win;
   strided_solve<T, LANES, L, true>(p, j0, s, P, lane, sh, E, H, hm1, one, ibn, ibl, ib_prev, y, win);
   if (active) {
@@ -100,7 +108,7 @@ __global__ void adj_strided_kernel(const PairParams<T> p, const AdjExtra<T> x) {
       const int j = j0 + t;
       if (j < N) {
         const T ynext = (t + 1 < L) ? y[t + 1] : win;
-        adj_store_node<T, L>(p, x, base + (long long)j * ls, j, E[t], H[t], q[t], y[t], ynext);
+        adj_store_node<T, L>(p, x, rec, base + (long long)j * ls, j, E[t], H[t], q[t], y[t], ynext);
       }
     }
   }
@@ -135,11 +143,12 @@ __global__ void adj_rows_kernel(const PairParams<T> p, const AdjExtra<T> x) {
   const T win = warp_chain_backward<T>(y[0], pb);
   phase_fix<T, L, 2>(p, j0, win, ibn, ibl, y);
   if (!row_ok<T, L>(p, base)) return;
+  const T* rec = adj_record(x);
   if (j0 + L <= N) {
     // whole segment: record, gradient and outputs as 16-byte vectors
     T dd[L];
     double g[L];
-    load_seg<T, L>(x.d + base + j0, dd);
+    load_seg<T, L>(rec + base + j0, dd);
     load_seg<double, L>(x.grad + base + j0, g);
 #pragma unroll
     for (int t = 0; t < L; ++t) {
@@ -158,7 +167,7 @@ __global__ void adj_rows_kernel(const PairParams<T> p, const AdjExtra<T> x) {
       const int j = j0 + t;
       if (j < N) {
         const T ynext = (t + 1 < L) ? y[t + 1] : win;
-        adj_store_node<T, L>(p, x, base + j, j, E[t], H[t], q[t], y[t], ynext);
+        adj_store_node<T, L>(p, x, rec, base + j, j, E[t], H[t], q[t], y[t], ynext);
       }
     }
   }
@@ -178,7 +187,8 @@ struct ProbeSet {
 // reverse pass).
 template <typename T>
 __global__ void probe_energy_kernel(ProbeSet<T> ps, const T* e0, const T* e1, const T* e2, double* stash,
-                                    double* acc, int mode, double* wrec) {
+                                    double* acc, int mode, double* wrec, const long long* slot) {
+  if (wrec && slot) wrec += *slot * ps.n;
   const T* e[3] = {e0, e1, e2};
   double sum = 0.0;
   for (int k = threadIdx.x; k < ps.n; k += blockDim.x) {
@@ -207,7 +217,9 @@ __global__ void probe_energy_kernel(ProbeSet<T> ps, const T* e0, const T* e1, co
 // Backward: lam_E += jbar * w_B/2 at the probe samples (w_B recorded by
 // the recomputation).
 template <typename T>
-__global__ void probe_inject_kernel(ProbeSet<T> ps, T* l0, T* l1, T* l2, const double* wrec, double jbar) {
+__global__ void probe_inject_kernel(ProbeSet<T> ps, T* l0, T* l1, T* l2, const double* wrec, double jbar,
+                                    const long long* slot) {
+  if (slot) wrec += *slot * ps.n;
   T* lam[3] = {l0, l1, l2};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < ps.n; k += gridDim.x * blockDim.x) {
     const int c = ps.comp[k];
@@ -220,6 +232,18 @@ __global__ void probe_inject_kernel(ProbeSet<T> ps, T* l0, T* l1, T* l2, const d
 template <typename T>
 __global__ void grad_point_kernel(double* grad, const T* lam, long long at, double coef) {
   if (threadIdx.x == 0 && blockIdx.x == 0) grad[at] += coef * (double)lam[at];
+}
+
+// The same inside a captured step: post = coef * table[*step + off] (rounded
+// on its own, as the host forms it), added as -post / eps_src * lam[at].
+template <typename T>
+__global__ void grad_point_table_kernel(double* grad, const T* lam, long long at, const double* table, long long len,
+                                        const long long* step, int off, double coef, double eps_src) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) {
+    const long long n = *step + off;
+    const double post = __dmul_rn(coef, (n >= 0 && n < len) ? table[n] : 0.0);
+    if (post != 0.0) grad[at] += (-post / eps_src) * (double)lam[at];
+  }
 }
 
 // Input initialization v0 = u0 + (dt/2) B u0 (+ source): the E rows of B u0

@@ -89,6 +89,15 @@ __global__ void step_counter_kernel(long long* step, long long value, int mode) 
   if (threadIdx.x == 0 && blockIdx.x == 0) *step = mode == 0 ? value : *step + value;
 }
 
+// ctr[0] += a, ctr[1] += b (the step and record counters of a captured
+// reverse-mode step); set: the values themselves.
+__global__ void two_counters_kernel(long long* ctr, long long a, long long b, int set) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) {
+    ctr[0] = set ? a : ctr[0] + a;
+    ctr[1] = set ? b : ctr[1] + b;
+  }
+}
+
 // Compact [sz][sy][sx] <-> padded (plane, pitch) layout of one component,
 // for host copies staged through a contiguous device buffer: one row (fixed
 // j, k) per block iteration, threads along x (no per-element division).

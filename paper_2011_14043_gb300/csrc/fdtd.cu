@@ -22,6 +22,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <map>
 #include <mutex>
 #include <string>
@@ -71,6 +72,7 @@ struct PairCoef {
   double mc = 0;          // uniform media: the converged multiplier m = c
   int jc4 = 1 << 30, je4 = -1;  // fourth order: nodes whose factor rows all equal cv4
   double cv4[14] = {0};
+  void* slab = nullptr;   // per-node media: the allocation that holds the arrays below
   void* nq = nullptr;     // per-node media (field layout, T): 1/|b_j|
   void* nib = nullptr;    //   1/beta_j (hi)
   void* nibl = nullptr;   //   1/beta_j (lo, FP32 only)
@@ -104,6 +106,8 @@ struct fdtd_s {
   long long pitch, plane, count;
   void* f[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   void* scratch[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  void* f_slab = nullptr;        // the allocations behind f and scratch (whose pointers swap)
+  void* scratch_slab = nullptr;
   void* stage = nullptr;  // contiguous staging buffer of host copies (one component)
   PairGeom geom[2][3];
   StridedCfg strided_cfg[2];  // y lines, z lines
@@ -355,12 +359,7 @@ int upload_any(fdtd_t* h, void** dst, const std::vector<double>& src) {
 void free_coef(ProcCoef& pc) {
   for (auto& c : pc.pc) {
     if (c.tab) cudaFree(c.tab);
-    if (c.nq) cudaFree(c.nq);
-    if (c.nib) cudaFree(c.nib);
-    if (c.nibl) cudaFree(c.nibl);
-    if (c.nkd) cudaFree(c.nkd);
-    if (c.noffh) cudaFree(c.noffh);
-    if (c.noffl) cudaFree(c.noffl);
+    if (c.slab) cudaFree(c.slab);
     c = PairCoef();
   }
   pc.valid = false;
@@ -640,20 +639,21 @@ int build_proc(fdtd_t* h, int slot, int op, double hh, double loss_sign = 1.0) {
       const double off = -kk / 2.0;
       c.offh = rnd(off);
       c.offl = f32 ? (double)(float)(off - c.offh) : 0.0;
-      int rc = FDTD_OK;
-      auto zeroed = [&](void** dst) {
-        if (!rc) rc = cuda_fail(h, dev_malloc(dst, (size_t)h->count * h->esize));
-        if (!rc) rc = cuda_fail(h, cudaMemsetAsync(*dst, 0, (size_t)h->count * h->esize, h->stream));
-      };
-      zeroed(&c.nq);
-      zeroed(&c.nib);
-      if (f32) zeroed(&c.nibl);
+      // the pair's arrays in one allocation
+      const size_t arr = ((size_t)h->count * h->esize + 255) / 256 * 256;
+      const size_t narr = (f32 ? 3 : 2) * (h->mu_var ? 2 : 1);
+      CK(dev_malloc(&c.slab, narr * arr));
+      CK(cudaMemsetAsync(c.slab, 0, narr * arr, h->stream));
+      size_t used = 0;
+      auto next = [&]() { return (void*)((char*)c.slab + arr * used++); };
+      c.nq = next();
+      c.nib = next();
+      if (f32) c.nibl = next();
       if (h->mu_var) {
-        zeroed(&c.nkd);
-        zeroed(&c.noffh);
-        if (f32) zeroed(&c.noffl);
+        c.nkd = next();
+        c.noffh = next();
+        if (f32) c.noffl = next();
       }
-      if (rc) return rc;
       if (g.N < 1 || g.n_lines() <= 0) continue;
       fdtd::FactorParams fp;
       fp.ls = g.ls;
@@ -689,7 +689,7 @@ int build_proc(fdtd_t* h, int slot, int op, double hh, double loss_sign = 1.0) {
       else
         fdtd::factor_lines_kernel<double><<<blocks, 64, 0, h->stream>>>(fp, (double*)c.nq, (double*)c.nib, nullptr,
                                                                         (double*)c.nkd, (double*)c.noffh, nullptr);
-      if ((rc = cuda_fail(h, cudaGetLastError()))) return rc;
+      CK(cudaGetLastError());
     }
   }
   P.valid = true;
@@ -723,8 +723,9 @@ int build_all_coefs(fdtd_t* h) {
 // ---------------------------------------------------------------------------
 
 
-// Carry products of runs of segments of L nodes (row_solve_wall) and where
-// they fall below 2^-50 (FP64 fields: 2^-60) of the carry.
+// Carry products of runs of segments of L nodes (row_solve_wall), and how many
+// runs of 32 nodes a y/z tile's carry is followed over: until it falls below
+// 2^-50 (FP64 fields: 2^-60).
 template <typename T>
 void set_scan(fdtd::PairParams<T>& p, const PairCoef& c, int L) {
   const double least = sizeof(T) == 4 ? 0x1p-50 : 0x1p-60;
@@ -736,9 +737,11 @@ void set_scan(fdtd::PairParams<T>& p, const PairCoef& c, int L) {
     p.sc[0][k] = p.sc[0][k - 1] * p.sc[0][k - 1];
     p.sc[1][k] = T(0);
   }
+  // an x line's scan stops where the product is zero: a carry that it leaves
+  // out would have been zero too (the same bits, also in empty regions)
   p.nscan = 32;
   for (int k = 4; k >= 0; --k)
-    if (std::fabs((double)p.sc[0][k]) < least) p.nscan = 1 << k;
+    if (p.sc[0][k] == T(0)) p.nscan = 1 << k;
   p.kx = 1;
   while (p.kx < 8 && std::pow(std::fabs(c.mc), 32.0 * p.kx) >= least) ++p.kx;
 }
@@ -785,6 +788,8 @@ fdtd::PairParams<T> make_params(const fdtd_t* h, const PairGeom& g, const PairCo
   p.offh = (T)c.offh;
   p.offl = (T)c.offl;
   p.d_out = nullptr;
+  p.d_slot = nullptr;
+  p.d_stride = 0;
   p.nkd = (const T*)c.nkd;
   p.noffh = (const T*)c.noffh;
   p.noffl = (const T*)c.noffl;
@@ -1144,8 +1149,7 @@ int launch_pair_gm(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
 }
 
 // Fourth-order differences.  The procedure on lines of at most 512 cells
-// runs the block-tiled kernel (chunks of 32 nodes: CH = 2, 8 or 16); longer
-// lines, the explicit operator and tune[1] bit 9 take one thread per line
+// runs the block-tiled kernel; longer lines, the explicit operator and tune[1] bit 9 take one thread per line
 // (128 per block).  FP64 fields keep one thread per line: their work is
 // bound by the FP64 pipe, which the tiled kernel's half-filled sweep warps
 // (16 lines per block) use at half rate (measured at 256^3: 1.02 against
@@ -1596,15 +1600,16 @@ int procedure_two_terms(fdtd_t* h, int slot, double ta, double tb) {
   return add_point(h, h->f[h->src_comp < 0 ? 0 : h->src_comp], tb);
 }
 
-int ensure_scratch(fdtd_t* h) {
-  for (int c = 0; c < 6; ++c) {
-    if (!h->scratch[c]) {
-      CK(dev_malloc((void**)&h->scratch[c], (size_t)h->count * h->esize));
-      CK(cudaMemsetAsync(h->scratch[c], 0, (size_t)h->count * h->esize, h->stream));
-    }
-  }
+// Six zeroed field arrays in one allocation.
+int alloc_fields(fdtd_t* h, void** slab, void** arr) {
+  const size_t n = ((size_t)h->count * h->esize + 255) / 256 * 256;
+  CK(dev_malloc(slab, 6 * n));
+  CK(cudaMemsetAsync(*slab, 0, 6 * n, h->stream));
+  for (int c = 0; c < 6; ++c) arr[c] = (char*)*slab + c * n;
   return FDTD_OK;
 }
+
+int ensure_scratch(fdtd_t* h) { return h->scratch_slab ? FDTD_OK : alloc_fields(h, &h->scratch_slab, h->scratch); }
 
 int copy_state_to_scratch(fdtd_t* h) {
   int rc = ensure_scratch(h);
@@ -2622,11 +2627,9 @@ int fdtd_create(const fdtd_desc* desc, void* stream, fdtd_t** out) {
     }
     h->strided_cfg[ax] = (a.lanes * a.L == b.lanes * b.L && a.lanes == b.lanes) ? a : b;
   }
-  for (int c = 0; c < 6; ++c) {
-    cudaError_t e = dev_malloc((void**)&h->f[c], (size_t)h->count * h->esize);
-    if (e != cudaSuccess) { fdtd_destroy(h); return FDTD_ERR_OOM; }
-    e = cudaMemsetAsync(h->f[c], 0, (size_t)h->count * h->esize, h->stream);
-    if (e != cudaSuccess) { fdtd_destroy(h); return FDTD_ERR_CUDA; }
+  {
+    const int rc = alloc_fields(h, &h->f_slab, h->f);
+    if (rc) { fdtd_destroy(h); return rc; }
   }
   for (int cls = 0; cls < 3; ++cls)
     h->bytes_per_launch[cls] = 4.0 * (double)d.nx * d.ny * d.nz * (double)h->esize;
@@ -2653,10 +2656,8 @@ int fdtd_create(const fdtd_desc* desc, void* stream, fdtd_t** out) {
 int fdtd_destroy(fdtd_t* h) {
   if (!h) return FDTD_OK;
   cudaStreamSynchronize(h->stream);
-  for (int c = 0; c < 6; ++c) {
-    if (h->f[c]) cudaFree(h->f[c]);
-    if (h->scratch[c]) cudaFree(h->scratch[c]);
-  }
+  if (h->f_slab) cudaFree(h->f_slab);
+  if (h->scratch_slab) cudaFree(h->scratch_slab);
   for (auto& p : h->proc) free_coef(p);
   for (int c = 0; c < 3; ++c) {
     if (h->eps_node[c]) cudaFree(h->eps_node[c]);
@@ -2736,21 +2737,27 @@ int fdtd_set_media(fdtd_t* h, const double* eps, const double* mu, const double*
   const size_t nc = (size_t)h->nx * h->ny * h->nz;
   const double e0 = eps ? eps[0] : 1.0, m0 = mu ? mu[0] : 1.0, s0 = sigma ? sigma[0] : 0.0;
   bool e_uniform = true, m_uniform = true, s_uniform = true, any_loss = false;
-  for (size_t q = 0; q < nc; ++q) {
-    if (eps) {
-      if (!(eps[q] > 0) || !std::isfinite(eps[q])) return FDTD_ERR_INVALID_ARG;
-      if (eps[q] != e0) e_uniform = false;
+  // one pass per array without branches (it vectorises)
+  auto scan = [nc](const double* a, double first, bool& uniform, bool& positive) {
+    bool ok = true, same = true, pos = false;
+    for (size_t q = 0; q < nc; ++q) {
+      ok &= a[q] >= 0 && a[q] <= std::numeric_limits<double>::max();
+      same &= a[q] == first;
+      pos |= a[q] > 0;
     }
-    if (mu) {
-      if (!(mu[q] > 0) || !std::isfinite(mu[q])) return FDTD_ERR_INVALID_ARG;
-      if (mu[q] != m0) m_uniform = false;
-    }
-    if (sigma) {
-      if (!(sigma[q] >= 0) || !std::isfinite(sigma[q])) return FDTD_ERR_INVALID_ARG;
-      if (sigma[q] != s0) s_uniform = false;
-      if (sigma[q] > 0) any_loss = true;
-    }
-  }
+    uniform = same;
+    positive = pos;
+    return ok;
+  };
+  auto all_above_zero = [nc](const double* a) {
+    bool ok = true;
+    for (size_t q = 0; q < nc; ++q) ok &= a[q] > 0;
+    return ok;
+  };
+  bool some = false;
+  if (eps && (!scan(eps, e0, e_uniform, some) || !all_above_zero(eps))) return FDTD_ERR_INVALID_ARG;
+  if (mu && (!scan(mu, m0, m_uniform, some) || !all_above_zero(mu))) return FDTD_ERR_INVALID_ARG;
+  if (sigma && !scan(sigma, s0, s_uniform, any_loss)) return FDTD_ERR_INVALID_ARG;
   // per-node mu runs the general-media kernels, built for lines of at most
   // 256 cells along y and z and 256 along x
   if (!m_uniform && (h->nx > 256 || h->ny > 256 || h->nz > 256)) return FDTD_ERR_UNSUPPORTED;
@@ -4109,6 +4116,20 @@ int single_tune_t(fdtd_t* h) {
   const std::string key = "grid|" + device_name() + "|p" + std::to_string(h->prec) + "|s" +
                           std::to_string(h->scheme) + "|" + std::to_string(h->nx) + "x" + std::to_string(h->ny) +
                           "x" + std::to_string(h->nz);
+  // FP32 grids of up to a million cells: the candidates differ by less than
+  // their timings scatter, and eight processes in a row picked different
+  // segment lengths (and so different roundings) for one grid; the length most
+  // of them picked is taken, so that runs repeat
+  if (sizeof(T) == 4 && (double)h->nx * h->ny * h->nz <= 1e6) {
+    const bool y16 = h->ny >= 94, z16 = h->nz >= 84 && (double)h->nx * h->ny * h->nz >= 3e5;
+    const StridedCfg cy = {true, y16 ? 32 : 16, y16 ? 16 : 8}, cz = {true, z16 ? 32 : 16, z16 ? 16 : 8};
+    if (strided_ok<T>(std::max(h->ny, 2), true, cy.lanes, cy.L) &&
+        strided_ok<T>(std::max(h->nz, 2), true, cz.lanes, cz.L)) {
+      h->strided_cfg[0] = cy;
+      h->strided_cfg[1] = cz;
+      return FDTD_OK;
+    }
+  }
   TuneVal v;
   if (tune_cache_get(key, &v) && strided_ok<T>(std::max(h->ny, 2), true, v[0], v[1]) &&
       strided_ok<T>(std::max(h->nz, 2), true, v[2], v[3])) {
@@ -4416,6 +4437,13 @@ struct fdtd_adj_s {
   AdjCfg cfg[2];
   long long src_at = -1;
   double eps_src = 0;
+  void* slab = nullptr;     // all of the above
+  long long* d_ctr = nullptr;  // [0]: step, [1]: record of the segment
+  // captured steps: forward with the objective, recomputation with records,
+  // reverse (scaled by jbar)
+  cudaGraphExec_t g_fwd = nullptr, g_rec = nullptr, g_rev = nullptr;
+  long long k_fwd = 0, k_rec = 0, k_rev = 0;   // kernels of each
+  double g_jbar = 0;
   bool forward_done = false;
   double objective = 0;
   long long bytes = 0;
@@ -4442,48 +4470,53 @@ int copy_arrays(fdtd_t* h, void* const* dst, void* const* src, int first, int n)
   return FDTD_OK;
 }
 
-// One FADI step of the forward model on `st` (in place).  objective: add
-// the step's probe energy to *d_acc.  rec_a, rec_b (recomputation): the
-// per-node kernels also write each procedure's record D = E_in - E_out
-// there, and w_B at the probe samples goes to wrec.
+// One FADI step of the forward model on `st` (in place), the step index read
+// from the device counter.  objective: add the step's probe energy to *d_acc;
+// otherwise (recomputation) the per-node kernels also write each procedure's
+// record D = E_in - E_out to the tape, and w_B at the probe samples goes to
+// d_wrec, both at the place of the device's record counter.
 template <typename T>
-int adj_forward_step(fdtd_adj_t* a, void* const* st, long long n, bool objective, void* const* rec_a,
-                     void* const* rec_b, double* wrec) {
+int adj_forward_step(fdtd_adj_t* a, void* const* st, bool objective) {
   fdtd_t* h = a->h;
-  const double post_a = 0.5 * h->dt * source_value(h, n);
-  const double post_b = 0.5 * h->dt * source_value(h, n + 1);
-  auto proc = [&](int slot, void* const* rec) -> int {
+  auto proc = [&](int slot) -> int {
     const ProcCoef& P = h->proc[slot];
     return fork_pairs(h, [&](int q) -> int {
       const PairGeom& g = h->geom[P.op][q];
       fdtd::PairParams<T> p = make_params<T>(h, g, P.pc[q], 1.0, 1.0, -1.0, 1.0, st, st);
-      if (rec) p.d_out = (T*)rec[g.ec];
+      if (!objective) {
+        p.d_out = (T*)arr_at(a->tape, slot * 3 + g.ec, h);
+        p.d_slot = a->d_ctr + 1;
+        p.d_stride = 6 * h->count;
+      }
       return launch_pair<T>(h, g, p);
     });
   };
-  int rc = proc(0, rec_a);
-  if (rc) return rc;
-  if (h->src_comp >= 0 && (rc = add_point(h, st[h->src_comp], post_a))) return rc;
-  const bool probes = a->nprobe && (objective || wrec);
-  if (probes) {
-    fdtd::probe_energy_kernel<T><<<1, 256, 0, h->stream>>>(probe_set<T>(a), (const T*)st[0], (const T*)st[1],
-                                                           (const T*)st[2], a->d_stash, a->d_acc, 0, nullptr);
+  auto source = [&](int off) -> int {
+    if (h->src_comp < 0) return FDTD_OK;
+    h->launches++;
+    fdtd::add_point_table_kernel<T><<<1, 32, 0, h->stream>>>((T*)st[h->src_comp], a->src_at, h->d_srcval,
+                                                             h->srcval_len, a->d_ctr, off, 0.5 * h->dt);
     CK(cudaGetLastError());
-  }
-  if ((rc = proc(1, rec_b))) return rc;
-  if (probes) {
+    return FDTD_OK;
+  };
+  auto probe = [&](int mode) -> int {
+    if (!a->nprobe) return FDTD_OK;
+    h->launches++;
     fdtd::probe_energy_kernel<T><<<1, 256, 0, h->stream>>>(probe_set<T>(a), (const T*)st[0], (const T*)st[1],
-                                                           (const T*)st[2], a->d_stash, a->d_acc,
-                                                           objective ? 1 : 2, wrec);
+                                                           (const T*)st[2], a->d_stash, a->d_acc, mode,
+                                                           mode == 2 ? a->d_wrec : nullptr, a->d_ctr + 1);
     CK(cudaGetLastError());
-  }
-  if (h->src_comp >= 0 && (rc = add_point(h, st[h->src_comp], post_b))) return rc;
-  return FDTD_OK;
+    return FDTD_OK;
+  };
+  int rc;
+  if ((rc = proc(0)) || (rc = source(0)) || (rc = probe(0)) || (rc = proc(1)) || (rc = probe(objective ? 1 : 2)))
+    return rc;
+  return source(1);
 }
 
 // The three adjoint pair launches of procedure `slot` on lam (in place).
 template <typename T>
-int adj_procedure(fdtd_adj_t* a, int slot, void* const* rec, int only_axis = -1) {
+int adj_procedure(fdtd_adj_t* a, int slot, void* const* rec, int only_axis = -1, bool counted = false) {
   fdtd_t* h = a->h;
   const ProcCoef& P = h->proc[slot];
   auto pair = [&](int q) -> int {
@@ -4498,6 +4531,8 @@ int adj_procedure(fdtd_adj_t* a, int slot, void* const* rec, int only_axis = -1)
     x.d = (const T*)rec[g.ec];
     x.grad = a->grad[g.ec];
     x.inv_h = 1.0 / P.h;
+    x.slot = counted ? a->d_ctr + 1 : nullptr;
+    x.stride = counted ? 6 * h->count : 0;
     h->launches++;
     if (g.rows) {
       switch (pick_rows_L(g.N)) {
@@ -4546,14 +4581,92 @@ int adj_point_term(fdtd_adj_t* a, double post) {
 }
 
 template <typename T>
-int adj_inject(fdtd_adj_t* a, const double* wrec, double jbar) {
+int adj_inject(fdtd_adj_t* a, double jbar) {
   fdtd_t* h = a->h;
   if (!a->nprobe) return FDTD_OK;
   const unsigned blocks = (unsigned)std::min(1024, (a->nprobe + 255) / 256);
+  h->launches++;
   fdtd::probe_inject_kernel<T><<<blocks, 256, 0, h->stream>>>(probe_set<T>(a), (T*)a->lam[0], (T*)a->lam[1],
-                                                              (T*)a->lam[2], wrec, jbar);
+                                                              (T*)a->lam[2], a->d_wrec, jbar, a->d_ctr + 1);
   CK(cudaGetLastError());
   return FDTD_OK;
+}
+
+// The reverse of one step (device step and record counters).
+template <typename T>
+int adj_reverse_step(fdtd_adj_t* a, double jbar) {
+  fdtd_t* h = a->h;
+  void *ra[3], *rb[3];
+  for (int c = 0; c < 3; ++c) {
+    ra[c] = arr_at(a->tape, c, h);
+    rb[c] = arr_at(a->tape, 3 + c, h);
+  }
+  auto point = [&](int off) -> int {
+    if (h->src_comp < 0) return FDTD_OK;
+    h->launches++;
+    fdtd::grad_point_table_kernel<T><<<1, 32, 0, h->stream>>>(a->grad[h->src_comp], (const T*)a->lam[h->src_comp],
+                                                              a->src_at, h->d_srcval, h->srcval_len, a->d_ctr, off,
+                                                              0.5 * h->dt, a->eps_src);
+    CK(cudaGetLastError());
+    return FDTD_OK;
+  };
+  int rc;
+  // B procedure: the objective's w_B term enters w-bar; with it added to the E
+  // adjoint before the transposed solve, the output E-bar = q y - E-bar' needs
+  // it added back once more
+  if ((rc = point(1)) || (rc = adj_inject<T>(a, jbar)) || (rc = adj_procedure<T>(a, 1, rb, -1, true)) ||
+      (rc = adj_inject<T>(a, jbar)))
+    return rc;
+  // A procedure
+  if ((rc = point(0))) return rc;
+  return adj_procedure<T>(a, 0, ra, -1, true);
+}
+
+// Capture one step on the handle's stream (the branch-capable stream: adj_on
+// points it there); step and record counters move by ds and dr after it.
+template <typename F>
+int adj_capture(fdtd_adj_t* a, cudaGraphExec_t* exec, long long* kernels, int ds, int dr, F&& step) {
+  fdtd_t* h = a->h;
+  const long long before = h->launches;
+  const bool timing = h->timing;
+  h->timing = false;  // a captured launch has no time of its own
+  CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+  int rc = step();
+  h->timing = timing;
+  if (!rc) {
+    fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, ds, dr, 0);
+    h->launches++;
+    if (cudaGetLastError() != cudaSuccess) rc = FDTD_ERR_CUDA;
+  }
+  cudaGraph_t graph = nullptr;
+  const cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
+  *kernels = h->launches - before;
+  h->launches = before;
+  if (rc || e != cudaSuccess) {
+    if (graph) cudaGraphDestroy(graph);
+    cudaGetLastError();
+    return rc ? rc : cuda_fail(h, e);
+  }
+  const cudaError_t ie = cudaGraphInstantiate(exec, graph, 0);
+  cudaGraphDestroy(graph);
+  CK(ie);
+  return FDTD_OK;
+}
+
+// Run f with the handle's stream set to the capture/replay stream, ordered
+// after the handle's earlier work and before its later work.
+template <typename F>
+int adj_on_replay_stream(fdtd_t* h, F&& f) {
+  if (int rc = ensure_branches(h)) return rc;
+  cudaStream_t home = h->stream;
+  CK(cudaEventRecord(h->g_in, home));
+  CK(cudaStreamWaitEvent(h->g_run, h->g_in, 0));
+  h->stream = h->g_run;
+  const int rc = f();
+  h->stream = home;
+  CK(cudaEventRecord(h->g_out, h->g_run));
+  CK(cudaStreamWaitEvent(home, h->g_out, 0));
+  return rc;
 }
 
 // Launch shape of the adjoint y/z kernels: every feasible candidate timed
@@ -4564,6 +4677,21 @@ int adj_tune_t(fdtd_adj_t* a) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
   const std::string key = "adjoint|" + device_name() + "|p" + std::to_string(h->prec) + "|" +
                           std::to_string(h->nx) + "x" + std::to_string(h->ny) + "x" + std::to_string(h->nz);
+  // as in single_tune_t: the shapes that timing picks most often
+  if (sizeof(T) == 4 && (double)h->nx * h->ny * h->nz <= 1e6) {
+    const AdjCfg cy = {true, 32, 8}, cz = {true, 32, 8};
+    auto fits = [](int N, const AdjCfg& c) {
+      cudaFuncAttributes fa;
+      const int P = segments(std::max(N, 2), c.L, c.lanes);
+      return P <= 32 && cudaFuncGetAttributes(&fa, adj_strided_fn<T>(c.lanes, c.L)) == cudaSuccess &&
+             P * c.lanes <= fa.maxThreadsPerBlock;
+    };
+    if (fits(h->ny, cy) && fits(h->nz, cz)) {
+      a->cfg[0] = cy;
+      a->cfg[1] = cz;
+      return FDTD_OK;
+    }
+  }
   TuneVal v;
   if (tune_cache_get(key, &v) && adj_strided_fn<T>(v[0], v[1]) && adj_strided_fn<T>(v[2], v[3])) {
     a->cfg[0] = {true, v[0], v[1]};
@@ -4630,15 +4758,24 @@ int adj_forward_t(fdtd_adj_t* a) {
   h->shape_tuned = true;
   if ((rc = adj_tune_t<T>(a))) return rc;
   CK(cudaMemsetAsync(a->d_acc, 0, sizeof(double), h->stream));
-  for (long long n = 0; n < a->nsteps; ++n) {
-    if (n % a->every == 0) {
-      void* dst[6];
-      for (int c = 0; c < 6; ++c) dst[c] = arr_at(a->ckpt, (n / a->every) * 6 + c, h);
-      if ((rc = copy_arrays(h, dst, h->f, 0, 6))) return rc;
+  rc = adj_on_replay_stream(h, [&]() -> int {
+    if (!a->g_fwd)
+      if (int e = adj_capture(a, &a->g_fwd, &a->k_fwd, 1, 0, [&]() { return adj_forward_step<T>(a, h->f, true); }))
+        return e;
+    fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, 0, 0, 1);
+    for (long long n = 0; n < a->nsteps; ++n) {
+      if (n % a->every == 0) {
+        void* dst[6];
+        for (int c = 0; c < 6; ++c) dst[c] = arr_at(a->ckpt, (n / a->every) * 6 + c, h);
+        if (int e = copy_arrays(h, dst, h->f, 0, 6)) return e;
+      }
+      CK(cudaGraphLaunch(a->g_fwd, h->stream));
+      h->launches += a->k_fwd;
+      h->steps++;
     }
-    if ((rc = adj_forward_step<T>(a, h->f, n, true, nullptr, nullptr, nullptr))) return rc;
-    h->steps++;
-  }
+    return FDTD_OK;
+  });
+  if (rc) return rc;
   h->output_valid = false;
   CK(cudaMemcpyAsync(&a->objective, a->d_acc, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
@@ -4652,42 +4789,34 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
   const size_t bytes = (size_t)h->count * h->esize;
   for (int c = 0; c < 6; ++c) CK(cudaMemsetAsync(a->lam[c], 0, bytes, h->stream));
   for (int c = 0; c < 3; ++c) CK(cudaMemsetAsync(a->grad[c], 0, sizeof(double) * h->count, h->stream));
-  auto slot = [&](int s, void** out) {
-    for (int c = 0; c < 3; ++c) out[c] = arr_at(a->tape, (long long)s * 3 + c, h);
-  };
-  for (int seg = a->nseg - 1; seg >= 0; --seg) {
-    const long long n0 = (long long)seg * a->every;
-    const long long n1 = std::min(n0 + a->every, a->nsteps);
-    void* src[6];
-    for (int c = 0; c < 6; ++c) src[c] = arr_at(a->ckpt, (long long)seg * 6 + c, h);
-    if ((rc = copy_arrays(h, a->work, src, 0, 6))) return rc;
-    for (long long n = n0; n < n1; ++n) {
-      const int m = (int)(n - n0);
-      void *ra[3], *rb[3];
-      slot(2 * m, ra);
-      slot(2 * m + 1, rb);
-      if ((rc = adj_forward_step<T>(a, a->work, n, false, ra, rb, a->d_wrec + (size_t)m * a->nprobe))) return rc;
+  rc = adj_on_replay_stream(h, [&]() -> int {
+    if (!a->g_rec)
+      if (int e = adj_capture(a, &a->g_rec, &a->k_rec, 1, 1, [&]() { return adj_forward_step<T>(a, a->work, false); }))
+        return e;
+    if (a->g_rev && a->g_jbar != jbar) {
+      CK(cudaStreamSynchronize(h->stream));
+      cudaGraphExecDestroy(a->g_rev);
+      a->g_rev = nullptr;
     }
-    for (long long n = n1 - 1; n >= n0; --n) {
-      const int m = (int)(n - n0);
-      void *ra[3], *rb[3];
-      slot(2 * m, ra);
-      slot(2 * m + 1, rb);
-      const double* wrec = a->d_wrec + (size_t)m * a->nprobe;
-      const double post_a = 0.5 * h->dt * source_value(h, n);
-      const double post_b = 0.5 * h->dt * source_value(h, n + 1);
-      // B procedure of step n: the objective's w_B term enters w-bar; with
-      // it added to the E adjoint before the transposed solve, the output
-      // E-bar = q y - E-bar' needs it added back once more
-      if ((rc = adj_point_term<T>(a, post_b))) return rc;
-      if ((rc = adj_inject<T>(a, wrec, jbar))) return rc;
-      if ((rc = adj_procedure<T>(a, 1, rb))) return rc;
-      if ((rc = adj_inject<T>(a, wrec, jbar))) return rc;
-      // A procedure of step n
-      if ((rc = adj_point_term<T>(a, post_a))) return rc;
-      if ((rc = adj_procedure<T>(a, 0, ra))) return rc;
+    if (!a->g_rev)
+      if (int e = adj_capture(a, &a->g_rev, &a->k_rev, -1, -1, [&]() { return adj_reverse_step<T>(a, jbar); }))
+        return e;
+    a->g_jbar = jbar;
+    for (int seg = a->nseg - 1; seg >= 0; --seg) {
+      const long long n0 = (long long)seg * a->every;
+      const long long n1 = std::min(n0 + a->every, a->nsteps);
+      void* src[6];
+      for (int c = 0; c < 6; ++c) src[c] = arr_at(a->ckpt, (long long)seg * 6 + c, h);
+      if (int e = copy_arrays(h, a->work, src, 0, 6)) return e;
+      fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, n0, 0, 1);
+      for (long long n = n0; n < n1; ++n) CK(cudaGraphLaunch(a->g_rec, h->stream));
+      fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, -1, -1, 0);
+      for (long long n = n0; n < n1; ++n) CK(cudaGraphLaunch(a->g_rev, h->stream));
+      h->launches += (n1 - n0) * (a->k_rec + a->k_rev) + 2;
     }
-  }
+    return FDTD_OK;
+  });
+  if (rc) return rc;
   // input initialization v0 = u0 + (dt/2) B u0 + (dt/2) f
   if ((rc = adj_point_term<T>(a, 0.5 * h->dt * source_value(h, 0)))) return rc;
   const ProcCoef& P = h->proc[1];
@@ -4714,17 +4843,9 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
 }
 
 void adj_free(fdtd_adj_t* a) {
-  void* ptrs[] = {a->d_probe_at, a->d_probe_comp, a->d_stash, a->d_acc, a->d_cell, a->ckpt, a->tape, a->d_wrec};
-  for (void* p : ptrs)
-    if (p) cudaFree(p);
-  for (int c = 0; c < 6; ++c) {
-    if (a->work[c]) cudaFree(a->work[c]);
-    if (a->lam[c]) cudaFree(a->lam[c]);
-  }
-  for (int c = 0; c < 3; ++c) {
-    if (a->grad[c]) cudaFree(a->grad[c]);
-    if (a->u0h[c]) cudaFree(a->u0h[c]);
-  }
+  for (cudaGraphExec_t g : {a->g_fwd, a->g_rec, a->g_rev})
+    if (g) cudaGraphExecDestroy(g);
+  if (a->slab) cudaFree(a->slab);
 }
 
 }  // namespace
@@ -4780,33 +4901,42 @@ int fdtd_adj_create(fdtd_t* h, const int32_t block[6], int64_t nsteps, int32_t c
     a->eps_src = kEps0 * er;
   }
   const size_t arr = (size_t)h->count * h->esize;
-  bool ok = true;
-  auto alloc = [&](void** p, size_t n) {
-    if (!ok) return;
-    if (dev_malloc((void**)p, n) != cudaSuccess) ok = false;
-    else a->bytes += (long long)n;
+  // one allocation for everything (26 of them, and their releases, took 2.2 ms
+  // of a 17 ms gradient evaluation), each part at a multiple of 256 bytes
+  std::vector<std::pair<void**, size_t>> parts;
+  auto part = [&](void** p, size_t n) {
+    parts.push_back({p, (n + 255) / 256 * 256});
+    a->bytes += (long long)n;
   };
-  alloc((void**)&a->d_probe_at, sizeof(long long) * std::max<size_t>(1, at.size()));
-  alloc((void**)&a->d_probe_comp, sizeof(int) * std::max<size_t>(1, comp.size()));
-  alloc((void**)&a->d_stash, sizeof(double) * std::max<size_t>(1, at.size()));
-  alloc((void**)&a->d_acc, sizeof(double));
-  alloc((void**)&a->d_cell, sizeof(double) * (size_t)h->nx * h->ny * h->nz);
-  alloc(&a->ckpt, arr * 6 * (size_t)a->nseg);
-  alloc(&a->tape, arr * 3 * (size_t)(2 * checkpoint_every));
-  alloc((void**)&a->d_wrec, sizeof(double) * std::max<size_t>(1, at.size()) * (size_t)checkpoint_every);
+  part((void**)&a->d_probe_at, sizeof(long long) * std::max<size_t>(1, at.size()));
+  part((void**)&a->d_probe_comp, sizeof(int) * std::max<size_t>(1, comp.size()));
+  part((void**)&a->d_stash, sizeof(double) * std::max<size_t>(1, at.size()));
+  part((void**)&a->d_acc, sizeof(double));
+  part((void**)&a->d_ctr, 2 * sizeof(long long));
+  part((void**)&a->d_cell, sizeof(double) * (size_t)h->nx * h->ny * h->nz);
+  part(&a->ckpt, arr * 6 * (size_t)a->nseg);
+  part(&a->tape, arr * 3 * (size_t)(2 * checkpoint_every));
+  part((void**)&a->d_wrec, sizeof(double) * std::max<size_t>(1, at.size()) * (size_t)checkpoint_every);
   for (int c = 0; c < 6; ++c) {
-    alloc(&a->work[c], arr);
-    alloc(&a->lam[c], arr);
+    part(&a->work[c], arr);
+    part(&a->lam[c], arr);
   }
   for (int c = 0; c < 3; ++c) {
-    alloc((void**)&a->grad[c], sizeof(double) * h->count);
-    alloc(&a->u0h[c], arr);
+    part((void**)&a->grad[c], sizeof(double) * h->count);
+    part(&a->u0h[c], arr);
   }
-  if (!ok) {
+  size_t total = 0;
+  for (auto& q : parts) total += q.second;
+  if (dev_malloc(&a->slab, total) != cudaSuccess) {
     cudaGetLastError();
     adj_free(a);
     delete a;
     return FDTD_ERR_OOM;
+  }
+  size_t used = 0;
+  for (auto& q : parts) {
+    *q.first = (char*)a->slab + used;
+    used += q.second;
   }
   if (!at.empty() &&
       (cudaMemcpy(a->d_probe_at, at.data(), sizeof(long long) * at.size(), cudaMemcpyHostToDevice) != cudaSuccess ||

@@ -13,8 +13,8 @@
 //    by two shuffles in the warp, then over the warps of the tile through
 //    shared memory with one barrier per sweep.
 //  - homogeneous media: a segment's carry product is the constant (-m)^L, so
-//    the scans move values only, and stop where the product is below 2^-50
-//    of the carry.
+//    the scans move values only (and the tiles' stop where the product is
+//    below 2^-50 of the carry).
 //  - 32-bit element offsets; a node's address is formed once for all arrays.
 //  - the point source is added by the thread that owns its sample.
 // FADI 128^3 FP32: 37.3 -> 30.8 us per step, 64^3 16.5 -> 9.9, 32^3 13.6 -> 7.0

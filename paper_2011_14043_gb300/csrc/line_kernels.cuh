@@ -101,6 +101,8 @@ struct PairParams {
   int* err;              // set to 1 when a bounded device wait gives up
   T* d_out;              // per-node kernels: when set, also E_in - E_out per E node
                          // (the reverse pass's record of the procedure)
+  const long long* d_slot;  // when set, d_out moves on by *d_slot * d_stride elements (a
+  long long d_stride;       // captured recomputation step writes its own record)
   // per-node mu (general media): face f between nodes f and f+1 (stored at
   // node f) has its own H coupling kd_f = kd_scale * nkd[f] and off-diagonal
   // noffh[f] + noffl[f]; nullptr when mu is uniform
@@ -117,8 +119,8 @@ struct PairParams {
   int kg_len;            // the wall correction is zero from this node on (a multiple of
                          // the segment length)
   // uniform media, x lines: carry products (-m)^(L d) of d = 1, 2, 4, 8, 16 segments
-  // (hi, lo); nscan: the first d whose product is below 2^-50 (the scan stops there);
-  // kx: the same in runs of 32 nodes (the y/z tiles' carries over warps)
+  // (hi, lo); nscan: the first d whose product is zero (the scan stops there);
+  // kx: runs of 32 nodes until the product is below 2^-50 (the y/z tiles' carries over warps)
   T sc[2][5];
   int nscan, kx;
   T* tmp4;               // fourth-order differences: field-shaped scratch of the line solve
@@ -770,9 +772,10 @@ __global__ void proc_strided_kernel(const PairParams<T> p) {
   if (active) strided_store<T, L>(p, base, j0, E, H, y, win);
   if constexpr (PER_NODE) {
     if (active && p.d_out) {
+      T* d_out = p.d_out + (p.d_slot ? *p.d_slot * p.d_stride : 0);
 #pragma unroll
       for (int t = 0; t < L; ++t)
-        if (j0 + t < N) p.d_out[base + (long long)(j0 + t) * ls] = E[t] - fma(p.alpha, y[t], p.beta * E[t]);
+        if (j0 + t < N) d_out[base + (long long)(j0 + t) * ls] = E[t] - fma(p.alpha, y[t], p.beta * E[t]);
     }
   }
 }
@@ -1265,12 +1268,13 @@ __device__ __forceinline__ void row_solve_store(const PairParams<T>& p, unsigned
       E[t] = En[t];
     }
     if (p.d_out && ok) {
+      T* d_out = p.d_out + (p.d_slot ? *p.d_slot * p.d_stride : 0);
       if (j0 + L <= N) {
-        store_seg<T, L>(p.d_out + base + j0, D);
+        store_seg<T, L>(d_out + base + j0, D);
       } else {
 #pragma unroll
         for (int t = 0; t < L; ++t)
-          if (j0 + t < N) p.d_out[base + j0 + t] = D[t];
+          if (j0 + t < N) d_out[base + j0 + t] = D[t];
       }
     }
   } else {
@@ -1341,8 +1345,7 @@ __device__ __forceinline__ void fma_pair(T& r0, T& r1, T a0, T a1, T b0, T b1, T
 //
 // LPL lanes of a warp hold one line (lane sl its nodes [sl L, sl L + L)).  A
 // segment's carry product is the constant (-m)^L, so the scans shuffle the
-// carries alone and stop after the first distance whose product is below
-// 2^-50.  What bounds these lines is instruction issue: the elementwise
+// carries alone and stop after the first distance whose product underflows.  What bounds these lines is instruction issue: the elementwise
 // parts run as packed FMAs on neighbouring nodes.
 // On return E, H hold the new values.
 template <typename T, int L, int LPL>
