@@ -1158,29 +1158,29 @@ int launch_pair_gm(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
 // running concurrently).
 
 template <typename T>
-size_t line4_tile_smem(const PairGeom& g) {
-  return 2 * (size_t)g.N * fdtd::line4_tile_stride<T>(g.rows) * sizeof(T);
-}
-
-template <typename T, bool ROWS, int CH>
-cudaError_t set_line4_tile_attr() {
-  return cudaFuncSetAttribute(fdtd::proc_line4_tile_kernel<T, ROWS, CH>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(2 * (size_t)32 * CH * fdtd::line4_tile_stride<T>(ROWS) * sizeof(T)));
+size_t line4_smem(const PairGeom& g, bool keep) {
+  return (keep ? 2 : 1) * (size_t)g.N * fdtd::line4_tile_stride<T>(g.rows) * sizeof(T);
 }
 
 // Dynamic shared memory limits of the tiled kernels (set outside any stream
 // capture, from fdtd_set_order).
+template <typename T, bool ROWS>
+cudaError_t set_line4_attr() {
+  const int per = (int)(fdtd::line4_tile_stride<T>(ROWS) * sizeof(T));
+  const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(fdtd::proc_line4_tile_kernel<T, ROWS, 2>, a, 2 * 64 * per);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fdtd::proc_line4_tile_kernel<T, ROWS, 8>, a, 2 * 256 * per);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fdtd::proc_line4_tile_kernel<T, ROWS, 16>, a, 2 * 512 * per);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fdtd::proc_line4_reread_kernel<T, ROWS>, a, kLine4TileMaxN * per);
+  return e;
+}
+
 template <typename T>
 cudaError_t ensure_line4_tile_attr() {
   static bool attr_set = false;
   if (attr_set) return cudaSuccess;
-  cudaError_t e = cudaSuccess;
-  const cudaError_t r[6] = {set_line4_tile_attr<T, true, 2>(),   set_line4_tile_attr<T, true, 8>(),
-                            set_line4_tile_attr<T, true, 16>(),  set_line4_tile_attr<T, false, 2>(),
-                            set_line4_tile_attr<T, false, 8>(), set_line4_tile_attr<T, false, 16>()};
-  for (cudaError_t x : r)
-    if (x != cudaSuccess) e = x;
+  cudaError_t e = set_line4_attr<T, true>();
+  if (e == cudaSuccess) e = set_line4_attr<T, false>();
   if (e == cudaSuccess) attr_set = true;
   return e;
 }
@@ -1194,20 +1194,26 @@ bool line4_tile_eligible(const fdtd_t* h, const PairGeom& g, const fdtd::PairPar
   return true;
 }
 
-template <typename T, bool ROWS, int CH>
-void launch_line4_tile_ch(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
+// Launches of at most two blocks per SM (the three pairs of a procedure run at
+// once) keep H and E on chip; more of them read both twice and put 5 on
+// an SM (measured in line4_kernels.cuh; 400x60x60, 113 blocks per x launch:
+// 114 against 150 us per step).
+template <typename T, bool ROWS>
+void launch_line4_tile(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
   constexpr int LN = fdtd::line4_tile_lines<T>();
   const long long blocks = ROWS ? (g.n_lines() + LN - 1) / LN
                                 : (long long)((g.lane_hi + LN - 1) / LN) * g.n_o;
-  fdtd::proc_line4_tile_kernel<T, ROWS, CH><<<(unsigned)blocks, 256, line4_tile_smem<T>(g), h->stream>>>(p);
-}
-
-template <typename T, bool ROWS>
-void launch_line4_tile(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
+  const bool keep = blocks <= 2LL * h->num_sms;
+  const size_t smem = line4_smem<T>(g, keep);
+  const unsigned nb = (unsigned)blocks;
+  if (!keep) {
+    fdtd::proc_line4_reread_kernel<T, ROWS><<<nb, 256, smem, h->stream>>>(p);
+    return;
+  }
   switch (fdtd::line4_tile_ch(g.N)) {
-    case 2: launch_line4_tile_ch<T, ROWS, 2>(h, g, p); break;
-    case 8: launch_line4_tile_ch<T, ROWS, 8>(h, g, p); break;
-    default: launch_line4_tile_ch<T, ROWS, 16>(h, g, p); break;
+    case 2: fdtd::proc_line4_tile_kernel<T, ROWS, 2><<<nb, 256, smem, h->stream>>>(p); break;
+    case 8: fdtd::proc_line4_tile_kernel<T, ROWS, 8><<<nb, 256, smem, h->stream>>>(p); break;
+    default: fdtd::proc_line4_tile_kernel<T, ROWS, 16><<<nb, 256, smem, h->stream>>>(p); break;
   }
 }
 

@@ -160,3 +160,21 @@ def test_batch_in_one_launch_per_procedure(scheme, media):
             for c in ("hx", "hy", "hz"):
                 assert np.array_equal(alone[q].get_state(c), s.get_state(c)), (q, c)
     b.close()
+
+
+@pytest.mark.parametrize("dims", [(70, 90, 110), (130, 40, 257), (512, 30, 40)])
+def test_fourth_order_kernels_of_many_blocks(dims):
+    """Fourth-order lines in launches of more than two blocks per SM (E and H
+    read twice) and fewer: bit for bit the one-thread-per-line kernel's."""
+    from paper_2011_14043_gb300 import Simulation
+    u0 = random_fields(*dims, 4)
+    out = []
+    for tune in ((0, 0), (0, 512)):
+        s = Simulation(*dims, 1e-3, scheme="fss", precision="f32", cfl=4.0, tune=tune)
+        s.set_order(4)
+        s.set_fields(u0)
+        s.step(2)
+        out.append({c: s.get_field(c) for c in u0})
+        s.close()
+    for c in u0:
+        assert np.array_equal(out[0][c], out[1][c]), c
