@@ -2060,8 +2060,16 @@ int plane_steps(fdtd_t* h, int64_t nsteps) {
   p.nx = h->nx;
   p.ny = h->ny;
   p.pitch = h->pitch;
-  p.R = (h->ny + fdtd::kPlaneBlocks - 1) / fdtd::kPlaneBlocks;
+  // rows and columns per block: multiples of L (a lane's nodes go to one block);
+  // padded by one 16-byte vector, which keeps the pushes aligned
+  auto share = [L](int n) { return ((n + fdtd::kPlaneBlocks - 1) / fdtd::kPlaneBlocks + L - 1) / L * L; };
+  const int vec = std::min(L, (int)(16 / sizeof(T)));
+  p.R = share(h->ny);
+  p.RP = p.R + vec;
+  p.C = share(h->nx);
+  p.CP = p.C + vec;
   p.ld = (h->nx + 1 + 3) / 4 * 4;
+  p.ldc = (h->ny + 1 + 3) / 4 * 4;
   static const int seq_fss[3] = {0, 1, 0};
   p.nproc = h->scheme == FDTD_FSS ? 3 : 2;
   for (int k = 0; k < 3; ++k) p.seq[k] = seq_fss[k];
@@ -2087,7 +2095,9 @@ int plane_steps(fdtd_t* h, int64_t nsteps) {
     const int c = h->probe_comp[q];
     const long long at = h->probe_at[q];
     const int k = (int)(at / h->plane), j = (int)(at % h->plane / h->pitch), i = (int)(at % h->pitch);
-    p.pk[q] = (k > 0 || j >= h->ny || (c != EZ && c != HX && c != HY)) ? 3 : (c == EZ ? 0 : (c == HX ? 1 : 2));
+    // (Hx on the walls i = 0, nx and all of row ny keep their values)
+    const bool fixed = k > 0 || j >= h->ny || (c == HX && (i == 0 || i >= h->nx));
+    p.pk[q] = fixed || (c != EZ && c != HX && c != HY) ? 3 : (c == EZ ? 0 : (c == HX ? 1 : 2));
     p.pi[q] = i;
     p.pj[q] = j;
     p.pptr[q] = (const T*)h->f[c] + at;
@@ -2096,12 +2106,13 @@ int plane_steps(fdtd_t* h, int64_t nsteps) {
   p.out = h->d_probe;
   p.cap = h->probe_cap;
   const void* fn = plane_fn<T>(L);
-  const size_t smem = 3 * (size_t)p.R * p.ld * sizeof(T);
+  const size_t smem =
+      ((size_t)(h->nx + 1) * p.RP + (size_t)(h->ny + 1) * p.CP + (size_t)p.R * p.ld + (size_t)p.C * p.ldc) * sizeof(T);
   CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   CK(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(fdtd::kPlaneBlocks);
-  cfg.blockDim = dim3((unsigned)std::min(16, std::max(4, p.R)) * 32);
+  cfg.blockDim = dim3((unsigned)std::min(16, std::max({4, p.R, p.C})) * 32);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = h->stream;
   cudaLaunchAttribute at;
