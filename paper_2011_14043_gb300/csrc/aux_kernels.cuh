@@ -221,10 +221,8 @@ struct ProbeParams {
 // mode 0: stash[p] = value;  mode 1: out[p][col] = (stash[p] + value - sub[p])/2;
 // mode 2: out[p][col] = value.
 template <typename T>
-__global__ void probe_kernel(const ProbeParams<T> pp, double* stash, double* out, long long ld,
-                             long long col, int mode) {
-  const int q = threadIdx.x;
-  if (q >= pp.n) return;
+__device__ __forceinline__ void record_probe(const ProbeParams<T>& pp, int q, double* stash, double* out,
+                                             long long ld, long long col, int mode) {
   const double v = (double)pp.arr[q][pp.at[q]];
   double sub = pp.sub[q];
   if (pp.step) {
@@ -241,6 +239,50 @@ __global__ void probe_kernel(const ProbeParams<T> pp, double* stash, double* out
   } else {
     out[(long long)q * ld + col] = v;
   }
+}
+
+template <typename T>
+__global__ void probe_kernel(const ProbeParams<T> pp, double* stash, double* out, long long ld,
+                             long long col, int mode) {
+  const int q = threadIdx.x;
+  if (q < pp.n) record_probe(pp, q, stash, out, ld, col, mode);
+}
+
+// What a captured step does between two procedures, in one launch (each small
+// launch in the chain costs the step 2 to 3 us): up to four source terms
+// added to one sample one after the other (as add_point_table_kernel adds
+// them), then the probes (mode >= 0), then the step counter's advance.
+template <typename T>
+struct Between {
+  T* y;
+  long long at;
+  int nterms;
+  double coef[4];
+  int off[4];
+  const double* table;
+  long long len;
+  long long* step;
+  long long advance;
+  ProbeParams<T> pp;
+  int mode;
+  double* stash;
+  double* out;
+  long long ld, col;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(32) between_kernel(const Between<T> b) {
+  const int q = threadIdx.x;
+  if (q == 0)
+    for (int m = 0; m < b.nterms; ++m) {
+      const long long n = *b.step + b.off[m];
+      const double v = (n >= 0 && n < b.len) ? b.table[n] : 0.0;
+      b.y[b.at] = (T)__dadd_rn((double)b.y[b.at], __dmul_rn(b.coef[m], v));
+    }
+  __syncwarp();
+  if (b.mode >= 0 && q < b.pp.n) record_probe(b.pp, q, b.stash, b.out, b.ld, b.col, b.mode);
+  __syncwarp();
+  if (q == 0 && b.advance) *b.step += b.advance;
 }
 
 // The six components' weighted sums of squares in one launch: per block one

@@ -1700,11 +1700,8 @@ int scheme_init(fdtd_t* h) {
   return FDTD_OK;
 }
 
-// sub_step >= 0: inside a captured step, that many steps past the device
-// counter; post is then the coefficient of the source value at offset 1.
 template <typename T>
-int record_probes(fdtd_t* h, int mode, double post, void* const* arrays, int sub_step = -1) {
-  if (h->nprobes == 0) return FDTD_OK;
+fdtd::ProbeParams<T> probe_params(const fdtd_t* h, double post, void* const* arrays) {
   fdtd::ProbeParams<T> pp = {};
   pp.n = h->nprobes;
   const long long src_at = h->src_comp >= 0 ? elem_index(h, h->src_i, h->src_j, h->src_k) : -1;
@@ -1713,15 +1710,15 @@ int record_probes(fdtd_t* h, int mode, double post, void* const* arrays, int sub
     pp.at[q] = h->probe_at[q];
     pp.sub[q] = (h->probe_comp[q] == h->src_comp && h->probe_at[q] == src_at) ? post : 0.0;
   }
+  return pp;
+}
+
+template <typename T>
+int record_probes(fdtd_t* h, int mode, double post, void* const* arrays) {
+  if (h->nprobes == 0) return FDTD_OK;
   h->launches++;
-  if (sub_step >= 0) {
-    pp.step = h->d_step;
-    pp.table = h->d_srcval;
-    pp.table_len = h->d_srcval ? h->srcval_len : 0;
-    pp.table_off = sub_step + 1;
-  }
-  fdtd::probe_kernel<T><<<1, 32, 0, h->stream>>>(pp, h->d_stash, h->d_probe, h->probe_cap,
-                                                 sub_step >= 0 ? sub_step : h->steps, mode);
+  fdtd::probe_kernel<T><<<1, 32, 0, h->stream>>>(probe_params<T>(h, post, arrays), h->d_stash, h->d_probe,
+                                                 h->probe_cap, h->steps, mode);
   CK(cudaGetLastError());
   return FDTD_OK;
 }
@@ -1858,8 +1855,52 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
     h->launches++;
     return cudaGetLastError();
   };
+  // source terms not yet launched, and the launch of what lies between two
+  // procedures: those terms, the probes (mode >= 0; FADI's after B takes off
+  // the source just added, post[1] f at offset 1) and the counter's advance
+  std::vector<std::pair<double, int>> terms;
+  auto between = [&](int st, int mode, long long advance) -> int {
+    if (terms.empty() && mode < 0 && advance == 0) return FDTD_OK;
+    auto go = [&](auto zero) {
+      using T = decltype(zero);
+      fdtd::Between<T> b = {};
+      b.y = src ? (T*)h->f[h->src_comp] : nullptr;
+      b.at = src_at;
+      b.nterms = (int)terms.size();
+      for (int m = 0; m < b.nterms; ++m) {
+        b.coef[m] = terms[m].first;
+        b.off[m] = terms[m].second;
+      }
+      b.table = h->d_srcval;
+      b.len = h->d_srcval ? h->srcval_len : 0;
+      b.step = h->d_step;
+      b.advance = advance;
+      b.mode = mode;
+      if (mode >= 0) {
+        b.pp = probe_params<T>(h, mode == 1 ? post[1] : 0.0, h->f);
+        b.pp.step = h->d_step;
+        b.pp.table = b.table;
+        b.pp.table_len = b.len;
+        b.pp.table_off = st + 1;
+        b.stash = h->d_stash;
+        b.out = h->d_probe;
+        b.ld = h->probe_cap;
+        b.col = st;
+      }
+      fdtd::between_kernel<T><<<1, 32, 0, h->g_run>>>(b);
+    };
+    if (h->prec == FDTD_F64) go(0.0);
+    else go(0.0f);
+    terms.clear();
+    h->launches++;
+    return cudaGetLastError() == cudaSuccess ? FDTD_OK : FDTD_ERR_CUDA;
+  };
+  auto term = [&](double coef, int off) {
+    if (src && coef != 0.0) terms.push_back({coef, off});
+  };
   cudaStream_t home = h->stream;
   const long long before = h->launches;
+  bool advanced = false;
   NvtxScope range("step graph capture");
   CK(cudaStreamBeginCapture(h->g_run, cudaStreamCaptureModeThreadLocal));
   int rc = FDTD_OK;
@@ -1896,8 +1937,11 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
           rc = FDTD_ERR_CUDA;
         continue;
       }
-      if (add_src(pre[k], st) != cudaSuccess) rc = FDTD_ERR_CUDA;
-      if (rc == FDTD_OK && add_src(pre2[k], st + 1) != cudaSuccess) rc = FDTD_ERR_CUDA;
+      // (at most two terms after a procedure and two before the next)
+      term(pre[k], st);
+      term(pre2[k], st + 1);
+      // FADI's probes stash their samples after A
+      rc = between(st, h->nprobes > 0 && h->scheme == FDTD_FADI && k == 1 ? 0 : -1, 0);
       if (rc == FDTD_OK && cudaEventRecord(h->g_fork, h->g_run) != cudaSuccess) rc = FDTD_ERR_CUDA;
       const ProcCoef& P = h->proc[seq[k]];
       for (int q = 0; q < 3 && rc == FDTD_OK; ++q) {
@@ -1916,20 +1960,17 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
                               cudaStreamWaitEvent(h->g_run, h->g_join[q], 0) != cudaSuccess))
           rc = FDTD_ERR_CUDA;
       }
-      if (rc == FDTD_OK && add_src(post[k], st + post_off[k]) != cudaSuccess) rc = FDTD_ERR_CUDA;
-      if (rc == FDTD_OK && add_src(post2[k], st + 1) != cudaSuccess) rc = FDTD_ERR_CUDA;
-      // probes as one_step records them
-      if (rc == FDTD_OK && h->nprobes > 0 && (h->scheme == FDTD_FADI || k == nproc - 1)) {
-        const int mode = h->scheme == FDTD_FADI ? k : 2;
-        const double sub = mode == 1 ? post[1] : 0.0;
-        h->stream = h->g_run;
-        rc = h->prec == FDTD_F64 ? record_probes<double>(h, mode, sub, h->f, st)
-                                 : record_probes<float>(h, mode, sub, h->f, st);
-        h->stream = home;
-      }
+      term(post[k], st + post_off[k]);
+      term(post2[k], st + 1);
+    }
+    if (!fused && rc == FDTD_OK) {
+      // the end of the step: its last source terms, probes as one_step records
+      // them, and (after the last step of the graph) the counter
+      advanced = st == count - 1 && counted;
+      rc = between(st, h->nprobes == 0 ? -1 : (h->scheme == FDTD_FADI ? 1 : 2), advanced ? count : 0);
     }
   }
-  if (rc == FDTD_OK && counted) {
+  if (rc == FDTD_OK && counted && !advanced) {
     fdtd::step_counter_kernel<<<1, 32, 0, h->g_run>>>(h->d_step, count, 1);
     h->launches++;
     if (cudaGetLastError() != cudaSuccess) rc = FDTD_ERR_CUDA;
