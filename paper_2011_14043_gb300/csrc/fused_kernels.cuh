@@ -35,7 +35,8 @@ constexpr int kFusedL = 8;         // nodes per segment
 constexpr int kFusedMaxN = 256;    // 8 warps x 4 segments x 8 nodes
 constexpr int kFusedThreads = 256;
 
-// A y/z thread's column: V adjacent x lines, one operation on all of them.
+// A y/z thread's column (FP32 fields): V = 2 adjacent x lines, one operation on
+// both of them.
 template <typename T>
 struct Wide;
 template <>
@@ -43,44 +44,29 @@ struct Wide<float> {
   using type = float2;
   static constexpr int V = 2;
 };
-template <>
-struct Wide<double> {
-  using type = double;
-  static constexpr int V = 1;
-};
 
 __device__ __forceinline__ float2 wset(float2, float a) { return make_float2(a, a); }
-__device__ __forceinline__ double wset(double, double a) { return a; }
 __device__ __forceinline__ float2 wfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ double wfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float2 wmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ double wmul(double a, double b) { return a * b; }
 __device__ __forceinline__ float2 wadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ double wadd(double a, double b) { return a + b; }
 __device__ __forceinline__ float2 wsub(float2 a, float2 b) {
   return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);  // one rounding, as a - b
 }
-__device__ __forceinline__ double wsub(double a, double b) { return a - b; }
 __device__ __forceinline__ float2 wup(float2 a, int d) {
   return make_float2(__shfl_up_sync(0xffffffffu, a.x, d), __shfl_up_sync(0xffffffffu, a.y, d));
 }
-__device__ __forceinline__ double wup(double a, int d) { return __shfl_up_sync(0xffffffffu, a, d); }
 __device__ __forceinline__ float2 wdown(float2 a, int d) {
   return make_float2(__shfl_down_sync(0xffffffffu, a.x, d), __shfl_down_sync(0xffffffffu, a.y, d));
 }
-__device__ __forceinline__ double wdown(double a, int d) { return __shfl_down_sync(0xffffffffu, a, d); }
 __device__ __forceinline__ float2 wfrom(float2 a, int l) {
   return make_float2(__shfl_sync(0xffffffffu, a.x, l), __shfl_sync(0xffffffffu, a.y, l));
 }
-__device__ __forceinline__ double wfrom(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
 __device__ __forceinline__ float2 wsel(bool c, float2 a, float2 b) { return make_float2(c ? a.x : b.x, c ? a.y : b.y); }
-__device__ __forceinline__ double wsel(bool c, double a, double b) { return c ? a : b; }
 
 // (hi + lo) x + c, the coefficient a scalar of the field precision
 template <typename T, typename W>
 __device__ __forceinline__ W wfma2(T hi, T lo, W x, W c) {
-  if constexpr (use_hilo<T>()) return wfma(wset(x, hi), x, wfma(wset(x, lo), x, c));
-  else return wfma(wset(x, hi), x, c);
+  return wfma(wset(x, hi), x, wfma(wset(x, lo), x, c));
 }
 
 // A point source on one E sample, added by the thread that owns it: before
@@ -162,7 +148,7 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
   const unsigned line = (unsigned)o * (unsigned)p.os + (unsigned)x;
   const bool in_grid = FDTD_IN_RANGE((long long)line, (long long)line + (long long)(N - 1) * p.ls + V, p.n_elem);
   const bool a0 = x >= p.lane_lo && x < p.lane_hi && in_grid;
-  const bool a1 = V == 2 && x + 1 >= p.lane_lo && x + 1 < p.lane_hi && in_grid;
+  const bool a1 = x + 1 >= p.lane_lo && x + 1 < p.lane_hi && in_grid;
   const bool any = a0 || a1;
   const unsigned lsb = (unsigned)p.ls * (unsigned)sizeof(T);
   const unsigned off = line * (unsigned)sizeof(T) + (unsigned)j0 * lsb;
@@ -187,7 +173,7 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
         if constexpr (PN) {
           y[t] = *reinterpret_cast<const W*>(at_bytes(p.nq, at));
           ib[t] = *reinterpret_cast<const W*>(at_bytes(p.nib, at));
-          if constexpr (use_hilo<T>()) il[t] = *reinterpret_cast<const W*>(at_bytes(p.nibl, at));
+          il[t] = *reinterpret_cast<const W*>(at_bytes(p.nibl, at));
         }
       }
     }
@@ -196,7 +182,7 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
       hm1 = *reinterpret_cast<const W*>(at_bytes(p.h_in, at));
       if constexpr (PN) {
         ibp = *reinterpret_cast<const W*>(at_bytes(p.nib, at));
-        if constexpr (use_hilo<T>()) ilp = *reinterpret_cast<const W*>(at_bytes(p.nibl, at));
+        ilp = *reinterpret_cast<const W*>(at_bytes(p.nibl, at));
       }
     }
   }
@@ -214,12 +200,8 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
 #pragma unroll
     for (int t = 0; t < L; ++t)
       if (t == src_t) {
-        if constexpr (V == 2) {
-          if (src_hi) E[t].y = source_add<T>(fp.src, coef, offs, E[t].y);
-          else E[t].x = source_add<T>(fp.src, coef, offs, E[t].x);
-        } else {
-          E[t] = source_add<T>(fp.src, coef, offs, E[t]);
-        }
+        if (src_hi) E[t].y = source_add<T>(fp.src, coef, offs, E[t].y);
+        else E[t].x = source_add<T>(fp.src, coef, offs, E[t].x);
       }
   };
   if (src_t >= 0) source(fp.src.pre, fp.src.pre_off);
@@ -264,10 +246,7 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
     W wn = zero;
 #pragma unroll
     for (int t = L - 1; t >= 0; --t) {
-      W u;
-      if constexpr (use_hilo<T>())
-        u = wfma(wset(zero, nmh), wn, wfma(wset(zero, nml), wn, wmul(y[t], wset(zero, p.cv[1]))));
-      else u = wmul(wset(zero, nmh), wn);
+      const W u = wfma(wset(zero, nmh), wn, wfma(wset(zero, nml), wn, wmul(y[t], wset(zero, p.cv[1]))));
       y[t] = wfma(y[t], wset(zero, p.cv[0]), u);
       wn = y[t];
     }
@@ -317,8 +296,8 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
     }
   } else {
     // rows scaled by 1/b_j; y holds q_j until the right-hand side is formed.
-    // Multipliers as in phase_forward / phase_backward: FP32 applies 1/beta and
-    // the off-diagonal as hi + lo one after the other, FP64 their product.
+    // Multipliers as in phase_forward / phase_backward: 1/beta and the
+    // off-diagonal, each as hi + lo, one after the other.
     const W nh = wset(zero, -p.offh), nl = wset(zero, -p.offl), ks = wset(zero, p.ks);
     const W one = wset(zero, T(1));
     W pr = one, hp = hm1;
@@ -330,11 +309,9 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
       const W m = wmul(nh, bp);
       if (t == 0) {
         y[t] = r;
-      } else if constexpr (use_hilo<T>()) {
+      } else {
         const W v = wfma(bp, y[t - 1], wmul(il[t - 1], y[t - 1]));
         y[t] = wfma(nh, v, wfma(nl, v, r));
-      } else {
-        y[t] = wfma(m, y[t - 1], r);
       }
       pr = wmul(pr, m);
     }
@@ -366,19 +343,15 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
       for (int k = 0; k < w; ++k) cx = wfma(sh.fp[w0 + k][c], cx, sh.fa[w0 + k][c]);
       yin = wfma(pe, cx, yin);
     }
-    // the carry, run through the segment's own multipliers (FP32: hi + lo, as
-    // in the sweep: products of their hi parts alone bias the first node of
+    // the carry, run through the segment's own multipliers (hi + lo, as in the
+    // sweep: products of their hi parts alone bias the first node of
     // every segment by up to 2^-24 of its carry, the same way at every step)
     W q = yin;
 #pragma unroll
     for (int t = 0; t < L; ++t) {
       const W bp = t == 0 ? ibp : ib[t == 0 ? 0 : t - 1];
-      if constexpr (use_hilo<T>()) {
-        const W v = wfma(bp, q, wmul(t == 0 ? ilp : il[t == 0 ? 0 : t - 1], q));
-        q = wfma(nh, v, wmul(nl, v));
-      } else {
-        q = wmul(q, wmul(nh, bp));
-      }
+      const W v = wfma(bp, q, wmul(t == 0 ? ilp : il[t == 0 ? 0 : t - 1], q));
+      q = wfma(nh, v, wmul(nl, v));
       y[t] = wadd(q, y[t]);
     }
     W wn = zero;
@@ -386,12 +359,8 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
 #pragma unroll
     for (int t = L - 1; t >= 0; --t) {
       const W m = wmul(nh, ib[t]);
-      if constexpr (use_hilo<T>()) {
-        const W u = wfma(nh, wn, wfma(nl, wn, y[t]));
-        y[t] = wfma(ib[t], u, wmul(il[t], u));
-      } else {
-        y[t] = wfma(y[t], ib[t], wmul(m, wn));
-      }
+      const W u = wfma(nh, wn, wfma(nl, wn, y[t]));
+      y[t] = wfma(ib[t], u, wmul(il[t], u));
       pr = wmul(pr, m);
       wn = y[t];
     }
@@ -427,12 +396,8 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
     q = win;
 #pragma unroll
     for (int t = L - 1; t >= 0; --t) {
-      if constexpr (use_hilo<T>()) {
-        const W u = wfma(nh, q, wmul(nl, q));
-        q = wfma(ib[t], u, wmul(il[t], u));
-      } else {
-        q = wmul(q, wmul(nh, ib[t]));
-      }
+      const W u = wfma(nh, q, wmul(nl, q));
+      q = wfma(ib[t], u, wmul(il[t], u));
       y[t] = wadd(q, y[t]);
     }
   }
@@ -446,7 +411,7 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
   }
   if (src_t >= 0) source(fp.src.post, fp.src.post_off);
   if (!any) return;
-  const bool both = V == 1 || (a0 && a1);
+  const bool both = a0 && a1;
 #pragma unroll
   for (int t = 0; t < L; ++t) {
     if (full || j0 + t < N) {
@@ -454,7 +419,7 @@ __device__ __forceinline__ void fused_strided_warp(const FusedParams<T>& fp, int
       if (both) {
         *reinterpret_cast<W*>(at_bytes(p.e_out, at)) = E[t];
         *reinterpret_cast<W*>(at_bytes(p.h_out, at)) = H[t];
-      } else if constexpr (V == 2) {
+      } else {
         // one of the two lines is a wall's or past the last one
         const unsigned a1b = at + (a0 ? 0u : (unsigned)sizeof(T));
         *at_bytes(p.e_out, a1b) = a0 ? E[t].x : E[t].y;
@@ -507,7 +472,7 @@ __device__ __forceinline__ void fused_rows_warp(const FusedParams<T>& fp, unsign
     if (mine) {
       load_seg<T, L>(at_bytes(p.nq, at), q);
       load_seg<T, L>(at_bytes(p.nib, at), ib);
-      if constexpr (use_hilo<T>()) load_seg<T, L>(at_bytes(p.nibl, at), il);
+      load_seg<T, L>(at_bytes(p.nibl, at), il);
     }
     row_solve_pn<T, L, LPL>(p, sl, E, H, q, ib, il);
   } else {
