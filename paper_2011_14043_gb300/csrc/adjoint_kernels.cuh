@@ -181,51 +181,81 @@ struct ProbeSet {
   int n;
 };
 
-// mode 0 stashes the E state before the B procedure; mode 1 adds
-// sum (w_B/2)^2 with w_B = E_after_B (before its source) + stash to *acc
-// (forward pass); mode 2 writes w_B to wrec[k] (recomputation, for the
-// reverse pass).
+// A point source of a captured step: coef * table[*step + off] on one sample.
 template <typename T>
-__global__ void probe_energy_kernel(ProbeSet<T> ps, const T* e0, const T* e1, const T* e2, double* stash,
-                                    double* acc, int mode, double* wrec, const long long* slot) {
-  if (wrec && slot) wrec += *slot * ps.n;
+struct AdjSource {
+  T* y;                   // the E component that holds the sample (nullptr: no source)
+  long long at;
+  const double* table;
+  long long len;
+  double coef;
+};
+
+template <typename T>
+__device__ __forceinline__ double adj_source_value(const AdjSource<T>& s, long long n) {
+  return __dmul_rn(s.coef, (n >= 0 && n < s.len) ? s.table[n] : 0.0);
+}
+
+// What a captured forward step does between its procedures, one block: after A
+// the source, then the stash of the probes' E; after B their sum (w_B/2)^2 to
+// *acc (w_B = E after B, before its source, + stash) or w_B itself to the
+// record of this step, then the source of the next procedure and the counters
+// (ctr[0]: step, ctr[1]: record).  One launch each: a small launch in the
+// chain costs the step 2 to 3 us.
+template <typename T>
+__global__ void __launch_bounds__(256) adj_after_a_kernel(ProbeSet<T> ps, const T* e0, const T* e1, const T* e2,
+                                                          double* stash, AdjSource<T> src, const long long* ctr) {
+  const T* e[3] = {e0, e1, e2};
+  if (threadIdx.x == 0 && src.y)
+    src.y[src.at] = (T)__dadd_rn((double)src.y[src.at], adj_source_value(src, ctr[0]));
+  __syncthreads();
+  for (int k = threadIdx.x; k < ps.n; k += blockDim.x) stash[k] = (double)e[ps.comp[k]][ps.at[k]];
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) adj_after_b_kernel(ProbeSet<T> ps, const T* e0, const T* e1, const T* e2,
+                                                          const double* stash, double* acc, double* wrec,
+                                                          AdjSource<T> src, long long* ctr) {
   const T* e[3] = {e0, e1, e2};
   double sum = 0.0;
+  if (wrec) wrec += ctr[1] * ps.n;
   for (int k = threadIdx.x; k < ps.n; k += blockDim.x) {
-    const double v = (double)e[ps.comp[k]][ps.at[k]];
-    if (mode == 0) {
-      stash[k] = v;
-    } else if (mode == 1) {
-      const double w = v + stash[k];
-      sum += 0.25 * w * w;
-    } else {
-      wrec[k] = v + stash[k];
-    }
+    const double w = (double)e[ps.comp[k]][ps.at[k]] + stash[k];
+    if (wrec) wrec[k] = w;
+    else sum += 0.25 * w * w;
   }
-  if (mode != 1) return;
   __shared__ double red[32];
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) acc[0] += v;
-  }
+  if (threadIdx.x >= 32) return;
+  double v = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if (threadIdx.x != 0) return;
+  if (!wrec) acc[0] += v;
+  if (src.y) src.y[src.at] = (T)__dadd_rn((double)src.y[src.at], adj_source_value(src, ctr[0] + 1));
+  ctr[0] += 1;
+  if (wrec) ctr[1] += 1;
 }
 
 // Backward: lam_E += jbar * w_B/2 at the probe samples (w_B recorded by
 // the recomputation).
 template <typename T>
-__global__ void probe_inject_kernel(ProbeSet<T> ps, T* l0, T* l1, T* l2, const double* wrec, double jbar,
-                                    const long long* slot) {
-  if (slot) wrec += *slot * ps.n;
-  T* lam[3] = {l0, l1, l2};
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < ps.n; k += gridDim.x * blockDim.x) {
+__device__ __forceinline__ void probe_inject(const ProbeSet<T>& ps, T* const (&lam)[3], const double* wrec, double jbar,
+                                             int first, int step) {
+  for (int k = first; k < ps.n; k += step) {
     const int c = ps.comp[k];
     const long long at = ps.at[k];
     lam[c][at] = (T)((double)lam[c][at] + jbar * 0.5 * wrec[k]);
   }
+}
+
+template <typename T>
+__global__ void probe_inject_kernel(ProbeSet<T> ps, T* l0, T* l1, T* l2, const double* wrec, double jbar,
+                                    const long long* slot) {
+  T* const lam[3] = {l0, l1, l2};
+  probe_inject(ps, lam, wrec + *slot * ps.n, jbar, (int)(blockIdx.x * blockDim.x + threadIdx.x),
+               (int)(gridDim.x * blockDim.x));
 }
 
 // grad[at] += coef * lam[at] (the eps dependence of a point source).
@@ -234,15 +264,32 @@ __global__ void grad_point_kernel(double* grad, const T* lam, long long at, doub
   if (threadIdx.x == 0 && blockIdx.x == 0) grad[at] += coef * (double)lam[at];
 }
 
-// The same inside a captured step: post = coef * table[*step + off] (rounded
-// on its own, as the host forms it), added as -post / eps_src * lam[at].
+// What a captured reverse step does before a transposed procedure, one block
+// (probe sets of at most a few thousand samples).  Before B (phase 0): the
+// counters step back, the source's eps term, the objective's term; before A
+// (phase 1): the objective's term once more, the source's eps term.
 template <typename T>
-__global__ void grad_point_table_kernel(double* grad, const T* lam, long long at, const double* table, long long len,
-                                        const long long* step, int off, double coef, double eps_src) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    const long long n = *step + off;
-    const double post = __dmul_rn(coef, (n >= 0 && n < len) ? table[n] : 0.0);
-    if (post != 0.0) grad[at] += (-post / eps_src) * (double)lam[at];
+__global__ void __launch_bounds__(256) adj_reverse_kernel(ProbeSet<T> ps, T* l0, T* l1, T* l2, const double* wrec,
+                                                          double jbar, AdjSource<T> src, double* grad, double eps_src,
+                                                          long long* ctr, int phase) {
+  T* const lam[3] = {l0, l1, l2};
+  if (phase == 0) {
+    if (threadIdx.x == 0) {
+      ctr[0] -= 1;
+      ctr[1] -= 1;
+    }
+    __syncthreads();
+  } else {
+    probe_inject(ps, lam, wrec + ctr[1] * ps.n, jbar, (int)threadIdx.x, (int)blockDim.x);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0 && src.y) {
+    const double post = adj_source_value(src, ctr[0] + (phase == 0 ? 1 : 0));
+    if (post != 0.0) grad[src.at] += (-post / eps_src) * (double)src.y[src.at];
+  }
+  if (phase == 0) {
+    __syncthreads();
+    probe_inject(ps, lam, wrec + ctr[1] * ps.n, jbar, (int)threadIdx.x, (int)blockDim.x);
   }
 }
 

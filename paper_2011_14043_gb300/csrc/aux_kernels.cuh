@@ -89,12 +89,11 @@ __global__ void step_counter_kernel(long long* step, long long value, int mode) 
   if (threadIdx.x == 0 && blockIdx.x == 0) *step = mode == 0 ? value : *step + value;
 }
 
-// ctr[0] += a, ctr[1] += b (the step and record counters of a captured
-// reverse-mode step); set: the values themselves.
-__global__ void two_counters_kernel(long long* ctr, long long a, long long b, int set) {
+// The step and record counters of the captured reverse-mode steps.
+__global__ void two_counters_kernel(long long* ctr, long long a, long long b) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
-    ctr[0] = set ? a : ctr[0] + a;
-    ctr[1] = set ? b : ctr[1] + b;
+    ctr[0] = a;
+    ctr[1] = b;
   }
 }
 

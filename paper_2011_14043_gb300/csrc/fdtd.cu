@@ -2149,7 +2149,8 @@ int plane_steps(fdtd_t* h, int64_t nsteps) {
   const void* fn = plane_fn<T>(L);
   const size_t smem =
       ((size_t)(h->nx + 1) * p.RP + (size_t)(h->ny + 1) * p.CP + (size_t)p.R * p.ld + (size_t)p.C * p.ldc) * sizeof(T);
-  CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // (one limit for every grid: handles of other sizes may launch from other threads)
+  CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
   CK(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(fdtd::kPlaneBlocks);
@@ -4528,6 +4529,13 @@ int copy_arrays(fdtd_t* h, void* const* dst, void* const* src, int first, int n)
   return FDTD_OK;
 }
 
+// The source of a captured step on `arr` (the state or the adjoint).
+template <typename T>
+fdtd::AdjSource<T> adj_source(const fdtd_adj_t* a, void* const* arr) {
+  const fdtd_t* h = a->h;
+  return {h->src_comp >= 0 ? (T*)arr[h->src_comp] : nullptr, a->src_at, h->d_srcval, h->srcval_len, 0.5 * h->dt};
+}
+
 // One FADI step of the forward model on `st` (in place), the step index read
 // from the device counter.  objective: add the step's probe energy to *d_acc;
 // otherwise (recomputation) the per-node kernels also write each procedure's
@@ -4549,27 +4557,18 @@ int adj_forward_step(fdtd_adj_t* a, void* const* st, bool objective) {
       return launch_pair<T>(h, g, p);
     });
   };
-  auto source = [&](int off) -> int {
-    if (h->src_comp < 0) return FDTD_OK;
-    h->launches++;
-    fdtd::add_point_table_kernel<T><<<1, 32, 0, h->stream>>>((T*)st[h->src_comp], a->src_at, h->d_srcval,
-                                                             h->srcval_len, a->d_ctr, off, 0.5 * h->dt);
-    CK(cudaGetLastError());
-    return FDTD_OK;
-  };
-  auto probe = [&](int mode) -> int {
-    if (!a->nprobe) return FDTD_OK;
-    h->launches++;
-    fdtd::probe_energy_kernel<T><<<1, 256, 0, h->stream>>>(probe_set<T>(a), (const T*)st[0], (const T*)st[1],
-                                                           (const T*)st[2], a->d_stash, a->d_acc, mode,
-                                                           mode == 2 ? a->d_wrec : nullptr, a->d_ctr + 1);
-    CK(cudaGetLastError());
-    return FDTD_OK;
-  };
+  const T* e[3] = {(const T*)st[0], (const T*)st[1], (const T*)st[2]};
+  const fdtd::AdjSource<T> src = adj_source<T>(a, st);
   int rc;
-  if ((rc = proc(0)) || (rc = source(0)) || (rc = probe(0)) || (rc = proc(1)) || (rc = probe(objective ? 1 : 2)))
-    return rc;
-  return source(1);
+  if ((rc = proc(0))) return rc;
+  h->launches += 2;
+  fdtd::adj_after_a_kernel<T><<<1, 256, 0, h->stream>>>(probe_set<T>(a), e[0], e[1], e[2], a->d_stash, src, a->d_ctr);
+  CK(cudaGetLastError());
+  if ((rc = proc(1))) return rc;
+  fdtd::adj_after_b_kernel<T><<<1, 256, 0, h->stream>>>(probe_set<T>(a), e[0], e[1], e[2], a->d_stash, a->d_acc,
+                                                        objective ? nullptr : a->d_wrec, src, a->d_ctr);
+  CK(cudaGetLastError());
+  return FDTD_OK;
 }
 
 // The three adjoint pair launches of procedure `slot` on lam (in place).
@@ -4659,31 +4658,33 @@ int adj_reverse_step(fdtd_adj_t* a, double jbar) {
     ra[c] = arr_at(a->tape, c, h);
     rb[c] = arr_at(a->tape, 3 + c, h);
   }
-  auto point = [&](int off) -> int {
-    if (h->src_comp < 0) return FDTD_OK;
-    h->launches++;
-    fdtd::grad_point_table_kernel<T><<<1, 32, 0, h->stream>>>(a->grad[h->src_comp], (const T*)a->lam[h->src_comp],
-                                                              a->src_at, h->d_srcval, h->srcval_len, a->d_ctr, off,
-                                                              0.5 * h->dt, a->eps_src);
-    CK(cudaGetLastError());
-    return FDTD_OK;
-  };
-  int rc;
   // B procedure: the objective's w_B term enters w-bar; with it added to the E
   // adjoint before the transposed solve, the output E-bar = q y - E-bar' needs
-  // it added back once more
-  if ((rc = point(1)) || (rc = adj_inject<T>(a, jbar)) || (rc = adj_procedure<T>(a, 1, rb, -1, true)) ||
-      (rc = adj_inject<T>(a, jbar)))
-    return rc;
-  // A procedure
-  if ((rc = point(0))) return rc;
-  return adj_procedure<T>(a, 0, ra, -1, true);
+  // it added back once more, before the A procedure
+  double* grad = h->src_comp >= 0 ? a->grad[h->src_comp] : nullptr;
+  int rc = FDTD_OK;
+  for (int phase = 0; phase < 2 && !rc; ++phase) {
+    // (large probe sets: the injection by many blocks, the rest without it)
+    fdtd::ProbeSet<T> ps = probe_set<T>(a);
+    const bool many = ps.n > 4096;
+    if (many) ps.n = 0;
+    if (many && phase == 1) rc = adj_inject<T>(a, jbar);
+    if (rc) return rc;
+    h->launches++;
+    fdtd::adj_reverse_kernel<T><<<1, 256, 0, h->stream>>>(ps, (T*)a->lam[0], (T*)a->lam[1], (T*)a->lam[2], a->d_wrec,
+                                                          jbar, adj_source<T>(a, a->lam), grad, a->eps_src, a->d_ctr,
+                                                          phase);
+    CK(cudaGetLastError());
+    if (many && phase == 0 && (rc = adj_inject<T>(a, jbar))) return rc;
+    rc = phase == 0 ? adj_procedure<T>(a, 1, rb, -1, true) : adj_procedure<T>(a, 0, ra, -1, true);
+  }
+  return rc;
 }
 
 // Capture one step on the handle's stream (the branch-capable stream: adj_on
-// points it there); step and record counters move by ds and dr after it.
+// points it there), which moves the device counters itself.
 template <typename F>
-int adj_capture(fdtd_adj_t* a, cudaGraphExec_t* exec, long long* kernels, int ds, int dr, F&& step) {
+int adj_capture(fdtd_adj_t* a, cudaGraphExec_t* exec, long long* kernels, F&& step) {
   fdtd_t* h = a->h;
   const long long before = h->launches;
   const bool timing = h->timing;
@@ -4691,11 +4692,6 @@ int adj_capture(fdtd_adj_t* a, cudaGraphExec_t* exec, long long* kernels, int ds
   CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
   int rc = step();
   h->timing = timing;
-  if (!rc) {
-    fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, ds, dr, 0);
-    h->launches++;
-    if (cudaGetLastError() != cudaSuccess) rc = FDTD_ERR_CUDA;
-  }
   cudaGraph_t graph = nullptr;
   const cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
   *kernels = h->launches - before;
@@ -4818,9 +4814,9 @@ int adj_forward_t(fdtd_adj_t* a) {
   CK(cudaMemsetAsync(a->d_acc, 0, sizeof(double), h->stream));
   rc = adj_on_replay_stream(h, [&]() -> int {
     if (!a->g_fwd)
-      if (int e = adj_capture(a, &a->g_fwd, &a->k_fwd, 1, 0, [&]() { return adj_forward_step<T>(a, h->f, true); }))
+      if (int e = adj_capture(a, &a->g_fwd, &a->k_fwd, [&]() { return adj_forward_step<T>(a, h->f, true); }))
         return e;
-    fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, 0, 0, 1);
+    fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, 0, 0);
     for (long long n = 0; n < a->nsteps; ++n) {
       if (n % a->every == 0) {
         void* dst[6];
@@ -4849,7 +4845,7 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
   for (int c = 0; c < 3; ++c) CK(cudaMemsetAsync(a->grad[c], 0, sizeof(double) * h->count, h->stream));
   rc = adj_on_replay_stream(h, [&]() -> int {
     if (!a->g_rec)
-      if (int e = adj_capture(a, &a->g_rec, &a->k_rec, 1, 1, [&]() { return adj_forward_step<T>(a, a->work, false); }))
+      if (int e = adj_capture(a, &a->g_rec, &a->k_rec, [&]() { return adj_forward_step<T>(a, a->work, false); }))
         return e;
     if (a->g_rev && a->g_jbar != jbar) {
       CK(cudaStreamSynchronize(h->stream));
@@ -4857,7 +4853,7 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
       a->g_rev = nullptr;
     }
     if (!a->g_rev)
-      if (int e = adj_capture(a, &a->g_rev, &a->k_rev, -1, -1, [&]() { return adj_reverse_step<T>(a, jbar); }))
+      if (int e = adj_capture(a, &a->g_rev, &a->k_rev, [&]() { return adj_reverse_step<T>(a, jbar); }))
         return e;
     a->g_jbar = jbar;
     for (int seg = a->nseg - 1; seg >= 0; --seg) {
@@ -4866,11 +4862,10 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
       void* src[6];
       for (int c = 0; c < 6; ++c) src[c] = arr_at(a->ckpt, (long long)seg * 6 + c, h);
       if (int e = copy_arrays(h, a->work, src, 0, 6)) return e;
-      fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, n0, 0, 1);
+      fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, n0, 0);
       for (long long n = n0; n < n1; ++n) CK(cudaGraphLaunch(a->g_rec, h->stream));
-      fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, -1, -1, 0);
       for (long long n = n0; n < n1; ++n) CK(cudaGraphLaunch(a->g_rev, h->stream));
-      h->launches += (n1 - n0) * (a->k_rec + a->k_rev) + 2;
+      h->launches += (n1 - n0) * (a->k_rec + a->k_rev) + 1;
     }
     return FDTD_OK;
   });
