@@ -737,11 +737,6 @@ void set_scan(fdtd::PairParams<T>& p, const PairCoef& c, int L) {
     p.sc[0][k] = p.sc[0][k - 1] * p.sc[0][k - 1];
     p.sc[1][k] = T(0);
   }
-  // an x line's scan stops where the product is zero: a carry that it leaves
-  // out would have been zero too (the same bits, also in empty regions)
-  p.nscan = 32;
-  for (int k = 4; k >= 0; --k)
-    if (p.sc[0][k] == T(0)) p.nscan = 1 << k;
   p.kx = 1;
   while (p.kx < 8 && std::pow(std::fabs(c.mc), 32.0 * p.kx) >= least) ++p.kx;
 }

@@ -119,10 +119,9 @@ struct PairParams {
   int kg_len;            // the wall correction is zero from this node on (a multiple of
                          // the segment length)
   // uniform media, x lines: carry products (-m)^(L d) of d = 1, 2, 4, 8, 16 segments
-  // (hi, lo); nscan: the first d whose product is zero (the scan stops there);
-  // kx: runs of 32 nodes until the product is below 2^-50 (the y/z tiles' carries over warps)
+  // (hi, lo); kx: runs of 32 nodes until the product is below 2^-50 (the y/z tiles' carries over warps)
   T sc[2][5];
-  int nscan, kx;
+  int kx;
   T* tmp4;               // fourth-order differences: field-shaped scratch of the line solve
   T c2_4;                // fourth-order difference weight -1/24 in the field precision
   int jc4, je4;          // fourth-order differences: the factor rows of nodes jc4..je4 all
@@ -1345,7 +1344,7 @@ __device__ __forceinline__ void fma_pair(T& r0, T& r1, T a0, T a1, T b0, T b1, T
 //
 // LPL lanes of a warp hold one line (lane sl its nodes [sl L, sl L + L)).  A
 // segment's carry product is the constant (-m)^L, so the scans shuffle the
-// carries alone and stop after the first distance whose product underflows.  What bounds these lines is instruction issue: the elementwise
+// carries alone.  What bounds these lines is instruction issue: the elementwise
 // parts run as packed FMAs on neighbouring nodes.
 // On return E, H hold the new values.
 template <typename T, int L, int LPL>
@@ -1371,7 +1370,6 @@ __device__ __forceinline__ void row_solve_wall(const PairParams<T>& p, int sl, T
   T a = y[L - 1];
 #pragma unroll
   for (int d = 1, k = 0; d < LPL; d <<= 1, ++k) {
-    if (d >= p.nscan) break;
     const T up = __shfl_up_sync(FULL, a, d, LPL);
     const T an = d == 1 ? fma2(HiLo<T>{p.sc[0][0], p.sc[1][0]}, up, a) : fma(p.sc[0][k], up, a);
     a = sl >= d ? an : a;
@@ -1403,7 +1401,6 @@ __device__ __forceinline__ void row_solve_wall(const PairParams<T>& p, int sl, T
   T b = y[0];
 #pragma unroll
   for (int d = 1, k = 0; d < LPL; d <<= 1, ++k) {
-    if (d >= p.nscan) break;
     const T dn = __shfl_down_sync(FULL, b, d, LPL);
     const T bn = d == 1 ? fma2(HiLo<T>{p.sc[0][0], p.sc[1][0]}, dn, b) : fma(p.sc[0][k], dn, b);
     b = sl + d < LPL ? bn : b;
