@@ -96,9 +96,11 @@ typedef enum { FDTD_EX = 0, FDTD_EY = 1, FDTD_EZ = 2, FDTD_HX = 3, FDTD_HY = 4, 
  * least 32768 lines) take the segmented solve instead of one thread per line
  * walking the Thomas recurrences (equal to rounding; the default needs a
  * scratch of three field arrays, allocated at the first fdtd_step); tune[1]
- * bit 11 set: lines along x of exactly 32 L cells (FP32, homogeneous media,
- * wall-corrected) keep the kernel with end-of-line masks instead of the one
- * without them (the same results). */
+ * bit 11 is accepted and has no effect (it chose between two x-line kernels
+ * with the same results).  With tune[0] = 0 and bits 0, 2 and 7 clear, FP32
+ * grids of moderate size run each procedure as one launch, and small 2-D
+ * grids every step of a call as one launch (bits 3, 4 and 10 clear too);
+ * these agree with the other kernels to rounding. */
 typedef struct {
   int32_t nx, ny, nz;        /* cells per axis: 2 <= nx <= 1024, 2 <= ny, 1 <= nz; lines
                                 along y and z are solved with at most 32 segments of
@@ -286,8 +288,9 @@ int fdtd_energy_noalloc(int nx, int ny, int nz, double dx, double dy, double dz,
  * launch-shape group (line direction, lanes, segment length and count)
  * covering every grid of the batch; the groups of one procedure run
  * concurrently on parallel graph branches, and one step of the whole batch
- * is captured once as a CUDA graph and replayed.  Every grid runs exactly the arithmetic of its own handle's
- * fdtd_step.  Handles must share scheme, precision and stream, be distinct,
+ * is captured once as a CUDA graph and replayed.  Every grid runs the arithmetic of its own handle's
+ * fdtd_step (bit for bit under a fixed launch shape and the handle's tune[0]; else to
+ * rounding).  Handles must share scheme, precision and stream, be distinct,
  * and have no source or probe (FDTD_ERR_UNSUPPORTED); they stay owned by
  * the caller, stay usable for set/get/energy, and must outlive the batch.
  * stream: the handles' stream.  Errors as for fdtd_step. */
@@ -322,7 +325,9 @@ int fdtd_batch_set_config(fdtd_batch_t* b, const int32_t* cfg);
  * lines) from a counter that a memset zeroes before the launch, until the
  * list is exhausted; both are captured in the step graph.  mode -1 (default): the first step times
  * both on the batch's own data (one-step graph replays writing scratch) and
- * keeps the faster (the persistent launches also with both y and z lines
+ * keeps the faster (mode 0 also as one fused launch per procedure and media
+ * kind, for FP32 grids of sides up to 256 when the shapes are not fixed;
+ * the persistent launches also with both y and z lines
  * at (16, 8) and (16, 16), a persistent win bringing its shape along);
  * cached like the shapes.  Persistent launches run blocks of 256 threads
  * and need per-node media on every grid, y and z lines of one shape with a
