@@ -4489,9 +4489,17 @@ struct fdtd_adj_s {
   double* grad[3] = {nullptr, nullptr, nullptr};
   void* u0h[3] = {nullptr, nullptr, nullptr};   // initial physical H
   AdjCfg cfg[2];
+  // the source of the forward run, taken over when it starts: the reverse pass
+  // (which may be repeated, from captured steps) recomputes that run whatever
+  // source the handle has by then
+  int src_comp = -1;
   long long src_at = -1;
   double eps_src = 0;
-  void* slab = nullptr;     // all of the above
+  double src_first = 0;     // its value at step 0
+  double* d_src = nullptr;  // its values per step, src_cap elements of the slab
+  long long src_len = 0, src_cap = 0;
+  double* d_src_own = nullptr;  // ... or an allocation of their own, where they are more
+  void* slab = nullptr;     // all of the above but d_src_own
   long long* d_ctr = nullptr;  // [0]: step, [1]: record of the segment
   // captured steps: forward with the objective, recomputation with records,
   // reverse (scaled by jbar)
@@ -4527,8 +4535,31 @@ int copy_arrays(fdtd_t* h, void* const* dst, void* const* src, int first, int n)
 // The source of a captured step on `arr` (the state or the adjoint).
 template <typename T>
 fdtd::AdjSource<T> adj_source(const fdtd_adj_t* a, void* const* arr) {
-  const fdtd_t* h = a->h;
-  return {h->src_comp >= 0 ? (T*)arr[h->src_comp] : nullptr, a->src_at, h->d_srcval, h->srcval_len, 0.5 * h->dt};
+  return {a->src_comp >= 0 ? (T*)arr[a->src_comp] : nullptr, a->src_at, a->d_src, a->src_len, 0.5 * a->h->dt};
+}
+
+// Take over the handle's source (component, sample, values, eps there).
+int adj_take_source(fdtd_adj_t* a) {
+  fdtd_t* h = a->h;
+  a->src_comp = h->src_comp;
+  if (a->src_comp < 0) return FDTD_OK;
+  a->src_at = elem_index(h, h->src_i, h->src_j, h->src_k);
+  a->src_first = source_value(h, 0);
+  a->src_len = (long long)h->src_current.size();
+  if (a->src_len > a->src_cap) {
+    if (a->d_src_own) CK(cudaFree(a->d_src_own));
+    a->d_src_own = nullptr;
+    CK(dev_malloc((void**)&a->d_src_own, sizeof(double) * (size_t)a->src_len));
+    a->d_src = a->d_src_own;
+  }
+  std::vector<double> v((size_t)a->src_len);
+  for (long long n = 0; n < a->src_len; ++n) v[(size_t)n] = source_value(h, n);
+  double er = 1.0;
+  CK(cudaMemcpyAsync(a->d_src, v.data(), sizeof(double) * v.size(), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemcpyAsync(&er, h->eps_node[a->src_comp] + a->src_at, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  a->eps_src = kEps0 * er;
+  return FDTD_OK;
 }
 
 // One FADI step of the forward model on `st` (in place), the step index read
@@ -4624,9 +4655,9 @@ int adj_procedure(fdtd_adj_t* a, int slot, void* const* rec, int only_axis = -1,
 template <typename T>
 int adj_point_term(fdtd_adj_t* a, double post) {
   fdtd_t* h = a->h;
-  if (h->src_comp < 0 || post == 0.0) return FDTD_OK;
+  if (a->src_comp < 0 || post == 0.0) return FDTD_OK;
   // post = (h/2) f with f proportional to 1/eps at the source sample
-  fdtd::grad_point_kernel<T><<<1, 32, 0, h->stream>>>(a->grad[h->src_comp], (const T*)a->lam[h->src_comp],
+  fdtd::grad_point_kernel<T><<<1, 32, 0, h->stream>>>(a->grad[a->src_comp], (const T*)a->lam[a->src_comp],
                                                       a->src_at, -post / a->eps_src);
   CK(cudaGetLastError());
   return FDTD_OK;
@@ -4656,7 +4687,7 @@ int adj_reverse_step(fdtd_adj_t* a, double jbar) {
   // B procedure: the objective's w_B term enters w-bar; with it added to the E
   // adjoint before the transposed solve, the output E-bar = q y - E-bar' needs
   // it added back once more, before the A procedure
-  double* grad = h->src_comp >= 0 ? a->grad[h->src_comp] : nullptr;
+  double* grad = a->src_comp >= 0 ? a->grad[a->src_comp] : nullptr;
   int rc = FDTD_OK;
   for (int phase = 0; phase < 2 && !rc; ++phase) {
     // (large probe sets: the injection by many blocks, the rest without it)
@@ -4801,6 +4832,7 @@ int adj_forward_t(fdtd_adj_t* a) {
   int rc;
   for (int c = 0; c < 3; ++c)
     CK(cudaMemcpyAsync(a->u0h[c], h->f[3 + c], (size_t)h->count * h->esize, cudaMemcpyDeviceToDevice, h->stream));
+  if ((rc = adj_take_source(a))) return rc;
   if ((rc = scheme_init(h))) return rc;
   // launch shapes: forward (as fdtd_step would choose them) and adjoint
   if (!h->shape_tuned && h->desc.tune[0] == 0 && (rc = single_tune(h))) return rc;
@@ -4866,7 +4898,7 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
   });
   if (rc) return rc;
   // input initialization v0 = u0 + (dt/2) B u0 + (dt/2) f
-  if ((rc = adj_point_term<T>(a, 0.5 * h->dt * source_value(h, 0)))) return rc;
+  if ((rc = adj_point_term<T>(a, 0.5 * h->dt * a->src_first))) return rc;
   const ProcCoef& P = h->proc[1];
   for (int q = 0; q < 3; ++q) {
     const PairGeom& g = h->geom[P.op][q];
@@ -4893,6 +4925,7 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
 void adj_free(fdtd_adj_t* a) {
   for (cudaGraphExec_t g : {a->g_fwd, a->g_rec, a->g_rev})
     if (g) cudaGraphExecDestroy(g);
+  if (a->d_src_own) cudaFree(a->d_src_own);
   if (a->slab) cudaFree(a->slab);
 }
 
@@ -4938,16 +4971,7 @@ int fdtd_adj_create(fdtd_t* h, const int32_t block[6], int64_t nsteps, int32_t c
         }
   }
   a->nprobe = (int)at.size();
-  if (h->src_comp >= 0) {
-    a->src_at = elem_index(h, h->src_i, h->src_j, h->src_k);
-    double er = 1.0;
-    if (cudaMemcpy(&er, h->eps_node[h->src_comp] + a->src_at, sizeof(double), cudaMemcpyDeviceToHost) !=
-        cudaSuccess) {
-      delete a;
-      return FDTD_ERR_CUDA;
-    }
-    a->eps_src = kEps0 * er;
-  }
+  a->src_cap = (long long)h->src_current.size();
   const size_t arr = (size_t)h->count * h->esize;
   // one allocation for everything (26 of them, and their releases, took 2.2 ms
   // of a 17 ms gradient evaluation), each part at a multiple of 256 bytes
@@ -4961,6 +4985,7 @@ int fdtd_adj_create(fdtd_t* h, const int32_t block[6], int64_t nsteps, int32_t c
   part((void**)&a->d_stash, sizeof(double) * std::max<size_t>(1, at.size()));
   part((void**)&a->d_acc, sizeof(double));
   part((void**)&a->d_ctr, 2 * sizeof(long long));
+  part((void**)&a->d_src, sizeof(double) * std::max<size_t>(1, h->src_current.size()));
   part((void**)&a->d_cell, sizeof(double) * (size_t)h->nx * h->ny * h->nz);
   part(&a->ckpt, arr * 6 * (size_t)a->nseg);
   part(&a->tape, arr * 3 * (size_t)(2 * checkpoint_every));
