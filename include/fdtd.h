@@ -366,7 +366,8 @@ int fdtd_batch_get_mode(const fdtd_batch_t* b, int32_t* persistent, double step_
  *   outlive it.
  * fdtd_adj_forward: runs the nsteps steps on h (h advances; its fields are
  *   afterwards those of step nsteps) and returns J (FP64 sum).  Once only.
- *   The source is the one that h has now; the backward pass keeps to it, also
+ *   FDTD_ERR_UNSUPPORTED when h has been given media since that fdtd_adj_create
+ *   refuses.  The source is the one that h has now; the backward pass keeps to it, also
  *   when h is given another one later.
  * fdtd_adj_backward: grad_eps_r[nz][ny][nx] (double; host or device) =
  *   jbar * dJ/d eps_r per cell.  Requires the forward pass; may be repeated.

@@ -4922,6 +4922,11 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
   return FDTD_OK;
 }
 
+// What the transposed kernels are built for: eps per node, uniform mu, no loss.
+bool adj_media_ok(const fdtd_t* h) {
+  return h->scheme == FDTD_FADI && h->per_node && !h->mu_var && !h->lossy && h->order == 2;
+}
+
 void adj_free(fdtd_adj_t* a) {
   for (cudaGraphExec_t g : {a->g_fwd, a->g_rec, a->g_rev})
     if (g) cudaGraphExecDestroy(g);
@@ -4938,8 +4943,7 @@ int fdtd_adj_create(fdtd_t* h, const int32_t block[6], int64_t nsteps, int32_t c
   if (!h || !block || !out || nsteps < 1 || checkpoint_every < 1) return FDTD_ERR_INVALID_ARG;
   *out = nullptr;
   if (h->poisoned) return FDTD_ERR_STATE;
-  if (h->scheme != FDTD_FADI || !h->per_node || h->mu_var || h->lossy || h->order != 2)
-    return FDTD_ERR_UNSUPPORTED;
+  if (!adj_media_ok(h)) return FDTD_ERR_UNSUPPORTED;
   if (!h->pending_init || h->steps != 0) return FDTD_ERR_STATE;
   if (h->nprobes > 0) return FDTD_ERR_UNSUPPORTED;
   const int i0 = block[0], i1 = block[1], j0 = block[2], j1 = block[3], k0 = block[4], k1 = block[5];
@@ -5036,6 +5040,8 @@ int fdtd_adj_forward(fdtd_adj_t* a, double* objective) {
   fdtd_t* h = a->h;
   if (h->poisoned) return FDTD_ERR_STATE;
   if (a->forward_done || !h->pending_init || h->steps != 0) return FDTD_ERR_STATE;
+  // media set since the context was created
+  if (!adj_media_ok(h)) return FDTD_ERR_UNSUPPORTED;
   NvtxScope range("adjoint forward");
   int rc = h->prec == FDTD_F64 ? adj_forward_t<double>(a) : adj_forward_t<float>(a);
   if (rc) return rc;

@@ -1,4 +1,4 @@
-"""Reverse mode and the handle's source: the reverse pass belongs to the run
+"""Reverse mode and what its handle is given around it: the reverse pass belongs to the run
 that fdtd_adj_forward made, whatever source the handle is given before,
 between and after the passes; probe sets larger than one block takes."""
 import numpy as np
@@ -98,3 +98,37 @@ def test_probe_sets_of_more_than_4096_samples(prec):
     run.close()
     assert abs(J / J_ref - 1.0) <= (1e-12 if prec == "f64" else 1e-4)
     assert np.linalg.norm(got - g_ref) <= (1e-6 if prec == "f64" else 1e-3) * np.linalg.norm(g_ref)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_media_set_after_the_context(prec):
+    """Media that fdtd_adj_create refuses are refused by the forward pass too
+    when they come after it (uniform eps has no per-node arrays to read);
+    another per-node eps is taken."""
+    import ctypes
+    from paper_2011_14043_gb300 import Simulation
+    from paper_2011_14043_gb300._lib import lib
+    L = lib()
+    one = np.ones_like(EPS)
+    mu = one.copy()
+    mu[:, :, :5] = 2.0
+    blk = (ctypes.c_int32 * 6)(*BLOCK)
+    for later, want in (((one, None, None), -6), ((EPS, mu, None), -6), ((EPS, None, 1e-3 * one), -6),
+                        ((EPS, None, None), 0)):
+        sim = Simulation(*N, 1e-3, scheme="fadi", precision=prec, dt=DT)
+        sim.set_material(0.5 + EPS)
+        sim.set_fields(U0)
+        sim.set_source(*SOURCE)
+        h, J = ctypes.c_void_p(), ctypes.c_double()
+        assert L.fdtd_adj_create(sim._h, blk, STEPS, EVERY, ctypes.byref(h)) == 0
+        sim.set_material(*later)
+        assert L.fdtd_adj_forward(h, ctypes.byref(J)) == want
+        if want == 0:
+            g = np.empty_like(EPS)
+            assert L.fdtd_adj_backward(h, 1.0, g.ctypes.data_as(ctypes.c_void_p), 0) == 0
+            same = start(prec, SOURCE)
+            assert same.forward() == J.value
+            assert np.array_equal(gradient(same), g)
+            same.close()
+        L.fdtd_adj_destroy(h)
+        sim.close()
