@@ -179,7 +179,8 @@ int fdtd_set_field(fdtd_t* h, int comp, const void* data, int on_device);
 /* Read one physical field component at the current time.  FADI applies the
  * output relation u = u~/2 (Eq. 9) in the equivalent state form
  * u = (I + dt/2 B)^{-1} (v - pending source); FLOD2 applies its output
- * processing (Eq. 23); FLOD/FSS return the state. */
+ * processing (Eq. 23); FLOD/FSS return the state.  FDTD_ERR_TIMEOUT where a
+ * kernel's bounded wait gave up in the steps or in that processing. */
 int fdtd_get_field(fdtd_t* h, int comp, void* out, int on_device);
 
 /* Raw scheme state (FADI: auxiliary v of Eq. 8; FLOD2: u^{n+1/4} of Eq. 21;
@@ -384,6 +385,11 @@ int fdtd_adj_destroy(fdtd_adj_t* a);
  * next one) fails as an out-of-memory would, without calling CUDA; n < 0
  * disarms it.  For exercising the error and clean-up paths; process-wide. */
 int fdtd_debug_fail_alloc(int64_t n);
+
+/* Test hook: the n-th launch of a kernel with bounded waits from now on (0 =
+ * the next one) sets its handle's device flag as a wait that gave up would
+ * (the kernel itself runs to its end); n < 0 disarms it.  Process-wide. */
+int fdtd_debug_fail_wait(int64_t n);
 
 /* Self-test of the bounded device waits (failure detection without a GPU
  * fault).  Every spin-wait in the kernels (the TMA kernels' mbarrier waits)

@@ -214,19 +214,25 @@ struct NvtxScope {
 // out-of-memory would, without calling CUDA, to exercise the error paths.
 std::atomic<long long> g_fail_alloc_in{-1};
 
+// Count an armed hook down; true when this is the event it was armed for.
+bool hook_due(std::atomic<long long>& in) {
+  long long k = in.load();
+  while (k >= 0)
+    if (in.compare_exchange_weak(k, k == 0 ? -1 : k - 1)) return k == 0;
+  return false;
+}
+
 cudaError_t dev_malloc(void** p, size_t n) {
-  long long k = g_fail_alloc_in.load();
-  while (k >= 0) {
-    if (g_fail_alloc_in.compare_exchange_weak(k, k == 0 ? -1 : k - 1)) {
-      if (k == 0) {
-        *p = nullptr;
-        return cudaErrorMemoryAllocation;
-      }
-      break;
-    }
+  if (hook_due(g_fail_alloc_in)) {
+    *p = nullptr;
+    return cudaErrorMemoryAllocation;
   }
   return cudaMalloc(p, n);
 }
+
+// The same for the kernels with bounded waits (fdtd_debug_fail_wait): the n-th
+// next launch sets the handle's flag as a wait that gave up would.
+std::atomic<long long> g_fail_wait_in{-1};
 
 int cuda_fail(fdtd_t* h, cudaError_t e) {
   if (e == cudaSuccess) return FDTD_OK;
@@ -991,6 +997,13 @@ cudaError_t ensure_tma_attr() {
   return e;
 }
 
+// A kernel with bounded waits has been launched on the handle's stream.
+int bounded_waits_launched(fdtd_t* h) {
+  h->waits = h->err_due = true;
+  if (hook_due(g_fail_wait_in)) CK(cudaMemsetAsync(h->d_err, 1, sizeof(int), h->stream));
+  return FDTD_OK;
+}
+
 template <typename T, int LANES, int MINB, int NST>
 int launch_strided_tma(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
   constexpr int L = tma_L<T>();
@@ -1016,9 +1029,8 @@ int launch_strided_tma(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& 
                  : fdtd::proc_strided_tma_kernel<T, LANES, L, MINB, NST>;
   CK((ensure_tma_attr<T, LANES, MINB, NST>()));
   const int grid = std::min(q.n_tiles, MINB * h->num_sms);
-  h->waits = h->err_due = true;
   kern<<<grid, P * LANES, smem, h->stream>>>(*tE, *tH, p, q);
-  return FDTD_OK;
+  return bounded_waits_launched(h);
 }
 
 // TMA-fed x lines (proc_rows_tma_kernel), on request (tune[1] bit 4): FP32
@@ -1082,14 +1094,13 @@ int launch_rows_tma(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<float>&
   q.tpp = (g.n_o + kRowsR - 1) / kRowsR;
   q.n_tiles = q.tpp * g.n_o2;
   CK(ensure_rows_tma_attr());
-  h->waits = h->err_due = true;
   switch ((h->desc.tune[1] >> 5) & 3) {
     case 1: launch_rows_tma_v<2, 4>(h, tE, tH, p, q); break;
     case 2: launch_rows_tma_v<4, 3>(h, tE, tH, p, q); break;
     case 3: launch_rows_tma_v<2, 6>(h, tE, tH, p, q); break;
     default: launch_rows_tma_v<3, 4>(h, tE, tH, p, q); break;
   }
-  return FDTD_OK;
+  return bounded_waits_launched(h);
 }
 
 int take_event(fdtd_t* h, int* idx) {
@@ -2316,6 +2327,26 @@ int check_device_flag(fdtd_t* h) {
   return v ? FDTD_ERR_TIMEOUT : FDTD_OK;
 }
 
+// The flag, where a kernel that can set it has run since it was last read, or
+// always (a read into host memory, which waits for the stream anyway).
+int read_flag(fdtd_t* h, bool always) {
+#ifdef FDTD_BOUNDS
+  always = true;
+#endif
+  return always || h->err_due ? check_device_flag(h) : FDTD_OK;
+}
+
+// The physical field into scratch, and the flag read after it: the output solve
+// of FP32 grids takes kernels with bounded waits, and where one gave up, tiles of
+// scratch hold an earlier field.  (One wait for the stream per solve: the
+// flag is not due again for the components that follow.)
+int physical_checked(fdtd_t* h, bool always) {
+  int rc = physical_to_scratch(h);
+  if (!rc) rc = read_flag(h, always);
+  if (rc) h->output_valid = false;
+  return rc;
+}
+
 // f_E = -I / (A eps) at the source sample (A = the sample's dual-face area).
 int refresh_src_scale(fdtd_t* h) {
   if (h->src_comp < 0) {
@@ -2558,6 +2589,11 @@ extern "C" {
 
 int fdtd_debug_fail_alloc(int64_t n) {
   g_fail_alloc_in.store(n < 0 ? -1 : (long long)n);
+  return FDTD_OK;
+}
+
+int fdtd_debug_fail_wait(int64_t n) {
+  g_fail_wait_in.store(n < 0 ? -1 : (long long)n);
   return FDTD_OK;
 }
 
@@ -2906,7 +2942,7 @@ int fdtd_set_field(fdtd_t* h, int comp, const void* data, int on_device) {
   int rc;
   if ((h->scheme == FDTD_FADI || h->scheme == FDTD_FLOD2) && !h->pending_init) {
     // back to the physical field, then re-initialise on the next step
-    if ((rc = physical_to_scratch(h))) return rc;
+    if ((rc = physical_checked(h, false))) return rc;
     for (int c = 0; c < 6; ++c) std::swap(h->f[c], h->scratch[c]);
     h->pending_init = true;
   }
@@ -2920,16 +2956,12 @@ int fdtd_set_field(fdtd_t* h, int comp, const void* data, int on_device) {
 int fdtd_get_field(fdtd_t* h, int comp, void* out, int on_device) {
   if (!h || !out || check_comp(comp)) return FDTD_ERR_INVALID_ARG;
   if (h->poisoned) return FDTD_ERR_STATE;
-  // a read into device memory waits for the flag only when a kernel that can
-  // set it has run since it was last read
-#ifndef FDTD_BOUNDS
-  if (!on_device || h->err_due)
-#endif
-    if (int rc0 = check_device_flag(h)) return rc0;
-  if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS || h->pending_init)
+  int rc;
+  if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS || h->pending_init) {
+    if ((rc = read_flag(h, !on_device))) return rc;
     return copy_component(h, comp, h->f[comp], out, on_device);
-  int rc = physical_to_scratch(h);
-  if (rc) return rc;
+  }
+  if ((rc = physical_checked(h, !on_device))) return rc;
   return copy_component(h, comp, h->scratch[comp], out, on_device);
 }
 
@@ -3050,7 +3082,7 @@ int fdtd_energy(fdtd_t* h, double out[2]) {
   if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS) {
     out[0] = out[1];
   } else {
-    if ((rc = physical_to_scratch(h))) return rc;
+    if ((rc = physical_checked(h, false))) return rc;
     if ((rc = energy(h, h->scratch, &out[0]))) return rc;
   }
   if (!std::isfinite(out[0]) || !std::isfinite(out[1])) return FDTD_ERR_UNSTABLE;
