@@ -24,6 +24,7 @@
 #include <cstring>
 #include <limits>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <new>
@@ -130,8 +131,10 @@ struct fdtd_s {
   // the second-difference part does not)
   ProcCoef proc[5];
   bool per_node = false;
-  bool adjoint = false;       // a reverse-mode context was created on this handle
-  bool batched = false;       // the handle was put into a batch (which steps it by its own kernels)
+  int adjoints = 0;           // reverse-mode contexts on this handle
+  // batches that hold this handle (each has a share in the count, and may be
+  // destroyed after the handle)
+  std::shared_ptr<std::atomic<int>> batches = std::make_shared<std::atomic<int>>(0);
   bool shape_tuned = false;   // per-node y/z launch shapes chosen by timing
   double eps_r = 1.0, mu_r = 1.0;          // uniform media
   double* eps_node[3] = {nullptr, nullptr, nullptr};  // per-node eps_r at E samples (device)
@@ -186,6 +189,7 @@ struct fdtd_s {
   cudaGraphExec_t g_exec = nullptr;     // one step
   cudaGraphExec_t g_run_exec = nullptr; // kStepRun steps (fused procedures)
   std::vector<const void*> g_bound;     // state pointers the graph was captured with
+  bool g_fused = false;                 // ... and whether its procedures are fused
   long long g_kernels = 0, g_run_kernels = 0;  // kernels per replay
   double* d_srcval = nullptr;           // f_E(n) = src_scale * I(n), n < src_current.size()
   long long srcval_len = 0;
@@ -1359,9 +1363,9 @@ int launch_pair(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
 // FP32 fields, second-order differences, uniform mu, sides of at most 256
 // cells (8 warps of 4 segments of 8 nodes hold a line), arrays of less than
 // 2^32 bytes.  The launch-shape overrides that name another kernel keep it,
-// the reverse pass the kernels whose records and rounding it replays, a
-// batch's handles the kernels that the batch steps them by, and handles with
-// probes the kernels whose rounding their FP64 series have always shown.
+// the reverse pass (while its context lives) the kernels whose records and
+// rounding it replays, a batch's handles (while it lives) the kernels that the
+// batch steps them by, and handles with probes the kernels whose rounding their FP64 series have always shown.
 //
 // The line: a procedure that moves at most 256 MB (24 B per cell), about twice
 // the L2 cache, or 150 MB with per-node media (60 B per cell).  FADI steps,
@@ -1388,7 +1392,7 @@ bool fused_shape_ok(const fdtd_t* h) {
 // off either way, 9e-5 apart).  Such runs keep the kernels they had.
 bool fused_ok(const fdtd_t* h) {
   if (h->src_comp >= 0 && !h->per_node) return false;
-  return !h->adjoint && !h->batched && h->nprobes == 0 && fused_shape_ok(h) &&
+  return h->adjoints == 0 && *h->batches == 0 && h->nprobes == 0 && fused_shape_ok(h) &&
          (double)h->nx * h->ny * h->nz * (h->per_node ? 60.0 : 24.0) <=
              (h->per_node ? kFusedMaxBytesPerNode : kFusedMaxBytes);
 }
@@ -2003,8 +2007,10 @@ int step_graph(fdtd_t* h, int64_t nsteps) {
   if (int rc = ensure_branches(h)) return rc;
   const bool src = h->src_comp >= 0;  // (a step without a source or probes reads no counter)
   std::vector<const void*> ptrs(h->f, h->f + 6);
-  if (ptrs != h->g_bound) graph_release(h);
-  const int64_t runs = fused_ok(h) ? nsteps / kStepRun : 0;
+  const bool fused = fused_ok(h);
+  if (ptrs != h->g_bound || fused != h->g_fused) graph_release(h);
+  h->g_fused = fused;
+  const int64_t runs = fused ? nsteps / kStepRun : 0;
   const int64_t singles = nsteps - runs * kStepRun;
   if (runs > 0 && !h->g_run_exec)
     if (int rc = capture_steps(h, kStepRun, &h->g_run_exec, &h->g_run_kernels)) return rc;
@@ -2073,7 +2079,8 @@ int fork_pairs(fdtd_t* h, F&& launch) {
 // their FP64 series have always shown; FLOD2 probes need the output
 // processing of the whole state every step.
 bool plane_ok(const fdtd_t* h) {
-  if (h->nz != 1 || h->order != 2 || h->per_node || h->mu_var || h->batched || h->adjoint || h->timing) return false;
+  if (h->nz != 1 || h->order != 2 || h->per_node || h->mu_var || h->timing) return false;
+  if (h->adjoints > 0 || *h->batches > 0) return false;
   if (h->desc.tune[0] != 0 || (h->desc.tune[1] & (1 | 4 | 8 | 16 | 128 | 1024)) != 0) return false;
   const int most = h->prec == FDTD_F64 ? 128 : 256;
   if (h->nx > most || h->ny > most) return false;
@@ -3166,6 +3173,7 @@ struct BatchGroup {
 
 struct fdtd_batch_s {
   std::vector<fdtd_t*> h;
+  std::vector<std::shared_ptr<std::atomic<int>>> counts;  // the handles' batch counts
   int prec = 0, scheme = 0;
   cudaStream_t stream = nullptr;       // the handles' stream
   cudaStream_t run = nullptr;          // capture/replay stream (never the legacy default)
@@ -4274,10 +4282,6 @@ int fdtd_batch_create(fdtd_t* const* handles, int count, void* stream, fdtd_batc
   fdtd_batch_t* b = new (std::nothrow) fdtd_batch_s();
   if (!b) return FDTD_ERR_OOM;
   b->h.assign(handles, handles + count);
-  for (fdtd_t* h : b->h) {
-    if (!h->batched) graph_release(h);
-    h->batched = true;
-  }
   b->prec = handles[0]->prec;
   b->scheme = handles[0]->scheme;
   b->stream = (cudaStream_t)stream;
@@ -4295,12 +4299,17 @@ int fdtd_batch_create(fdtd_t* const* handles, int count, void* stream, fdtd_batc
   if (b->prec == FDTD_F64) {
     b->cfg.lanes[0] = b->cfg.lanes[1] = 16;
   }
+  for (fdtd_t* h : b->h) {
+    b->counts.push_back(h->batches);
+    ++*h->batches;
+  }
   *out = b;
   return FDTD_OK;
 }
 
 int fdtd_batch_destroy(fdtd_batch_t* b) {
   if (!b) return FDTD_OK;
+  for (auto& n : b->counts) --*n;
   if (b->run) cudaStreamSynchronize(b->run);
   cudaStreamSynchronize(b->stream);
   free_groups(b);
@@ -4985,7 +4994,6 @@ int fdtd_adj_create(fdtd_t* h, const int32_t block[6], int64_t nsteps, int32_t c
   fdtd_adj_t* a = new (std::nothrow) fdtd_adj_s();
   if (!a) return FDTD_ERR_OOM;
   a->h = h;
-  h->adjoint = true;
   a->nsteps = nsteps;
   a->every = checkpoint_every;
   a->nseg = (int)((nsteps + checkpoint_every - 1) / checkpoint_every);
@@ -5063,6 +5071,7 @@ int fdtd_adj_create(fdtd_t* h, const int32_t block[6], int64_t nsteps, int32_t c
       return FDTD_ERR_UNSUPPORTED;
     }
   }
+  h->adjoints++;
   *out = a;
   return FDTD_OK;
 }
@@ -5106,6 +5115,7 @@ int fdtd_adj_memory(const fdtd_adj_t* a, int64_t* bytes) {
 int fdtd_adj_destroy(fdtd_adj_t* a) {
   if (!a) return FDTD_OK;
   cudaStreamSynchronize(a->h->stream);
+  a->h->adjoints--;
   adj_free(a);
   delete a;
   return FDTD_OK;
