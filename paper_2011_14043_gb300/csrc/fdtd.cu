@@ -3638,12 +3638,10 @@ int launch_persistent(const fdtd_batch_t::Persistent& q, int* counter, cudaStrea
   return FDTD_OK;
 }
 
-// The fused launches of a batch (FP32 grids that the fused kernel takes):
+// The fused launches of a batch (batch_fused_candidate):
 // the parameters of every grid, and a list of blocks.  Warps per block: the
 // count that leaves the fewest idle over all grids.
 int build_fused(const fdtd_batch_t* b, bool scratch_out, fdtd_batch_t::Fused (&fl)[2][2]) {
-  for (fdtd_t* h : b->h)
-    if (!fused_shape_ok(h)) return FDTD_ERR_UNSUPPORTED;
   for (int slot = 0; slot < 2; ++slot)
     for (int pn = 0; pn < 2; ++pn) {
       int bw = 8;
@@ -3910,7 +3908,7 @@ int time_step_modes(fdtd_batch_t* b, const BatchCfg& cfg, int reps, double out[2
 }
 
 // Time of one fused step (ms, best of `reps` replays writing scratch), or a
-// negative value where a grid does not take the fused kernel.
+// negative value where it could not be timed.
 double time_fused(fdtd_batch_t* b, int reps) {
   fdtd_batch_t::Fused fl[2][2];
   double best = -1.0;
@@ -3948,11 +3946,25 @@ double time_fused(fdtd_batch_t* b, int reps) {
   return best;
 }
 
+// Whether one fused launch per procedure is a candidate: FP32 grids that the
+// fused kernel takes, and shapes that are the tuner's to choose.
+bool batch_fused_candidate(const fdtd_batch_t* b) {
+  if (b->prec != FDTD_F32 || !b->autotune) return false;
+  for (const fdtd_t* h : b->h)
+    if (!fused_shape_ok(h)) return false;
+  return true;
+}
+
+// The choice among the modes with the shapes in use.  With the fused launches
+// among the candidates it has a key of its own: a choice made without them
+// (shapes fixed by the caller, handles with launch-shape overrides, a file
+// written before they existed) says nothing about them, and the other way
+// round.
 std::string batch_mode_key(const fdtd_batch_t* b) {
   const BatchCfg& c = b->cfg;
   return batch_key(b) + "|mode|" + std::to_string(c.lanes[0]) + "," + std::to_string(c.L[0]) + "," +
          std::to_string(c.lanes[1]) + "," + std::to_string(c.L[1]) + "," + std::to_string(c.wpb) + "," +
-         std::to_string(c.xpack);
+         std::to_string(c.xpack) + (batch_fused_candidate(b) ? "|fused" : "");
 }
 
 // The tuner's choice between the two modes (cached like the shapes): the
@@ -3978,7 +3990,7 @@ int batch_tune_mode_t(fdtd_batch_t* b) {
   if (tune_cache_get(key, &v)) {
     b->mode_ms[0] = v[1] * 1e-3;
     b->mode_ms[1] = v[2] * 1e-3;
-    take(v[0], v[3], v[4], v[5]);
+    take(v[0], v[3], v[4], batch_fused_candidate(b) ? v[5] : 0);
     return FDTD_OK;
   }
   BCK(cudaEventRecord(b->ev_in, b->stream));
@@ -4008,7 +4020,7 @@ int batch_tune_mode_t(fdtd_batch_t* b) {
   // when the shapes are the tuner's to choose
   int fused = 0;
   if constexpr (sizeof(T) == 4) {
-    if (b->autotune) {
+    if (batch_fused_candidate(b)) {
       const double f = time_fused(b, 5);
       if (f > 0 && (ms[0] < 0 || f < ms[0])) {
         fused = 1;
@@ -4113,7 +4125,7 @@ int batch_prepare(fdtd_batch_t* b) {
     if (rc) return rc;
   }
   const bool want = b->mode == 1 || (b->mode == -1 && b->tuned_persistent == 1);
-  const bool want_fused = b->mode == -1 && b->autotune && !want && b->tuned_fused == 1;
+  const bool want_fused = b->mode == -1 && !want && b->tuned_fused == 1 && batch_fused_candidate(b);
   std::vector<const void*> ptrs;
   for (fdtd_t* h : b->h)
     for (int c = 0; c < 6; ++c) ptrs.push_back(h->f[c]);
@@ -4121,11 +4133,16 @@ int batch_prepare(fdtd_batch_t* b) {
     return FDTD_OK;
   free_groups(b);
   b->fused = false;
-  if (want_fused && build_fused(b, false, b->fl) == FDTD_OK) {
-    b->fused = true;
-    b->persistent = false;
-    b->bound = ptrs;
-    return FDTD_OK;
+  if (want_fused) {
+    if (build_fused(b, false, b->fl) == FDTD_OK) {
+      b->fused = true;
+      b->persistent = false;
+      b->bound = ptrs;
+      return FDTD_OK;
+    }
+    free_fused(b->fl);  // (out of memory: the launch groups, from now on)
+    cudaGetLastError();
+    b->tuned_fused = 0;
   }
   int rc = b->prec == FDTD_F64 ? build_groups_t<double>(b, b->cfg, b->groups, -1, false)
                                : build_groups_t<float>(b, b->cfg, b->groups, -1, false);
