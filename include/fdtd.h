@@ -289,9 +289,10 @@ int fdtd_energy_noalloc(int nx, int ny, int nz, double dx, double dy, double dz,
  * launch-shape group (line direction, lanes, segment length and count)
  * covering every grid of the batch; the groups of one procedure run
  * concurrently on parallel graph branches, and one step of the whole batch
- * is captured once as a CUDA graph and replayed.  Every grid runs the arithmetic of its own handle's
- * fdtd_step (bit for bit under a fixed launch shape and the handle's tune[0]; else to
- * rounding).  Handles must share scheme, precision and stream, be distinct,
+ * is captured once as a CUDA graph and replayed.  Every grid runs exactly the
+ * arithmetic of its own handle's fdtd_step while the batch lives (per-node
+ * media outside the fused launches: where the tuned segment lengths agree).
+ * Handles must share scheme, precision and stream, be distinct,
  * and have no source or probe (FDTD_ERR_UNSUPPORTED); they stay owned by
  * the caller, stay usable for set/get/energy, and must outlive the batch.
  * stream: the handles' stream.  Errors as for fdtd_step. */
@@ -336,8 +337,9 @@ int fdtd_batch_set_config(fdtd_batch_t* b, const int32_t* cfg);
  * tiles take at most 256 threads (lines of at most 128 cells at L = 8, 256
  * at L = 16), and x lines packed by 8, 16 or 32 lanes: mode 1 otherwise
  * fails with FDTD_ERR_UNSUPPORTED at the next step, and mode -1 keeps the
- * launches.  Both modes run the same arithmetic per line: the
- * fields agree to the last bit.  fdtd_batch_get_mode (valid after a step)
+ * launches.  Modes 0 and 1 run the same arithmetic per line: the
+ * fields agree to the last bit (with the fused launches that mode -1 may keep,
+ * to rounding).  fdtd_batch_get_mode (valid after a step)
  * gives the mode in use (1 persistent) and the tuned time of one step in
  * each mode (ms; 0 when not timed). */
 int fdtd_batch_set_mode(fdtd_batch_t* b, int mode);

@@ -135,6 +135,7 @@ struct fdtd_s {
   // batches that hold this handle (each has a share in the count, and may be
   // destroyed after the handle)
   std::shared_ptr<std::atomic<int>> batches = std::make_shared<std::atomic<int>>(0);
+  bool batch_fused = false;   // the batch steps it by the fused kernel
   bool shape_tuned = false;   // per-node y/z launch shapes chosen by timing
   double eps_r = 1.0, mu_r = 1.0;          // uniform media
   double* eps_node[3] = {nullptr, nullptr, nullptr};  // per-node eps_r at E samples (device)
@@ -1392,9 +1393,10 @@ bool fused_shape_ok(const fdtd_t* h) {
 // off either way, 9e-5 apart).  Such runs keep the kernels they had.
 bool fused_ok(const fdtd_t* h) {
   if (h->src_comp >= 0 && !h->per_node) return false;
-  return h->adjoints == 0 && *h->batches == 0 && h->nprobes == 0 && fused_shape_ok(h) &&
-         (double)h->nx * h->ny * h->nz * (h->per_node ? 60.0 : 24.0) <=
-             (h->per_node ? kFusedMaxBytesPerNode : kFusedMaxBytes);
+  if (h->adjoints > 0 || h->nprobes > 0 || !fused_shape_ok(h)) return false;
+  if (*h->batches > 0) return h->batch_fused;
+  return (double)h->nx * h->ny * h->nz * (h->per_node ? 60.0 : 24.0) <=
+         (h->per_node ? kFusedMaxBytesPerNode : kFusedMaxBytes);
 }
 
 unsigned reciprocal(int d) { return d <= 1 ? 0u : (unsigned)(((1ull << 32) + (unsigned)d - 1) / (unsigned)d); }
@@ -4104,7 +4106,7 @@ int batch_tune_t(fdtd_batch_t* b) {
   return FDTD_OK;
 }
 
-int batch_prepare(fdtd_batch_t* b) {
+int batch_prepare_tables(fdtd_batch_t* b) {
   for (fdtd_t* h : b->h) {
     int rc = scheme_init(h);
     if (rc) return rc;
@@ -4158,6 +4160,13 @@ int batch_prepare(fdtd_batch_t* b) {
   }
   b->bound = ptrs;
   return FDTD_OK;
+}
+
+// ... and the handles' own steps follow the batch's kernels.
+int batch_prepare(fdtd_batch_t* b) {
+  const int rc = batch_prepare_tables(b);
+  for (fdtd_t* h : b->h) h->batch_fused = rc == FDTD_OK && b->fused;
+  return rc;
 }
 
 // ---------------------------------------------------------------------------

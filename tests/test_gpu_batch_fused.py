@@ -90,6 +90,42 @@ def test_choices_with_and_without_the_fused_launches_are_kept_apart(scheme, tmp_
     assert len(lines) == 3 and lines[2].split()[0] == f"{key}|mode|{SHAPES}"
 
 
+def child_own_steps(case):
+    """From one state, `steps` steps by the batch and by each handle itself
+    (in between and again): the grids whose bits differ."""
+    from paper_2011_14043_gb300 import Batch
+    sims = [sim(case, q) for q in range(len(GRIDS))]
+    b = Batch(sims)
+    b.step(1)
+    differ = []
+    for n in (1, 18):
+        before = [{c: s.get_state(c) for c in ("ex", "ey", "ez", "hx", "hy", "hz")} for s in sims]
+        b.step(n)
+        after = [{c: s.get_state(c) for c in before[0]} for s in sims]
+        for q, s in enumerate(sims):
+            for c in before[q]:
+                s.set_state(c, before[q][c])
+            s.step(n)
+            if not all(np.array_equal(s.get_state(c), after[q][c]) for c in before[q]):
+                differ.append(q)
+    out = {"launches": b.launches_per_step(), "differ": differ}
+    b.close()
+    return out
+
+
+@pytest.mark.parametrize("fused", [0, 1])
+@pytest.mark.parametrize("media_kind", ["uniform", "blocks", "both"])
+@pytest.mark.parametrize("scheme", ["fadi", "fss"])
+def test_a_batch_runs_the_arithmetic_of_its_handles(scheme, media_kind, fused, tmp_path):
+    """Bit for bit (per-node media outside the fused launches: only where the
+    tuned segment lengths agree, so those grids are left out)."""
+    case = {"what": "own_steps", "scheme": scheme, "media": media_kind}
+    got, _ = run_child(case, tmp_path, entry(batch_key(case, SCHEMES[scheme]), fused, "|fused"))
+    if fused:
+        assert got["launches"] == (3 if scheme == "fss" else 2) * (2 if media_kind == "both" else 1)
+    assert [q for q in got["differ"] if fused or media(case, q) is None] == []
+
+
 if __name__ == "__main__":
     CASE = json.loads(sys.argv[1])
     print(json.dumps(globals()["child_" + CASE["what"]](CASE)))
