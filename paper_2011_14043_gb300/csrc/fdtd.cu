@@ -4241,10 +4241,21 @@ int single_tune_t(fdtd_t* h) {
   const std::string key = "grid|" + device_name() + "|p" + std::to_string(h->prec) + "|s" +
                           std::to_string(h->scheme) + "|" + std::to_string(h->nx) + "x" + std::to_string(h->ny) +
                           "x" + std::to_string(h->nz);
-  // FP32 grids of up to a million cells: the candidates differ by less than
-  // their timings scatter, and eight processes in a row picked different
-  // segment lengths (and so different roundings) for one grid; the length most
-  // of them picked is taken, so that runs repeat
+  TuneVal v;
+  if (tune_cache_get(key, &v) && strided_ok<T>(std::max(h->ny, 2), true, v[0], v[1]) &&
+      strided_ok<T>(std::max(h->nz, 2), true, v[2], v[3])) {
+    h->strided_cfg[0] = {true, v[0], v[1]};
+    h->strided_cfg[1] = {true, v[2], v[3]};
+    return FDTD_OK;
+  }
+  // FP32 grids of up to a million cells that no cache names: a fixed shape.
+  // Over 70 grids of 8e3 to 1e6 cells (cubes; y or z lines of 24 to 256 cells
+  // against sides of 16 to 200) the launches of one axis at (16, 8) and at
+  // (32, 16) took the same time: 13.4 and 13.6 us at 32x112x90, 17.1 and 17.1 at
+  // 92^3, either one ahead by the 2 to 3 us in which the timer moves.  Their
+  // roundings differ, so timing them made runs of one program differ.  The
+  // lines below carry no speed: they keep, grid by grid, the segment length that
+  // timing had picked most often, and with it the results.
   if (sizeof(T) == 4 && (double)h->nx * h->ny * h->nz <= 1e6) {
     const bool y16 = h->ny >= 94, z16 = h->nz >= 84 && (double)h->nx * h->ny * h->nz >= 3e5;
     const StridedCfg cy = {true, y16 ? 32 : 16, y16 ? 16 : 8}, cz = {true, z16 ? 32 : 16, z16 ? 16 : 8};
@@ -4254,13 +4265,6 @@ int single_tune_t(fdtd_t* h) {
       h->strided_cfg[1] = cz;
       return FDTD_OK;
     }
-  }
-  TuneVal v;
-  if (tune_cache_get(key, &v) && strided_ok<T>(std::max(h->ny, 2), true, v[0], v[1]) &&
-      strided_ok<T>(std::max(h->nz, 2), true, v[2], v[3])) {
-    h->strided_cfg[0] = {true, v[0], v[1]};
-    h->strided_cfg[1] = {true, v[2], v[3]};
-    return FDTD_OK;
   }
   static const int c32[][2] = {{32, 8}, {32, 16}, {16, 8}, {16, 16}, {16, 32}};
   static const int c64[][2] = {{16, 8}, {16, 16}, {8, 16}, {8, 32}, {16, 32}};
@@ -4829,25 +4833,23 @@ int adj_tune_t(fdtd_adj_t* a) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
   const std::string key = "adjoint|" + device_name() + "|p" + std::to_string(h->prec) + "|" +
                           std::to_string(h->nx) + "x" + std::to_string(h->ny) + "x" + std::to_string(h->nz);
-  // as in single_tune_t: the shapes that timing picks most often
-  if (sizeof(T) == 4 && (double)h->nx * h->ny * h->nz <= 1e6) {
-    const AdjCfg cy = {true, 32, 8}, cz = {true, 32, 8};
-    auto fits = [](int N, const AdjCfg& c) {
-      cudaFuncAttributes fa;
-      const int P = segments(std::max(N, 2), c.L, c.lanes);
-      return P <= 32 && cudaFuncGetAttributes(&fa, adj_strided_fn<T>(c.lanes, c.L)) == cudaSuccess &&
-             P * c.lanes <= fa.maxThreadsPerBlock;
-    };
-    if (fits(h->ny, cy) && fits(h->nz, cz)) {
-      a->cfg[0] = cy;
-      a->cfg[1] = cz;
-      return FDTD_OK;
-    }
-  }
+  auto fits = [](int N, int lanes, int L) {
+    cudaFuncAttributes fa;
+    const void* fn = adj_strided_fn<T>(lanes, L);
+    const int P = fn ? segments(std::max(N, 2), L, lanes) : 33;
+    return P <= 32 && cudaFuncGetAttributes(&fa, fn) == cudaSuccess && P * lanes <= fa.maxThreadsPerBlock;
+  };
   TuneVal v;
-  if (tune_cache_get(key, &v) && adj_strided_fn<T>(v[0], v[1]) && adj_strided_fn<T>(v[2], v[3])) {
+  if (tune_cache_get(key, &v) && fits(h->ny, v[0], v[1]) && fits(h->nz, v[2], v[3])) {
     a->cfg[0] = {true, v[0], v[1]};
     a->cfg[1] = {true, v[2], v[3]};
+    return FDTD_OK;
+  }
+  // as in single_tune_t; here L = 8 is the faster one: the y launches of 32^3 cells at
+  // (16, 8), (32, 8), (16, 16), (32, 16), (16, 32) take 15.7, 16.1, 22.1, 22.4 and
+  // 33.7 us, those of 96^3 29.2, 27.2, 28.9, 29.0 and 39.4
+  if (sizeof(T) == 4 && (double)h->nx * h->ny * h->nz <= 1e6 && fits(h->ny, 32, 8) && fits(h->nz, 32, 8)) {
+    a->cfg[0] = a->cfg[1] = {true, 32, 8};
     return FDTD_OK;
   }
   const size_t bytes = (size_t)h->count * h->esize;
