@@ -99,7 +99,8 @@ typedef enum { FDTD_EX = 0, FDTD_EY = 1, FDTD_EZ = 2, FDTD_HX = 3, FDTD_HY = 4, 
  * bit 11 is accepted and has no effect (it chose between two x-line kernels
  * with the same results).  With tune[0] = 0 and bits 0, 2 and 7 clear, FP32
  * grids of moderate size run each procedure as one launch, and small 2-D
- * grids every step of a call as one launch (bits 3, 4 and 10 clear too);
+ * grids every step of a call as one launch (bits 3, 4 and 10 clear too, on
+ * devices that can hold its cluster of 16 thread blocks);
  * these agree with the other kernels to rounding. */
 typedef struct {
   int32_t nx, ny, nz;        /* cells per axis: 2 <= nx <= 1024, 2 <= ny, 1 <= nz; lines
@@ -392,6 +393,12 @@ int fdtd_debug_fail_alloc(int64_t n);
  * the next one) sets its handle's device flag as a wait that gave up would
  * (the kernel itself runs to its end); n < 0 disarms it.  Process-wide. */
 int fdtd_debug_fail_wait(int64_t n);
+
+/* Test hook: the n-th question from now on (0 = the next one) whether the
+ * device can hold a cluster of thread blocks is answered with no, as on a
+ * device or partition that is too small for it; n < 0 disarms it.
+ * Process-wide. */
+int fdtd_debug_fail_cluster(int64_t n);
 
 /* Self-test of the bounded device waits (failure detection without a GPU
  * fault).  Every spin-wait in the kernels (the TMA kernels' mbarrier waits)

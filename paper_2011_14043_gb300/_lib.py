@@ -36,6 +36,7 @@ EXPORTS = (
     "fdtd_batch_launches", "fdtd_batch_get_config", "fdtd_batch_set_config", "fdtd_batch_set_mode",
     "fdtd_batch_get_mode", "fdtd_adj_create", "fdtd_adj_forward", "fdtd_adj_backward", "fdtd_adj_memory",
     "fdtd_adj_destroy", "fdtd_selftest_bounded_wait", "fdtd_debug_fail_alloc", "fdtd_debug_fail_wait",
+    "fdtd_debug_fail_cluster",
     "fdtd_probe_fp64_fma",
 )
 
@@ -122,6 +123,7 @@ def lib() -> ctypes.CDLL:
         "fdtd_selftest_bounded_wait": (i32, [i64, i32, vp]),
         "fdtd_debug_fail_alloc": (i32, [i64]),
         "fdtd_debug_fail_wait": (i32, [i64]),
+        "fdtd_debug_fail_cluster": (i32, [i64]),
         "fdtd_probe_fp64_fma": (i32, [i64, dp, vp]),
         "fdtd_energy_noalloc": (i32, [i32, i32, i32, ctypes.c_double, ctypes.c_double, ctypes.c_double,
                                       ctypes.c_double, ctypes.c_double, i32, ctypes.POINTER(vp),

@@ -137,6 +137,7 @@ struct fdtd_s {
   std::shared_ptr<std::atomic<int>> batches = std::make_shared<std::atomic<int>>(0);
   bool batch_fused = false;   // the batch steps it by the fused kernel
   bool shape_tuned = false;   // per-node y/z launch shapes chosen by timing
+  int plane_resident = -1;    // whether the plane kernel's cluster fits the device (-1: not asked)
   double eps_r = 1.0, mu_r = 1.0;          // uniform media
   double* eps_node[3] = {nullptr, nullptr, nullptr};  // per-node eps_r at E samples (device)
   // lossy media: electric conductivity sigma [S/m]; the loss -sigma/eps E is
@@ -238,6 +239,10 @@ cudaError_t dev_malloc(void** p, size_t n) {
 // The same for the kernels with bounded waits (fdtd_debug_fail_wait): the n-th
 // next launch sets the handle's flag as a wait that gave up would.
 std::atomic<long long> g_fail_wait_in{-1};
+
+// ... and for the question whether a cluster fits the device
+// (fdtd_debug_fail_cluster): the n-th next one is answered with no.
+std::atomic<long long> g_fail_cluster_in{-1};
 
 int cuda_fail(fdtd_t* h, cudaError_t e) {
   if (e == cudaSuccess) return FDTD_OK;
@@ -2098,11 +2103,69 @@ const void* plane_fn(int L) {
   return nullptr;
 }
 
+// Rows and columns per block, and the launch (one cluster).
 template <typename T>
-int plane_steps(fdtd_t* h, int64_t nsteps) {
+const void* plane_launch(const fdtd_t* h, fdtd::PlaneParams<T>& p, int* L_out, cudaLaunchConfig_t* cfg,
+                         cudaLaunchAttribute* at) {
   const int N = std::max(h->nx, h->ny);
   const int L = N <= 64 ? 2 : (N <= 128 ? 4 : 8);
+  *L_out = L;
+  // multiples of L (a lane's nodes go to one block); padded by one 16-byte
+  // vector, which keeps the pushes aligned
+  auto share = [L](int n) { return ((n + fdtd::kPlaneBlocks - 1) / fdtd::kPlaneBlocks + L - 1) / L * L; };
+  const int vec = std::min(L, (int)(16 / sizeof(T)));
+  p.R = share(h->ny);
+  p.RP = p.R + vec;
+  p.C = share(h->nx);
+  p.CP = p.C + vec;
+  p.ld = (h->nx + 1 + 3) / 4 * 4;
+  p.ldc = (h->ny + 1 + 3) / 4 * 4;
+  *cfg = {};
+  cfg->gridDim = dim3(fdtd::kPlaneBlocks);
+  cfg->blockDim = dim3((unsigned)std::min(16, std::max({4, p.R, p.C})) * 32);
+  cfg->dynamicSmemBytes =
+      ((size_t)(h->nx + 1) * p.RP + (size_t)(h->ny + 1) * p.CP + (size_t)p.R * p.ld + (size_t)p.C * p.ldc) * sizeof(T);
+  cfg->stream = h->stream;
+  *at = {};
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = fdtd::kPlaneBlocks;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg->attrs = at;
+  cfg->numAttrs = 1;
+  return plane_fn<T>(L);
+}
+
+// Whether the device can hold that cluster: 16 blocks are above the portable
+// size, and need as many free SMs within one GPC.  Asked once per handle; where it
+// cannot, the steps go by graph replays.
+template <typename T>
+bool plane_fits(const fdtd_t* h) {
+  if (hook_due(g_fail_cluster_in)) return false;
   fdtd::PlaneParams<T> p = {};
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  int L, n = 0;
+  const void* fn = plane_launch<T>(h, p, &L, &cfg, &at);
+  // (one limit for every grid: handles of other sizes may launch from other threads)
+  const bool ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) == cudaSuccess &&
+                  cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                  cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0;
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
+bool plane_resident(fdtd_t* h) {
+  if (h->plane_resident < 0) h->plane_resident = (h->prec == FDTD_F64 ? plane_fits<double>(h) : plane_fits<float>(h)) ? 1 : 0;
+  return h->plane_resident > 0;
+}
+
+template <typename T>
+int plane_steps(fdtd_t* h, int64_t nsteps) {
+  fdtd::PlaneParams<T> p = {};
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  int L;
+  const void* fn = plane_launch<T>(h, p, &L, &cfg, &at);
   for (int op = 0; op < 2; ++op)
     for (int q = 0; q < 3; ++q) {
       const PairGeom& g = h->geom[op][q];
@@ -2116,16 +2179,6 @@ int plane_steps(fdtd_t* h, int64_t nsteps) {
   p.nx = h->nx;
   p.ny = h->ny;
   p.pitch = h->pitch;
-  // rows and columns per block: multiples of L (a lane's nodes go to one block);
-  // padded by one 16-byte vector, which keeps the pushes aligned
-  auto share = [L](int n) { return ((n + fdtd::kPlaneBlocks - 1) / fdtd::kPlaneBlocks + L - 1) / L * L; };
-  const int vec = std::min(L, (int)(16 / sizeof(T)));
-  p.R = share(h->ny);
-  p.RP = p.R + vec;
-  p.C = share(h->nx);
-  p.CP = p.C + vec;
-  p.ld = (h->nx + 1 + 3) / 4 * 4;
-  p.ldc = (h->ny + 1 + 3) / 4 * 4;
   static const int seq_fss[3] = {0, 1, 0};
   p.nproc = h->scheme == FDTD_FSS ? 3 : 2;
   for (int k = 0; k < 3; ++k) p.seq[k] = seq_fss[k];
@@ -2161,23 +2214,6 @@ int plane_steps(fdtd_t* h, int64_t nsteps) {
   }
   p.out = h->d_probe;
   p.cap = h->probe_cap;
-  const void* fn = plane_fn<T>(L);
-  const size_t smem =
-      ((size_t)(h->nx + 1) * p.RP + (size_t)(h->ny + 1) * p.CP + (size_t)p.R * p.ld + (size_t)p.C * p.ldc) * sizeof(T);
-  // (one limit for every grid: handles of other sizes may launch from other threads)
-  CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
-  CK(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(fdtd::kPlaneBlocks);
-  cfg.blockDim = dim3((unsigned)std::min(16, std::max({4, p.R, p.C})) * 32);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = h->stream;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = fdtd::kPlaneBlocks;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
   while (nsteps > 0) {  // launches of a few milliseconds
     p.n0 = h->steps;
     p.nsteps = std::min<int64_t>(nsteps, 2048);
@@ -2602,6 +2638,11 @@ int fdtd_debug_fail_alloc(int64_t n) {
 
 int fdtd_debug_fail_wait(int64_t n) {
   g_fail_wait_in.store(n < 0 ? -1 : (long long)n);
+  return FDTD_OK;
+}
+
+int fdtd_debug_fail_cluster(int64_t n) {
+  g_fail_cluster_in.store(n < 0 ? -1 : (long long)n);
   return FDTD_OK;
 }
 
@@ -3061,7 +3102,7 @@ int fdtd_step(fdtd_t* h, int64_t nsteps) {
   if (!fused_ok(h)) h->shape_tuned = true;
   if ((rc = ensure_probe_capacity(h, h->steps + nsteps))) return rc;
   if (h->waits) h->err_due = true;
-  if (plane_ok(h)) {
+  if (plane_ok(h) && plane_resident(h)) {
     if ((rc = h->prec == FDTD_F64 ? plane_steps<double>(h, nsteps) : plane_steps<float>(h, nsteps))) return rc;
   } else if (graph_usable(h)) {
     if ((rc = step_graph(h, nsteps))) return rc;
