@@ -1126,6 +1126,7 @@ int resolve_events(fdtd_t* h) {
   CK(cudaStreamSynchronize(h->stream));
   for (auto& r : h->ev_rec) {
     float ms = 0;
+    CK(cudaEventSynchronize(h->ev_pool[r.second.second]));  // (pairs on parallel branches)
     CK(cudaEventElapsedTime(&ms, h->ev_pool[r.second.first], h->ev_pool[r.second.second]));
     h->timed_ms[r.first] += ms;
     h->timed_launches[r.first] += 1;
@@ -4824,17 +4825,16 @@ int adj_reverse_step(fdtd_adj_t* a, double jbar) {
   return rc;
 }
 
-// Capture one step on the handle's stream (the branch-capable stream: adj_on
-// points it there), which moves the device counters itself.
+// One step on the handle's stream (the branch-capable stream:
+// adj_on_replay_stream points it there), captured the first time; it moves the
+// device counters itself.  With per-launch timing on, the step's launches go
+// one by one, each line solve of the forward steps with its event pair.
 template <typename F>
 int adj_capture(fdtd_adj_t* a, cudaGraphExec_t* exec, long long* kernels, F&& step) {
   fdtd_t* h = a->h;
   const long long before = h->launches;
-  const bool timing = h->timing;
-  h->timing = false;  // a captured launch has no time of its own
   CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
   int rc = step();
-  h->timing = timing;
   cudaGraph_t graph = nullptr;
   const cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
   *kernels = h->launches - before;
@@ -4847,6 +4847,17 @@ int adj_capture(fdtd_adj_t* a, cudaGraphExec_t* exec, long long* kernels, F&& st
   const cudaError_t ie = cudaGraphInstantiate(exec, graph, 0);
   cudaGraphDestroy(graph);
   CK(ie);
+  return FDTD_OK;
+}
+
+template <typename F>
+int adj_step(fdtd_adj_t* a, cudaGraphExec_t* exec, long long* kernels, F&& step) {
+  fdtd_t* h = a->h;
+  if (h->timing) return step();
+  if (!*exec)
+    if (int rc = adj_capture(a, exec, kernels, step)) return rc;
+  CK(cudaGraphLaunch(*exec, h->stream));
+  h->launches += *kernels;
   return FDTD_OK;
 }
 
@@ -4955,9 +4966,6 @@ int adj_forward_t(fdtd_adj_t* a) {
   if ((rc = adj_tune_t<T>(a))) return rc;
   CK(cudaMemsetAsync(a->d_acc, 0, sizeof(double), h->stream));
   rc = adj_on_replay_stream(h, [&]() -> int {
-    if (!a->g_fwd)
-      if (int e = adj_capture(a, &a->g_fwd, &a->k_fwd, [&]() { return adj_forward_step<T>(a, h->f, true); }))
-        return e;
     fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, 0, 0);
     for (long long n = 0; n < a->nsteps; ++n) {
       if (n % a->every == 0) {
@@ -4965,8 +4973,7 @@ int adj_forward_t(fdtd_adj_t* a) {
         for (int c = 0; c < 6; ++c) dst[c] = arr_at(a->ckpt, (n / a->every) * 6 + c, h);
         if (int e = copy_arrays(h, dst, h->f, 0, 6)) return e;
       }
-      CK(cudaGraphLaunch(a->g_fwd, h->stream));
-      h->launches += a->k_fwd;
+      if (int e = adj_step(a, &a->g_fwd, &a->k_fwd, [&]() { return adj_forward_step<T>(a, h->f, true); })) return e;
       h->steps++;
     }
     return FDTD_OK;
@@ -4986,17 +4993,11 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
   for (int c = 0; c < 6; ++c) CK(cudaMemsetAsync(a->lam[c], 0, bytes, h->stream));
   for (int c = 0; c < 3; ++c) CK(cudaMemsetAsync(a->grad[c], 0, sizeof(double) * h->count, h->stream));
   rc = adj_on_replay_stream(h, [&]() -> int {
-    if (!a->g_rec)
-      if (int e = adj_capture(a, &a->g_rec, &a->k_rec, [&]() { return adj_forward_step<T>(a, a->work, false); }))
-        return e;
     if (a->g_rev && a->g_jbar != jbar) {
       CK(cudaStreamSynchronize(h->stream));
       cudaGraphExecDestroy(a->g_rev);
       a->g_rev = nullptr;
     }
-    if (!a->g_rev)
-      if (int e = adj_capture(a, &a->g_rev, &a->k_rev, [&]() { return adj_reverse_step<T>(a, jbar); }))
-        return e;
     a->g_jbar = jbar;
     for (int seg = a->nseg - 1; seg >= 0; --seg) {
       const long long n0 = (long long)seg * a->every;
@@ -5005,9 +5006,11 @@ int adj_backward_t(fdtd_adj_t* a, double jbar) {
       for (int c = 0; c < 6; ++c) src[c] = arr_at(a->ckpt, (long long)seg * 6 + c, h);
       if (int e = copy_arrays(h, a->work, src, 0, 6)) return e;
       fdtd::two_counters_kernel<<<1, 32, 0, h->stream>>>(a->d_ctr, n0, 0);
-      for (long long n = n0; n < n1; ++n) CK(cudaGraphLaunch(a->g_rec, h->stream));
-      for (long long n = n0; n < n1; ++n) CK(cudaGraphLaunch(a->g_rev, h->stream));
-      h->launches += (n1 - n0) * (a->k_rec + a->k_rev) + 1;
+      h->launches++;
+      for (long long n = n0; n < n1; ++n)
+        if (int e = adj_step(a, &a->g_rec, &a->k_rec, [&]() { return adj_forward_step<T>(a, a->work, false); })) return e;
+      for (long long n = n0; n < n1; ++n)
+        if (int e = adj_step(a, &a->g_rev, &a->k_rev, [&]() { return adj_reverse_step<T>(a, jbar); })) return e;
     }
     return FDTD_OK;
   });

@@ -132,3 +132,36 @@ def test_media_set_after_the_context(prec):
             same.close()
         L.fdtd_adj_destroy(h)
         sim.close()
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_launch_timing_in_reverse_mode(prec):
+    """fdtd_set_timing counts the line solves of the forward and the
+    recomputed steps, and changes no result."""
+    run = start(prec, SOURCE)
+    J = run.forward()
+    g = gradient(run)
+    run.close()
+    run = start(prec, SOURCE)
+    run.sim.set_timing(True)
+    assert run.forward() == J
+    st = run.sim.stats()
+    assert st["timed_launches"] == [2 * STEPS] * 3 and min(st["timed_ms"]) > 0
+    assert np.array_equal(gradient(run), g)
+    assert run.sim.stats()["timed_launches"] == [4 * STEPS] * 3
+    run.sim.set_timing(False)       # (and captured steps after timed ones)
+    assert np.array_equal(gradient(run), g)
+    assert run.sim.stats()["timed_launches"] == [4 * STEPS] * 3
+    run.close()
+
+
+def test_launch_timing_of_long_runs():
+    """More timed launches than are kept unresolved (4096), on parallel branches."""
+    from paper_2011_14043_gb300.adjoint import AdjointRun, ProbeEnergyProblem
+    n, steps = (9, 8, 7), 700
+    run = AdjointRun(ProbeEnergyProblem(*n, 1e-3, steps=steps, probe_block=(2, 4, 2, 4, 2, 4), cfl=4.0,
+                                        precision="f32", checkpoint_every=50), np.ones(n[::-1]))
+    run.sim.set_timing(True)
+    run.forward()
+    assert run.sim.stats()["timed_launches"] == [2 * steps] * 3
+    run.close()
