@@ -2471,11 +2471,25 @@ int stage_pack(fdtd_t* h, int sx, int sy, int sz, const void* src_padded) {
   return FDTD_OK;
 }
 
+// Memory that a kernel on the current device may touch for sure: its own, or
+// managed.  A caller's pointer to anything else (another device's memory, the
+// host's) goes to a copy call, which reaches it or answers with an error.
+bool kernel_reaches(const void* p) {
+  cudaPointerAttributes a;
+  int dev = 0;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+}
+
 // Between a padded component and the caller's compact device array by
-// repack_rows_kernel; 1 when the caller's pointer is not aligned to its
-// elements (the pitched copy takes any address).
+// repack_rows_kernel; 1 when the caller's pointer is not one for a kernel or not
+// aligned to its elements (the pitched copy takes any address).
 int repack(fdtd_t* h, bool pack, int sx, int sy, int sz, const void* src, void* dst) {
   if (((uintptr_t)src | (uintptr_t)dst) % h->esize != 0) return 1;
+  if (!kernel_reaches(pack ? dst : src)) return 1;
   const long long rows = (long long)sy * sz;
   const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>((rows + 7) / 8, 152LL * 16));
   auto go = [&](auto zero) {
