@@ -2385,9 +2385,9 @@ int read_flag(fdtd_t* h, bool always) {
 // The physical field into scratch, and the flag read after it: the output solve
 // of FP32 grids takes kernels with bounded waits, and where one gave up, tiles of
 // scratch hold an earlier field.
-int physical_checked(fdtd_t* h) {
+int physical_checked(fdtd_t* h, bool always) {
   int rc = physical_to_scratch(h);
-  if (!rc) rc = read_flag(h, false);
+  if (!rc) rc = read_flag(h, always);
   if (rc) h->output_valid = false;
   return rc;
 }
@@ -3006,7 +3006,7 @@ int fdtd_set_field(fdtd_t* h, int comp, const void* data, int on_device) {
   int rc;
   if ((h->scheme == FDTD_FADI || h->scheme == FDTD_FLOD2) && !h->pending_init) {
     // back to the physical field, then re-initialise on the next step
-    if ((rc = physical_checked(h))) return rc;
+    if ((rc = physical_checked(h, false))) return rc;
     for (int c = 0; c < 6; ++c) std::swap(h->f[c], h->scratch[c]);
     h->pending_init = true;
   }
@@ -3020,19 +3020,19 @@ int fdtd_set_field(fdtd_t* h, int comp, const void* data, int on_device) {
 int fdtd_get_field(fdtd_t* h, int comp, void* out, int on_device) {
   if (!h || !out || check_comp(comp)) return FDTD_ERR_INVALID_ARG;
   if (h->poisoned) return FDTD_ERR_STATE;
-  // The flag of the steps, then the solve and the copy, then the solve's flag;
-  // the components that follow wait for neither.  20 steps and a read of the six
-  // 256^3 components into device memory, us: 5606; without the first wait, the
-  // solve queued behind the steps, 5702; with the direct-load y/z kernels, which
-  // have no waits to check, 5625; with the solve's flag left to the next call 5587.
-  int rc = read_flag(h, !on_device);
-  if (rc) return rc;
-  const bool is_state = h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS || h->pending_init;
-  if (!is_state) rc = physical_to_scratch(h);
-  if (!rc) rc = copy_component(h, comp, is_state ? h->f[comp] : h->scratch[comp], out, on_device);
-  if (!rc) rc = read_flag(h, false);
-  if (rc) h->output_valid = false;
-  return rc;
+  if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS || h->pending_init) {
+    if (int rc = read_flag(h, !on_device)) return rc;
+    return copy_component(h, comp, h->f[comp], out, on_device);
+  }
+  // Where the flag has to be read, the steps are waited for before the solve and
+  // the flag is read after it; the components that follow wait for neither.
+  // 20 steps and a read of the six 256^3 components into device memory, us: 5597;
+  // without the first wait, the solve queued behind the steps, 5702; with the copy
+  // before the flag 5606; with the direct-load y/z kernels, which have no waits to
+  // check, 5625; with the solve's flag left to the next call 5601.
+  if (!h->output_valid && (!on_device || h->err_due)) CK(cudaStreamSynchronize(h->stream));
+  if (int rc = physical_checked(h, !on_device)) return rc;
+  return copy_component(h, comp, h->scratch[comp], out, on_device);
 }
 
 int fdtd_get_state(fdtd_t* h, int comp, void* out, int on_device) {
@@ -3152,7 +3152,7 @@ int fdtd_energy(fdtd_t* h, double out[2]) {
   if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS) {
     out[0] = out[1];
   } else {
-    if ((rc = physical_checked(h))) return rc;
+    if ((rc = physical_checked(h, false))) return rc;
     if ((rc = energy(h, h->scratch, &out[0]))) return rc;
   }
   if (!std::isfinite(out[0]) || !std::isfinite(out[1])) return FDTD_ERR_UNSTABLE;
