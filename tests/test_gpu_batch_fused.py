@@ -126,6 +126,42 @@ def test_a_batch_runs_the_arithmetic_of_its_handles(scheme, media_kind, fused, t
     assert [q for q in got["differ"] if fused or media(case, q) is None] == []
 
 
+def child_values(case):
+    """Errors of the batch against the FP64 oracle, and the grids whose bits
+    differ from those of the same grid stepped alone."""
+    from gpu_helpers import energy_norm_rel, oracle_problem, random_fields
+    from oracle import schemes as S
+    from paper_2011_14043_gb300 import Batch
+    steps = 18
+    sims = [sim(case, q) for q in range(len(GRIDS))]
+    b = Batch(sims)
+    b.step(1)
+    b.step(steps - 1)
+    out = {"launches": b.launches_per_step(), "errors": [], "differ": []}
+    states = [{c: s.get_state(c) for c in ("ex", "ey", "ez", "hx", "hy", "hz")} for s in sims]
+    for q, s in enumerate(sims):
+        u0 = {c: v.astype(np.float32).astype(np.float64) for c, v in random_fields(*GRIDS[q], 20 + q).items()}
+        P = oracle_problem(*GRIDS[q], 1e-3, 1e-3, 1e-3, s.dt, eps=media(case, q))
+        out["errors"].append(energy_norm_rel(s.get_fields(), S.run_fundamental(P, case["scheme"], u0, steps)[0]))
+        alone = sim(case, q)
+        alone.step(steps)
+        if not all(np.array_equal(alone.get_state(c), states[q][c]) for c in states[q]):
+            out["differ"].append(q)
+        alone.close()
+    b.close()
+    return out
+
+
+@pytest.mark.parametrize("media_kind", ["uniform", "blocks", "both"])
+@pytest.mark.parametrize("scheme", ["fadi", "fss"])
+def test_fused_batch_against_the_oracle_and_grids_stepped_alone(scheme, media_kind, tmp_path):
+    case = {"what": "values", "scheme": scheme, "media": media_kind}
+    got, _ = run_child(case, tmp_path, entry(batch_key(case, SCHEMES[scheme]), 1, "|fused"))
+    assert got["launches"] == (3 if scheme == "fss" else 2) * (2 if media_kind == "both" else 1)
+    assert max(got["errors"]) <= 1e-4     # the library's stated bound for a few steps
+    assert got["differ"] == []
+
+
 if __name__ == "__main__":
     CASE = json.loads(sys.argv[1])
     print(json.dumps(globals()["child_" + CASE["what"]](CASE)))
