@@ -1848,9 +1848,11 @@ __device__ __forceinline__ T group_chain_backward(T b, HiLo<T> pm, int sl) {
 
 // One x line of a per-node medium on LPL lanes (lane sl its nodes
 // [sl L, sl L + L)): the sweeps of phase_forward / phase_backward with the
-// group scans; a carry runs through its segment by the segment's own
-// multipliers (FP32: hi + lo, as in the sweeps), not by products of their hi
-// parts.  On return E, H hold the new values.
+// group scans.  In FP32 a carry runs through its segment by the segment's own
+// multipliers (hi + lo, as in the sweeps), not by products of their hi parts;
+// FP64 has no lo parts, and takes the products, whose chain does not wait for the
+// carry (the x launches of 64 cavities 3.28 ms per FADI step; the other way 3.53).
+// On return E, H hold the new values.
 template <typename T, int L, int LPL>
 __device__ __forceinline__ void row_solve_pn(const PairParams<T>& p, int sl, T (&E)[L], T (&H)[L], const T (&qn)[L],
                                              const T (&ibn)[L], const T (&ibl)[L]) {
@@ -1866,31 +1868,30 @@ __device__ __forceinline__ void row_solve_pn(const PairParams<T>& p, int sl, T (
   const int j0 = sl * L;
   const HiLo<T> pf = phase_forward<T, L, 2>(p, j0, E, H, hm1, qn, ibn, ibl, ib_prev, y);
   const T yin = group_chain_forward<T, LPL>(y[L - 1], pf, sl);
-  T q = yin;
+  T win;
+  if constexpr (use_hilo<T>()) {
+    T q = yin;
 #pragma unroll
-  for (int t = 0; t < L; ++t) {
-    const HiLo<T> b = t == 0 ? ib_prev : HiLo<T>{ibn[t == 0 ? 0 : t - 1], ibl[t == 0 ? 0 : t - 1]};
-    if constexpr (use_hilo<T>()) {
+    for (int t = 0; t < L; ++t) {
+      const HiLo<T> b = t == 0 ? ib_prev : HiLo<T>{ibn[t == 0 ? 0 : t - 1], ibl[t == 0 ? 0 : t - 1]};
       const T v = fma(b.hi, q, b.lo * q);
       q = fma(-p.offh, v, -p.offl * v);
-    } else {
-      q *= -p.offh * b.hi;
+      y[t] += q;
     }
-    y[t] += q;
-  }
-  // the backward sweep of phase_backward (its carry fix done above)
-  const HiLo<T> pb = phase_backward<T, L, 2, false>(p, j0, T(0), ibn, ibl, ib_prev, y);
-  const T win = group_chain_backward<T, LPL>(y[0], pb, sl);
-  q = win;
+    // the backward sweep of phase_backward (its carry fix done above)
+    const HiLo<T> pb = phase_backward<T, L, 2, false>(p, j0, T(0), ibn, ibl, ib_prev, y);
+    win = group_chain_backward<T, LPL>(y[0], pb, sl);
+    q = win;
 #pragma unroll
-  for (int t = L - 1; t >= 0; --t) {
-    if constexpr (use_hilo<T>()) {
+    for (int t = L - 1; t >= 0; --t) {
       const T u = fma(-p.offh, q, -p.offl * q);
       q = fma(ibn[t], u, ibl[t] * u);
-    } else {
-      q *= -p.offh * ibn[t];
+      y[t] += q;
     }
-    y[t] += q;
+  } else {
+    const HiLo<T> pb = phase_backward<T, L, 2>(p, j0, yin, ibn, ibl, ib_prev, y);
+    win = group_chain_backward<T, LPL>(y[0], pb, sl);
+    phase_fix<T, L, 2>(p, j0, win, ibn, ibl, y);
   }
 #pragma unroll
   for (int t = 0; t < L; ++t) {
