@@ -2083,7 +2083,12 @@ int fork_pairs(fdtd_t* h, F&& launch) {
 // ---------------------------------------------------------------------------
 // Homogeneous media, sides that a warp holds as one line: 128 cells in FP64
 // (L <= 4; beyond, 16 SMs' FP64 pipes lose to the whole chip's) and 256 in
-// FP32 (L <= 8).  FP32 handles with probes keep the kernels whose rounding
+// FP32 (L <= 8).  FP32 grids without a source have the fused procedures as the
+// other choice, which are the faster ones beyond 128 x 128 cells: us per FADI
+// step, 100 steps to a call, here and fused, 128^2 3.8 / 6.6, 256x64 6.6 / 7.7,
+// 64x256 6.1 / 6.6, 160^2 8.5 / 7.2, 200^2 10.1 / 7.5, 256^2 12.1 / 7.8 (FSS 18.9 /
+// 11.7); with a source (launches per pair) 160^2 8.6 / 14.5, 256^2 12.1 / 14.5.
+// FP32 handles with probes keep the kernels whose rounding
 // their FP64 series have always shown; FLOD2 probes need the output
 // processing of the whole state every step.
 bool plane_ok(const fdtd_t* h) {
@@ -2092,6 +2097,7 @@ bool plane_ok(const fdtd_t* h) {
   if (h->desc.tune[0] != 0 || (h->desc.tune[1] & (1 | 4 | 8 | 16 | 128 | 1024)) != 0) return false;
   const int most = h->prec == FDTD_F64 ? 128 : 256;
   if (h->nx > most || h->ny > most) return false;
+  if (h->prec == FDTD_F32 && h->src_comp < 0 && h->nx * h->ny > 128 * 128) return false;
   if (h->src_comp >= 0 && (h->src_comp != EZ || !h->d_srcval)) return false;
   return h->nprobes == 0 || (h->prec == FDTD_F64 && h->scheme != FDTD_FLOD2);
 }
