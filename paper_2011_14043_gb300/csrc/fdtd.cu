@@ -1284,6 +1284,19 @@ int ensure_yseq(fdtd_t* h) {
   return FDTD_OK;
 }
 
+// Bytes that a procedure moves, and the lines up to which it is one launch
+// (fused_ok).
+constexpr double kFusedMaxBytes = 256e6, kFusedMaxBytesPerNode = 150e6;
+double procedure_bytes(const fdtd_t* h) { return (double)h->nx * h->ny * h->nz * (h->per_node ? 60.0 : 24.0); }
+
+// The register-store kernel also writes out of place (the tensor maps only
+// describe what it loads): the output solves of grids beyond the fused line.  A
+// read has to wait for their flag before it copies, so smaller grids take the
+// direct-load kernel (the same results) and one wait less: 12 us of a read.
+bool tma_out_of_place(const fdtd_t* h) {
+  return (h->desc.tune[1] & 4) == 0 && procedure_bytes(h) > kFusedMaxBytes;
+}
+
 template <typename T>
 int launch_pair_raw(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
   const bool pn = h->per_node;
@@ -1319,10 +1332,8 @@ int launch_pair_raw(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) 
       case 32: launch_rows_L<T, 32>(h, g, p, pn); break;
       default: return FDTD_ERR_UNSUPPORTED;
     }
-  } else if (sizeof(T) == 4 && tma_eligible(h, g) && (p.e_in == p.e_out || (h->desc.tune[1] & 4) == 0) &&
+  } else if (sizeof(T) == 4 && tma_eligible(h, g) && (p.e_in == p.e_out || tma_out_of_place(h)) &&
              p.e_in == (const T*)h->f[g.ec] && p.h_in == (const T*)h->f[g.hc]) {
-    // (the register-store kernel also writes out of place: the tensor maps
-    // only describe what it loads)
     // 16-line tiles, two blocks per SM, two-stage ring (measured at 256^3:
     // a three-stage ring 9 % slower, three blocks per SM 12 % slower, 32-line
     // tiles with one block per SM equal)
@@ -1372,7 +1383,8 @@ int launch_pair(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
 // 2^32 bytes.  The launch-shape overrides that name another kernel keep it,
 // the reverse pass (while its context lives) the kernels whose records and
 // rounding it replays, a batch's handles (while it lives) the kernels that the
-// batch steps them by, and handles with probes the kernels whose rounding their FP64 series have always shown.
+// batch steps them by, and handles with probes the kernels whose rounding their
+// FP64 series have always shown.
 //
 // The line: a procedure that moves at most 256 MB (24 B per cell), about twice
 // the L2 cache, or 150 MB with per-node media (60 B per cell).  FADI steps,
@@ -1384,9 +1396,8 @@ int launch_pair(fdtd_t* h, const PairGeom& g, const fdtd::PairParams<T>& p) {
 // one-warp-per-line kernel's 40 warps per SM (x).  FP64 fields gain nothing
 // (their pipe binds: 40^3 44.5 against 33.5).  Per-node tiles hold 128
 // registers, 2 blocks per SM; with E and H loaded again after the solve and 3
-// blocks (80 registers, spills) 128^3 took 92 us.
-constexpr double kFusedMaxBytes = 256e6, kFusedMaxBytesPerNode = 150e6;
-
+// blocks (80 registers, spills) 128^3 took 92 us.  (kFusedMaxBytes,
+// kFusedMaxBytesPerNode)
 bool fused_shape_ok(const fdtd_t* h) {
   if (h->order != 2 || h->mu_var || h->desc.tune[0] != 0 || (h->desc.tune[1] & (1 | 4 | 128)) != 0) return false;
   if (h->nx > fdtd::kFusedMaxN || h->ny > fdtd::kFusedMaxN || h->nz > fdtd::kFusedMaxN) return false;
@@ -1401,8 +1412,7 @@ bool fused_ok(const fdtd_t* h) {
   if (h->src_comp >= 0 && !h->per_node) return false;
   if (h->adjoints > 0 || h->nprobes > 0 || !fused_shape_ok(h)) return false;
   if (*h->batches > 0) return h->batch_fused;
-  return (double)h->nx * h->ny * h->nz * (h->per_node ? 60.0 : 24.0) <=
-         (h->per_node ? kFusedMaxBytesPerNode : kFusedMaxBytes);
+  return procedure_bytes(h) <= (h->per_node ? kFusedMaxBytesPerNode : kFusedMaxBytes);
 }
 
 unsigned reciprocal(int d) { return d <= 1 ? 0u : (unsigned)(((1ull << 32) + (unsigned)d - 1) / (unsigned)d); }
@@ -2389,11 +2399,11 @@ int read_flag(fdtd_t* h, bool always) {
 }
 
 // The physical field into scratch, and the flag read after it: the output solve
-// of FP32 grids takes kernels with bounded waits, and where one gave up, tiles of
-// scratch hold an earlier field.
-int physical_checked(fdtd_t* h, bool always) {
+// of large FP32 grids takes kernels with bounded waits, and where one gave up,
+// tiles of scratch hold an earlier field.
+int physical_checked(fdtd_t* h) {
   int rc = physical_to_scratch(h);
-  if (!rc) rc = read_flag(h, always);
+  if (!rc) rc = read_flag(h, false);
   if (rc) h->output_valid = false;
   return rc;
 }
@@ -3012,7 +3022,7 @@ int fdtd_set_field(fdtd_t* h, int comp, const void* data, int on_device) {
   int rc;
   if ((h->scheme == FDTD_FADI || h->scheme == FDTD_FLOD2) && !h->pending_init) {
     // back to the physical field, then re-initialise on the next step
-    if ((rc = physical_checked(h, false))) return rc;
+    if ((rc = physical_checked(h))) return rc;
     for (int c = 0; c < 6; ++c) std::swap(h->f[c], h->scratch[c]);
     h->pending_init = true;
   }
@@ -3026,18 +3036,16 @@ int fdtd_set_field(fdtd_t* h, int comp, const void* data, int on_device) {
 int fdtd_get_field(fdtd_t* h, int comp, void* out, int on_device) {
   if (!h || !out || check_comp(comp)) return FDTD_ERR_INVALID_ARG;
   if (h->poisoned) return FDTD_ERR_STATE;
-  if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS || h->pending_init) {
-    if (int rc = read_flag(h, !on_device)) return rc;
+  // The flag of the steps, then the solve, its own flag where it has one, then the
+  // copy; the components that follow wait for neither.  20 steps and a read of
+  // the six 256^3 components into device memory, us: 5596; without the first wait,
+  // the solve queued behind the steps, 5702; the copy before the second flag 5606;
+  // with the direct-load y/z kernels, which have no waits to check, 5625; with the
+  // solve's flag left to the next call 5601.
+  if (int rc = read_flag(h, !on_device)) return rc;
+  if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS || h->pending_init)
     return copy_component(h, comp, h->f[comp], out, on_device);
-  }
-  // Where the flag has to be read, the steps are waited for before the solve and
-  // the flag is read after it; the components that follow wait for neither.
-  // 20 steps and a read of the six 256^3 components into device memory, us: 5597;
-  // without the first wait, the solve queued behind the steps, 5702; with the copy
-  // before the flag 5606; with the direct-load y/z kernels, which have no waits to
-  // check, 5625; with the solve's flag left to the next call 5601.
-  if (!h->output_valid && (!on_device || h->err_due)) CK(cudaStreamSynchronize(h->stream));
-  if (int rc = physical_checked(h, !on_device)) return rc;
+  if (int rc = physical_checked(h)) return rc;
   return copy_component(h, comp, h->scratch[comp], out, on_device);
 }
 
@@ -3158,7 +3166,7 @@ int fdtd_energy(fdtd_t* h, double out[2]) {
   if (h->scheme == FDTD_FLOD || h->scheme == FDTD_FSS) {
     out[0] = out[1];
   } else {
-    if ((rc = physical_checked(h, false))) return rc;
+    if ((rc = physical_checked(h))) return rc;
     if ((rc = energy(h, h->scratch, &out[0]))) return rc;
   }
   if (!std::isfinite(out[0]) || !std::isfinite(out[1])) return FDTD_ERR_UNSTABLE;
