@@ -1844,6 +1844,22 @@ SourceTerms source_terms(const fdtd_t* h) {
   return s;
 }
 
+// FP64 per-node handles with probes whose y or z lines go one thread per line
+// (kSeqMinLines): the pairs of a procedure one after the other.  On parallel
+// branches, between the launches of the probes, they push one another's lines out
+// of the L2 cache: us per FADI step with a probe, in order against on branches,
+// 200x190x180 1217 / 1508 to 1631, 180x200x220 1583 / 1635 to 1698, 256x256x128
+// 1568 / 1595 to 1682, 256^3 2677 / 2780 to 2824.  (Without probes the branches
+// take 1392 to 1527, 1434 to 1479, 1590 to 1702 and 2666 to 2755 there, in order
+// 1211, 1578, 1563 and 2672: neither for all, so they stay.)
+bool pairs_in_order(const fdtd_t* h) {
+  if (h->nprobes == 0 || !h->per_node || !h->yseq || !seq_wanted(h)) return false;
+  for (int op = 0; op < 2; ++op)
+    for (const PairGeom& g : h->geom[op])
+      if (!g.rows && g.n_lines() >= kSeqMinLines) return true;
+  return false;
+}
+
 // Capture `count` steps as a graph.  Fused procedures: one launch each, the
 // source added inside it, chained by programmatic edges.  Otherwise each
 // procedure forks its three pair launches (disjoint arrays) onto parallel
@@ -1926,6 +1942,7 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
   auto term = [&](double coef, int off) {
     if (src && coef != 0.0) terms.push_back({coef, off});
   };
+  const bool in_order = pairs_in_order(h);
   cudaStream_t home = h->stream;
   const long long before = h->launches;
   bool advanced = false;
@@ -1973,8 +1990,8 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
       if (rc == FDTD_OK && cudaEventRecord(h->g_fork, h->g_run) != cudaSuccess) rc = FDTD_ERR_CUDA;
       const ProcCoef& P = h->proc[seq[k]];
       for (int q = 0; q < 3 && rc == FDTD_OK; ++q) {
-        if (cudaStreamWaitEvent(h->g_br[q], h->g_fork, 0) != cudaSuccess) { rc = FDTD_ERR_CUDA; break; }
-        h->stream = h->g_br[q];
+        if (!in_order && cudaStreamWaitEvent(h->g_br[q], h->g_fork, 0) != cudaSuccess) { rc = FDTD_ERR_CUDA; break; }
+        h->stream = in_order ? h->g_run : h->g_br[q];
         const PairGeom& g = h->geom[P.op][q];
         if (h->prec == FDTD_F64) {
           fdtd::PairParams<double> p = make_params<double>(h, g, P.pc[q], 1.0, 1.0, -1.0, 1.0, h->f, h->f);
@@ -1984,8 +2001,8 @@ int capture_steps(fdtd_t* h, int count, cudaGraphExec_t* exec, long long* kernel
           rc = launch_pair<float>(h, g, p);
         }
         h->stream = home;
-        if (rc == FDTD_OK && (cudaEventRecord(h->g_join[q], h->g_br[q]) != cudaSuccess ||
-                              cudaStreamWaitEvent(h->g_run, h->g_join[q], 0) != cudaSuccess))
+        if (rc == FDTD_OK && !in_order && (cudaEventRecord(h->g_join[q], h->g_br[q]) != cudaSuccess ||
+                                           cudaStreamWaitEvent(h->g_run, h->g_join[q], 0) != cudaSuccess))
           rc = FDTD_ERR_CUDA;
       }
       term(post[k], st + post_off[k]);

@@ -40,3 +40,28 @@ def test_fused_graphs_bit_identical_to_single_launches(scheme, media, dims):
             assert np.array_equal(sims[0].get_state(c), sims[1].get_state(c)), (n, c)
     for s in sims:
         s.close()
+
+
+@pytest.mark.parametrize("dims,lines", [((190, 180, 182), True), ((190, 100, 182), True), ((60, 50, 40), False)])
+def test_fp64_probed_graphs_bit_identical_to_single_launches(dims, lines):
+    """Per-node media with a probe and a source, with pairs of at least 32768 lines
+    along y and z, along y alone, and of fewer (the former captured one
+    after the other, the latter on parallel branches)."""
+    from paper_2011_14043_gb300 import Simulation
+    nx, ny, nz = dims
+    assert (nx * nz >= 32768) == lines
+    eps = np.random.default_rng(6).uniform(1.0, 6.0, dims[::-1])
+    u0 = random_fields(*dims, 4)
+    cur = np.random.default_rng(7).standard_normal(9) * 1e-3
+    got = []
+    for path in (0, 8):
+        s = Simulation(*dims, 1e-3, scheme="fadi", precision="f64", cfl=5.0, tune=(0, path))
+        s.set_material(eps)
+        s.set_fields(u0)
+        s.set_source("ez", nx // 2, ny // 2, nz // 2, cur)
+        pids = [s.add_probe("ez", nx // 2, ny // 2, nz // 2), s.add_probe("hx", 3, 4, 5)]
+        s.step(3)
+        s.step(4)
+        got.append([s.get_state(c) for c in u0] + [s.get_probe(p, 7) for p in pids])
+        s.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*got))
