@@ -539,8 +539,8 @@ __global__ void __launch_bounds__(kFusedThreads, PN ? 2 : 3)
 // The same for many grids: blocks[b] names the grid and the block within it;
 // its parameters are copied to shared memory.  Ten cavities (5.9 M cells,
 // eps_r blocks): 312 -> 280 us per FADI step against 16 launches per step on
-// four branches, homogeneous ones 345 -> 217; 64 cavities (31 M cells) stay
-// with the launches (1.27 ms either way).
+// four branches, homogeneous ones 345 -> 217; 64 cavities (34 M cells) stay
+// with the launches (1.35 ms against 1.73).
 template <typename T, bool PN>
 __global__ void __launch_bounds__(kFusedThreads, PN ? 2 : 3)
     proc_fused_batch_kernel(const FusedParams<T>* __restrict__ grids, const int2* __restrict__ blocks) {
